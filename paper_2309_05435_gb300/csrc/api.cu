@@ -59,6 +59,11 @@ struct DenseSlot {
   void *U2 = nullptr, *V2 = nullptr, *Wp = nullptr, *Wp2 = nullptr;  // tensor-core sweep panels
   void *Sp[4] = {nullptr, nullptr, nullptr, nullptr};  // the panel update's operands split into TF32 hi / lo
   void *Gs[4] = {nullptr, nullptr, nullptr, nullptr};  // Takahashi operands split into TF32 hi / lo (2 matrices)
+  // binary64 form on digit products: digit planes and row exponents of a
+  // product's operands, and the sweep's panels
+  uint16_t *Od[2] = {nullptr, nullptr};
+  int32_t *Oe[2] = {nullptr, nullptr};
+  OzSweep oz;
   void *wbuf = nullptr;                // T_max x n_pad x ld correction samples
   void *tra = nullptr, *trb = nullptr; // ld x n_pad transposes (tensor-core correction products)
   void *ybuf = nullptr, *tmp = nullptr, *bright = nullptr;
@@ -71,6 +76,7 @@ using namespace qsel;
 struct qsel_ctx {
   int n_s = 0, n_t = 0, n = 0, ld = 0, k = 0, n_pad = 0, n_l = 0, bsize = 64;
   bool mixed = false;
+  bool oz = false;                    // binary64 dense products as bf16 digit products (oz.cuh)
   int tc_passes = 0;                  // mixed path: 3 or 1 = tcgen05 TF32 GEMMs, 0 = CUDA-core FP32
   double sigma = 1.0, obs_w = 1.0;
   qsel_theta theta{};
@@ -90,6 +96,7 @@ struct qsel_ctx {
   double *d_mu = nullptr;              // posterior mean, n
   double *d_hyp = nullptr;             // quadratic forms (3), gradient (3), terms (9)
   double *d_K = nullptr, *d_Kp = nullptr, *d_Ku = nullptr, *d_Kv = nullptr;   // dense K, sweep scratch
+  void *d_Koz = nullptr;               // its digit planes
   bool have_data = false;
   // fixed effects (qsel_set_covariates): Z (n_obs x n_beta), the observed
   // nodes in order, and S, m, S^-1, mu_beta, C, Schur traces (3), diag corr (n)
@@ -865,9 +872,12 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
   // 64 kSweepPanel each), Vk (64 kSweepPanel x 64) and P (64 x 64)
   const size_t panel = (size_t)n_pad * 64 * kSweepPanel * esz;
   const bool split_panels = c->mixed && c->tc_passes == 3;
+  const int oz_rows = std::max(n_pad, c->ld);   // the wider operand of the digit products
+  const size_t oz_operand = (size_t)oz_digit_bytes(oz_rows, n_pad) + (size_t)oz_rows * sizeof(int32_t);
   auto slot_bytes = [&](int T) {
-    return (size_t)(T + 5 + (split_panels ? 4 : 0)) * mat + (split_panels ? 10 : 6) * panel +
-           (size_t)2 * kSweepPanel * (kSweepPanel + 1) * 64 * 64 * esz + (size_t)(T + 5) * svec + 4096;
+    const size_t base = (size_t)(T + 5 + (split_panels ? 4 : 0)) * mat + (split_panels ? 10 : 6) * panel +
+                        (size_t)2 * kSweepPanel * (kSweepPanel + 1) * 64 * 64 * esz + (size_t)(T + 5) * svec + 4096;
+    return base + (c->oz ? 2 * oz_operand + (size_t)oz_sweep_bytes(n_pad) : 0);
   };
   size_t free_b = 0, total_b = 0;
   QSEL_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
@@ -883,6 +893,15 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
       tslabs.push_back(TraceSlab{sd.e0 + tl, sd.slot_base + tl, (tl + 1 < sd.T) ? sd.slot_base + sd.T + tl : -1,
                                  (tl > 0) ? sd.slot_base + sd.T + tl - 1 : -1});
     c->T_max = sd.T;
+  }
+  // Digit products for the binary64 form where the tensor cores can be used and
+  // their scratch (about four matrices a slot) neither makes a wave smaller nor
+  // takes a slot of the two-ended form; the sums are exact up to K = 16384.
+  if (!c->mixed && n_pad <= 16384 && oz_available()) {
+    const size_t want = c->twist ? 2 : (size_t)std::min({kMaxBatch, c->slot_cap, np});
+    const size_t plain = std::min(want, budget / slot_bytes(c->T_max));
+    c->oz = true;
+    if (plain == 0 || budget / slot_bytes(c->T_max) < plain) c->oz = false;
   }
   const size_t per_slot = slot_bytes(c->T_max);
   const size_t fit = budget / per_slot;
@@ -914,6 +933,15 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
     TRY(c->alloc_bytes(&sl.U2, panel));
     TRY(c->alloc_bytes(&sl.V2, panel));
     TRY(c->alloc_bytes(&sl.Wp2, panel));
+    if (c->oz) {
+      for (int q = 0; q < 2; ++q) {
+        TRY(c->alloc_bytes(reinterpret_cast<void **>(&sl.Od[q]), (size_t)oz_digit_bytes(oz_rows, n_pad)));
+        TRY(c->alloc(&sl.Oe[q], (size_t)oz_rows));
+      }
+      void *ozs = nullptr;
+      TRY(c->alloc_bytes(&ozs, (size_t)oz_sweep_bytes(n_pad)));
+      sl.oz = oz_sweep_at(ozs, n_pad);
+    }
     if (split_panels) {
       for (auto &sp : sl.Sp) TRY(c->alloc_bytes(&sp, panel));
       for (auto &gs : sl.Gs) TRY(c->alloc_bytes(&gs, mat));
@@ -1492,6 +1520,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
       we.Wp[1] = buf(sl.Wp2);
       we.Vk = buf(sl.Vk);
       for (int q = 0; q < 4; ++q) we.Sp[q] = buf(sl.Sp[q]);
+      we.oz = sl.oz;
       if (t + 1 < sd.T) {
         SpEntry<T, T> &ge = gb.e[gb.count++];
         ge.B = Dinv(p, t);
@@ -1542,10 +1571,9 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
   std::vector<T *> sig_next(p1 - p0, nullptr);
   std::vector<int> flip(p1 - p0, 0);
   for (int p = p0; p < p1; ++p) sig_next[p - p0] = Dinv(p, part(p).T - 1);
-  bool use_tc = false;
-  if constexpr (std::is_same<T, float>::value) use_tc = c->tc_passes > 0;
+  const bool use_tc = std::is_same<T, float>::value ? c->tc_passes > 0 : c->oz;
   if (use_tc) {
-    if constexpr (std::is_same<T, float>::value) {
+    {
       // Tensor-core form: Wt = c_t D_t^-1 Q_s (= W^T), Yt = Wt Sigma_{t+1} (= Y^T),
       // Sigma_t = D_t^-1 + Yt (Wt)^T; both products have K-major operands.
       for (int b = 0; b < maxT; ++b) {
@@ -1601,21 +1629,51 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
             if (tl <= sd.hi) {
               ExtractEntry<T> &xe = xs.e[xs.count++];
               xe.S = sig_cur;
-              xe.diag_out = nullptr;
+              xe.diag_out = c->mixed ? nullptr : c->d_selinv + (size_t)tg * n_s;
               xe.sums = c->d_sums + kMaxTheta * (size_t)(sd.slot_base + tl);
               set_sum_vals(xe, c->dmod.diag, c->dmod.n, tg);
               xe.D0 = nullptr;
               xe.V = nullptr;
-              DiagRowEntry<T> &de = db.e[db.count++];
-              de.D0 = Dinv(p, tl);
-              de.P = buf(sl.Y);
-              de.R = buf(sl.W);
-              de.diag_out = c->d_selinv + (size_t)tg * n_s;
+              // mixed path: the Takahashi diagonal accumulated in double
+              if (c->mixed) {
+                DiagRowEntry<T> &de = db.e[db.count++];
+                de.D0 = Dinv(p, tl);
+                de.P = buf(sl.Y);
+                de.R = buf(sl.W);
+                de.diag_out = c->d_selinv + (size_t)tg * n_s;
+              }
             }
           }
         }
         if (active.empty()) break;
         launch_sp_colgather<T>(s, wb, c->pat, n_s, n_pad);
+        if constexpr (std::is_same<T, double>::value) {
+          // digit planes of W and Sigma_{t+1}, then of Y in Sigma's place
+          OzSplitJob js[2 * kMaxBatch];
+          OzGemmBatch y2{}, s2{};
+          int nj = 0;
+          for (int q = 0; q < yb.count; ++q) {
+            DenseSlot &sl = slot(active[q]);
+            js[nj++] = OzSplitJob{yb.e[q].A, sl.Od[0], sl.Oe[0], n_pad};
+            js[nj++] = OzSplitJob{yb.e[q].B, sl.Od[1], sl.Oe[1], n_pad};
+            y2.e[y2.count++] = OzGemmEntry{sl.Od[0], sl.Od[1], sl.Oe[0], sl.Oe[1], nullptr, yb.e[q].C, 0};
+          }
+          launch_oz_split_rows(s, js, nj, n_pad, n_pad);
+          if (!launch_oz_gemm(s, y2, n_pad, n_pad, n_pad, n_pad, false, -1, c->d_err))
+            return fail(QSEL_ECUDA, "digit-product GEMM: tensor map encoding failed");
+          launch_extract<T>(s, xy, c->pat, c->dmod.n, n_s, n_pad, c->d_diag_scratch);
+          nj = 0;
+          for (int a = 0; a < (int)active.size() && s2.count < sgb.count; ++a) {
+            DenseSlot &sl = slot(active[a]);
+            const GemmEntry<T> &ge = sgb.e[s2.count];
+            if (ge.A != buf(sl.Y)) continue;
+            js[nj++] = OzSplitJob{buf(sl.Y), sl.Od[1], sl.Oe[1], n_pad};
+            s2.e[s2.count++] = OzGemmEntry{sl.Od[1], sl.Od[0], sl.Oe[1], sl.Oe[0], ge.C0, ge.C, 0};
+          }
+          launch_oz_split_rows(s, js, nj, n_pad, n_pad);
+          if (!launch_oz_gemm(s, s2, n_pad, n_pad, n_pad, n_pad, true, -1, c->d_err))
+            return fail(QSEL_ECUDA, "digit-product GEMM: tensor map encoding failed");
+        } else {
         const int64_t mm = (int64_t)n_pad * n_pad;
         if (slot(active[0]).Gs[0] != nullptr) {
           // 3xTF32 on operands split once in HBM: W and Sigma_{t+1}, then
@@ -1658,6 +1716,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
           launch_extract<T>(s, xy, c->pat, c->dmod.n, n_s, n_pad, c->d_diag_scratch);
           if (!launch_tc_gemm(s, sgb, n_pad, n_pad, n_pad, n_pad, n_pad, n_pad, true, c->tc_passes, c->d_err))
             return fail(QSEL_ECUDA, "tensor-core GEMM: tensor map encoding failed");
+        }
         }
         launch_diag64_rows<T>(s, db, n_s, n_pad);
         launch_mirror<T>(s, mb, n_pad);
@@ -1806,6 +1865,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
     // (through the transposed product, with each part's ld x n_pad scratch
     // tra / trb), else the tile GEMM
     void *bt[kMaxBatch], *pt[kMaxBatch];
+    DenseSlot *slot_of[kMaxBatch];
     auto block_product = [&](const GemmBatch<T> &gb) -> Err {
       if constexpr (std::is_same<T, float>::value) {
         if (c->tc_passes > 0) {
@@ -1814,6 +1874,22 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
             return fail(QSEL_ECUDA, "tensor-core GEMM: tensor map encoding failed");
           return ok();
         }
+      } else if (c->oz) {
+        // D_t^-1's digit planes by rows, the block's by columns
+        OzSplitJob ja[kMaxBatch], jb[kMaxBatch];
+        OzGemmBatch og{};
+        for (int q = 0; q < gb.count; ++q) {
+          DenseSlot &sl = *slot_of[q];
+          ja[q] = OzSplitJob{gb.e[q].A, sl.Od[0], sl.Oe[0], n_pad};
+          jb[q] = OzSplitJob{gb.e[q].B, sl.Od[1], sl.Oe[1], ld};
+          og.e[og.count++] = OzGemmEntry{sl.Od[0], sl.Od[1], sl.Oe[0], sl.Oe[1], gb.e[q].C0, gb.e[q].C,
+                                         gb.e[q].alpha < 0.0 ? 1 : 0};
+        }
+        launch_oz_split_rows(s, ja, gb.count, n_pad, n_pad);
+        if (!launch_oz_split_cols(s, jb, gb.count, n_pad, ld, ld) ||
+            !launch_oz_gemm(s, og, n_pad, ld, n_pad, ld, false, -1, c->d_err))
+          return fail(QSEL_ECUDA, "digit-product GEMM could not be launched");
+        return ok();
       }
       launch_gemm<T>(s, gb, n_pad, ld, n_pad, n_pad, ld, ld, false);
       return ok();
@@ -1832,6 +1908,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
         if (t >= sd.T) continue;
         bt[ub.count] = sl.tra;
         pt[ub.count] = sl.trb;
+        slot_of[ub.count] = &sl;
         GemmEntry<T> &g = ub.e[ub.count++];
         g.A = Dinv(p, t);
         g.B = buf(sl.ybuf);
@@ -1873,6 +1950,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
         e.beta = 0.0;
         bt[wb.count] = sl.tra;
         pt[wb.count] = sl.trb;
+        slot_of[wb.count] = &sl;
         GemmEntry<T> &g = wb.e[wb.count++];
         g.A = Dinv(p, t);
         g.B = buf(sl.tmp);
@@ -2620,6 +2698,9 @@ qsel_status qsel_loglik_grad(qsel_ctx *ctx, double grad_out[3], double terms_out
   if (e.code == 0 && !c->d_Kp) e = c->alloc(&c->d_Kp, 64 * 64);
   if (e.code == 0 && !c->d_Ku) e = c->alloc(&c->d_Ku, (size_t)n_pad * 64);
   if (e.code == 0 && !c->d_Kv) e = c->alloc(&c->d_Kv, (size_t)n_pad * 64);
+  // digit planes for K's sweep (the CUDA-core tiles serve when there is no room)
+  if (e.code == 0 && !c->d_Koz && oz_available() && c->alloc_bytes(&c->d_Koz, (size_t)oz_sweep_bytes(n_pad)).code)
+    c->d_Koz = nullptr;
   if (e.code) return finish(c, e);
   // mu^T dQ_j mu: dQ_j mu by the block-tridiagonal SpMM with the derivative's
   // coefficients (no observation term), its per-column dot partials with mu
@@ -2652,6 +2733,7 @@ qsel_status qsel_loglik_grad(qsel_ctx *ctx, double grad_out[3], double terms_out
   kb.e[0].P = c->d_Kp;
   kb.e[0].U = c->d_Ku;
   kb.e[0].V = c->d_Kv;
+  if (c->d_Koz) kb.e[0].oz = oz_sweep_at(c->d_Koz, n_pad);
   spd_inverse<double>(s, kb, n_pad, c->d_err, 0);
   launch_loglik_combine(s, c->d_K, n_pad, c->d_cdiag, c->n_s, c->n_t, c->d_theta, c->d_traces,
                         c->n_beta > 0 ? c->fe_trace() : nullptr, c->d_hyp, c->d_hyp + 3, c->d_hyp + 6);
@@ -2662,6 +2744,7 @@ qsel_status qsel_loglik_grad(qsel_ctx *ctx, double grad_out[3], double terms_out
   if (ce == cudaSuccess) ce = cudaGetLastError();
   if (ce != cudaSuccess) return finish(c, cuda_fail(ce, "hyperparameter gradient", __FILE__, __LINE__));
   err = c->h_counters[0];
+  if (err & 2) return finish(c, fail(QSEL_ETIMEOUT, "a bounded device-side wait of the tensor-core GEMM gave up"));
   if (err & 1) return finish(c, fail(QSEL_ENOTSPD, "K = kappa^2 C + G was not positive definite"));
   for (int j = 0; j < 3; ++j) grad_out[j] = c->h_small[j];
   if (terms_out)

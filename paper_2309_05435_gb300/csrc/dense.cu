@@ -973,15 +973,29 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
     }
   }
   for (int k = 0; k < nt; ++k) {
-    g_launch_count += 3;
+    ++g_launch_count;
     {
       ProfScope ps_(s, PROF_PIVOT, 2.0 * 64.0 * 64.0 * 64.0 * b.count);
       k_sweep_pivot<T><<<b.count, 256, 0, s>>>(b, k, n_pad, err_flag);
+    }
+    if constexpr (std::is_same<T, double>::value) {
+      if (b.e[0].oz.Ud) {
+        // the panel and the rank-64 update as digit products (row and column k
+        // are the panel's)
+        launch_oz_sweep_panel(s, b, k, n_pad, err_flag);
+        OzGemmBatch gb{};
+        gb.count = b.count;
+        for (int e = 0; e < b.count; ++e)
+          gb.e[e] = OzGemmEntry{b.e[e].oz.Ud, b.e[e].oz.Vd, b.e[e].oz.Eu, b.e[e].oz.Ev, b.e[e].A, b.e[e].A, 1};
+        if (nt > 1) launch_oz_gemm(s, gb, n_pad, n_pad, 64, n_pad, true, k, err_flag);
+        continue;
+      }
     }
     {
       ProfScope ps_(s, PROF_PANEL);
       if (nt > 1) k_sweep_panel<T><<<dim3(nt - 1, b.count), 256, 0, s>>>(b, k, n_pad);
     }
+    g_launch_count += 2;
     Profiler::Rec rec{PROF_SWEEP, nullptr, nullptr, 0.0};
     if (g_prof) {
       // rank-64 update of the lower tiles off row/column k: 2 * 64^3 FLOPs each

@@ -199,6 +199,16 @@ void launch_gemm(cudaStream_t s, const GemmBatch<T> &b, int M, int N, int K, int
 // 64 kSweepPanel).
 constexpr int kSweepPanel = 4;
 
+// Binary64 sweep on digit products (null: CUDA-core tiles): digit planes of the
+// pivot's U and V (n_pad x 64 each) and their row exponents.
+struct OzSweep {
+  uint16_t *Ud = nullptr, *Vd = nullptr;
+  int32_t *Eu = nullptr, *Ev = nullptr;
+};
+// Bytes of that scratch, and the scratch at base (16-byte aligned).
+int64_t oz_sweep_bytes(int n_pad);
+OzSweep oz_sweep_at(void *base, int n_pad);
+
 template <typename T>
 struct SweepEntry {
   T *A;          // n_pad x n_pad, row-major, lower tiles used
@@ -212,6 +222,7 @@ struct SweepEntry {
                  // panel rows of the pivot column, per panel parity and pivot)
   T *Sp[4];      // tensor-core path: the panel update's U and V split into TF32 hi / lo
                  // (U_hi, U_lo, V_hi, V_lo; n_pad x 64 kSweepPanel each), or null
+  OzSweep oz;    // double only
 };
 // Streams and events of the tensor-core sweep's look-ahead: the pivot chain
 // (pivots, the panel's and the next panel's rows) runs on hi (high priority);
@@ -281,6 +292,44 @@ struct DiagRowBatch {
 };
 template <typename T>
 void launch_diag64_rows(cudaStream_t s, const DiagRowBatch<T> &b, int n_s, int n_pad);
+
+// ---------------------------------------------------------------- oz_gemm.cu
+// Binary64 products as exact bf16 digit products on the tensor cores (oz.cuh).
+// Bytes of the eight digit planes of a rows x cols operand.
+int64_t oz_digit_bytes(int rows, int cols);
+struct OzSplitJob {
+  const double *src;
+  uint16_t *dig;            // digit planes (16-byte aligned)
+  int32_t *exp;             // exponent of every row (or column)
+  int rows;
+};
+// Digit planes of the rows of rows x cols blocks (leading dimension ld; cols and
+// ld multiples of 4), or of the columns of K x cols blocks (cols a multiple of
+// 32, K of 64): the K-major operands of launch_oz_gemm.  Up to 2 kMaxBatch jobs.
+bool launch_oz_split_rows(cudaStream_t s, const OzSplitJob *jobs, int count, int cols, int ld);
+bool launch_oz_split_cols(cudaStream_t s, const OzSplitJob *jobs, int count, int K, int cols, int ld);
+struct OzGemmEntry {
+  const uint16_t *A, *B;    // digit planes: A of M rows, B of N rows, K entries each
+  const int32_t *Ea, *Eb;
+  const double *C0;         // added, or null; may alias C
+  double *C;
+  int negate;               // C = C0 - A B^T instead of C0 + A B^T
+};
+struct OzGemmBatch {
+  OzGemmEntry e[kMaxBatch];
+  int count;
+};
+// C = C0 +- A B^T (K a multiple of 32 and at most 16384, N a multiple of 32, ldc
+// even).  lower: only the 128 x 64 tiles that touch the lower triangle; skip >= 0:
+// rows and columns of that 64-wide tile index are left as they are.  err gets bit 1 when a
+// bounded wait gives up.  False when nothing could be launched.
+bool oz_available();
+bool launch_oz_gemm(cudaStream_t s, const OzGemmBatch &b, int M, int N, int K, int ldc, bool lower, int skip,
+                    int32_t *err);
+
+// One pivot k of the binary64 sweep on digit products: the column panel and its
+// digit planes (SweepEntry::oz), see oz_gemm.cu.
+void launch_oz_sweep_panel(cudaStream_t s, const SweepBatch<double> &b, int k, int n_pad, int32_t *err);
 
 // ---------------------------------------------------------------- tc_gemm.cu
 // tcgen05 tensor-core GEMM (FP32 data, TF32 MMAs): C = alpha A B^T + beta C0

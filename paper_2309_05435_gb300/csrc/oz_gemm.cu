@@ -1,0 +1,704 @@
+// Binary64 matrix products as exact bf16 digit products on the tensor cores
+// (oz.cuh): C = alpha A B^T + beta C0 with A: M x K, B: N x K given as digit
+// planes, alpha = +-1, beta = 0 or 1.
+//
+// What bounds it: GB300 runs binary64 FMAs at 1.2 TFLOP/s; 36 bf16 digit products
+// at 1.95 PFLOP/s are worth 54 TFLOP/s of binary64 products.  Output tiles of
+// 128 x 64: the eight groups of digit products with equal i + j take 64
+// accumulator columns each, all 512 columns of the SM's tensor memory.  A wider
+// tile would need two passes over the operands, a narrower one is bound by
+// shared memory (a 128 x 32 tile reads 125 bytes per cycle of the 128 there are;
+// this one 104, since one MMA takes up to four digits of B).
+//   warp 0      one thread issues the TMA loads of K = 32 stages (A: 8 digits x
+//               128 rows, B: 8 digits x 64 rows, 96 KB) into a 2-stage ring;
+//   warp 1      owns the 512 TMEM columns; one thread issues 12 MMAs per K = 16;
+//   warps 2-9   after every kChunk of K: tcgen05.ld, FP32 sums to integers, 64-bit
+//               integer accumulation (exact); at the end one rounding to binary64.
+// Every wait is bounded: after the limit the CTA raises bit 1 of *err, stops
+// issuing work, waits (bounded) for its loads and MMAs in flight, frees its
+// tensor memory and returns.
+//
+// Measured: two 1600 x 1600 x 1600 products 13.3 ms on the CUDA cores (k_gemm64)
+// -> 0.53 ms (31 TFLOP/s of binary64 products; 38 at 4096, where a K = 128 block
+// takes 9.2k cycles of MMAs and 8k of reading the sums); one 64-wide update of a
+// 1600-node block 236 -> 44 us.  The products' error against a 113-bit reference
+// is 5e-17 relative in the 2-norm (the final rounding) at K = 64 .. 1024, the FMA
+// chain's 1e-16 .. 1e-15, on random, decaying, equal-sign and widely scaled
+// operands.  It is used at every size: a 64 x 64 x 64 product takes 66 us on one
+// SM's binary64 pipe and 19 us here.
+#include <algorithm>
+#include <cstring>
+#include <mutex>
+
+#include "qsel.h"
+#include "kernels.cuh"
+#include "tc_common.cuh"
+#include "oz.cuh"
+
+namespace qsel {
+namespace oz {
+using namespace tc;
+
+constexpr int KS = 32;                         // K of a stage: 64-byte rows
+constexpr int BN_OZ = 64;
+constexpr int STAGES = 2;
+constexpr int ROWB = KS * 2;
+constexpr int A_TILE = BM * ROWB;              // one digit of A
+constexpr int B_TILE = BN_OZ * ROWB;
+constexpr int A_BYTES = kDigits * A_TILE;      // 64 KiB
+constexpr int B_BYTES = kDigits * B_TILE;      // 32 KiB
+constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 256 + 1024;
+constexpr int EP_WARPS = 8;
+constexpr int THREADS = 64 + 32 * EP_WARPS;
+constexpr int GROUP = 8;
+
+struct Params {
+  CUtensorMap tm[kMaxBatch][2];
+  const int32_t *Ea[kMaxBatch], *Eb[kMaxBatch];
+  const double *C0[kMaxBatch];
+  double *C[kMaxBatch];
+  int negate[kMaxBatch];
+  int M, N, K, ldc, lower, skip;
+  int tiles_m, tiles_n, per_matrix, total;
+  int32_t *err;
+  long long wait_cycles;
+  int skip_loads;
+};
+
+// Tile l of one matrix: full tiles in groups of GROUP tile rows (column by
+// column inside a group), or the tiles that touch the lower triangle row by row.
+__device__ __forceinline__ void tile_of(const Params &p, int l, int &bm, int &bn) {
+  if (!p.lower) {
+    const int per_group = GROUP * p.tiles_n;
+    const int g = l / per_group, g0 = g * GROUP;
+    const int rows = min(GROUP, p.tiles_m - g0);
+    const int w = l - g * per_group;
+    bn = w / rows;
+    bm = g0 + (w - bn * rows);
+    return;
+  }
+  int r = 0;
+  for (;;) {
+    const int cnt = min(p.tiles_n, 2 * r + 2);
+    if (l < cnt) break;
+    l -= cnt;
+    ++r;
+  }
+  bm = r;
+  bn = l;
+}
+
+__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity) {
+  const long long t0 = clock64();
+  uint32_t done = 0;
+  while (!done && clock64() - t0 < kWaitCycles) {
+    asm volatile(
+        "{\n\t.reg .pred r;\n\tmbarrier.try_wait.parity.shared::cta.b64 r, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, r;\n\t}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+  }
+}
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *tm, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+          dst),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
+
+__global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ Params p) {
+  extern __shared__ unsigned char smem_raw[];
+  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t *bars = reinterpret_cast<uint64_t *>(base + STAGES * STAGE_BYTES);
+  // bars: [0, S) full, [S, 2S) empty, [2S] accumulator full, [2S+1] accumulator
+  // read, [2S+2] all MMAs done
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * STAGES + 3);
+  volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nk = p.K / KS;
+  const uint32_t bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
+  const uint32_t accf_bar = bar0 + 8u * (2 * STAGES), accr_bar = accf_bar + 8u, fin_bar = accf_bar + 16u;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    mbar_init(accf_bar, 1);
+    mbar_init(accr_bar, EP_WARPS);
+    mbar_init(fin_bar, 1);
+    *abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      long long g = 0;   // stages issued
+      bool go = !p.skip_loads;
+      for (int L = blockIdx.x; L < p.total && go; L += gridDim.x) {
+        const int z = L / p.per_matrix;
+        int bm, bn;
+        tile_of(p, L - z * p.per_matrix, bm, bn);
+        if (bn == p.skip) continue;
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          const int s = (int)(g % STAGES);
+          const uint32_t u = (uint32_t)(g / STAGES);
+          if (!mbar_wait(empty_bar(s), (u & 1) ^ 1, abort, p.err, p.wait_cycles)) {
+            go = false;
+            break;
+          }
+          uint8_t *st = base + s * STAGE_BYTES;
+          mbar_expect_tx(full_bar(s), STAGE_BYTES);
+          tma_load_3d(smem_u32(st), &p.tm[z][0], kb * KS, bm * BM, 0, full_bar(s));
+          tma_load_3d(smem_u32(st + A_BYTES), &p.tm[z][1], kb * KS, bn * BN_OZ, 0, full_bar(s));
+        }
+      }
+      if (*abort) {
+        // let the loads already issued land before the CTA's shared memory goes away
+        for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
+          drain(full_bar((int)(q % STAGES)), (uint32_t)((q / STAGES) & 1));
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      long long g = 0;
+      uint32_t chunk = 0;
+      bool go = true;
+      for (int L = blockIdx.x; L < p.total && go; L += gridDim.x) {
+        const int z = L / p.per_matrix;
+        int bm, bn;
+        tile_of(p, L - z * p.per_matrix, bm, bn);
+        if (bn == p.skip) continue;
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          const bool first = kb % (kChunk / KS) == 0;
+          if (first) {
+            if (!mbar_wait(accr_bar, (chunk & 1) ^ 1, abort, p.err, p.wait_cycles)) {
+              go = false;
+              break;
+            }
+            tc_fence_after();
+          }
+          const int s = (int)(g % STAGES);
+          const uint32_t u = (uint32_t)(g / STAGES);
+          if (!mbar_wait(full_bar(s), u & 1, abort, p.err, p.wait_cycles)) {
+            go = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t st = smem_u32(base + s * STAGE_BYTES);
+#pragma unroll
+          for (int j = 0; j < KS / 16; ++j)
+            mma_digits<ROWB>(tmem, st + 32 * j, st + A_BYTES + 32 * j, A_TILE, B_TILE, first && j == 0);
+          mma_commit(empty_bar(s));
+          if (kb + 1 == nk || (kb + 1) % (kChunk / KS) == 0) {
+            mma_commit(accf_bar);
+            ++chunk;
+          }
+        }
+      }
+      mma_commit(fin_bar);   // arrives once every MMA issued above has completed
+    }
+  } else {
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows, columns
+    // 32 ((w - 2) / 4) .. + 31 of the tile
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + 32u * half;
+    const int n_chunks = (p.K + kChunk - 1) / kChunk;
+    uint32_t chunk = 0;
+    bool go = true;
+    for (int L = blockIdx.x; L < p.total && go; L += gridDim.x) {
+      const int z = L / p.per_matrix;
+      int bm, bn;
+      tile_of(p, L - z * p.per_matrix, bm, bn);
+      if (bn == p.skip) continue;
+      int64_t hi[32], lo[32];
+#pragma unroll
+      for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
+      for (int ch = 0; ch < n_chunks; ++ch, ++chunk) {
+        int okay = 0;
+        if (lane == 0) okay = mbar_wait(accf_bar, chunk & 1, abort, p.err, p.wait_cycles) && !*abort;
+        okay = __shfl_sync(0xffffffffu, okay, 0);
+        if (!okay) {
+          go = false;
+          break;
+        }
+        tc_fence_after();
+#pragma unroll
+        for (int cb = 0; cb < 4; ++cb) accumulate8(t0 + 8u * cb, hi + 8 * cb, lo + 8 * cb);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(accr_bar);
+      }
+      const int row = bm * BM + 32 * q + lane, col = bn * BN_OZ + 32 * half;
+      if (!go || row >= p.M || col >= p.N || (row >> 6) == p.skip) continue;
+      const bool neg = p.negate[z] != 0;
+      const int32_t Ea = p.Ea[z][row];
+      const int32_t *Eb = p.Eb[z] + col;
+      const double *c0 = p.C0[z] ? p.C0[z] + (int64_t)row * p.ldc + col : nullptr;
+      double *c = p.C[z] + (int64_t)row * p.ldc + col;
+#pragma unroll
+      for (int cc = 0; cc < 32; cc += 2) {
+        double2 o = make_double2(value(hi[cc], lo[cc], Ea, Eb[cc], neg), value(hi[cc + 1], lo[cc + 1], Ea, Eb[cc + 1], neg));
+        if (c0) {
+          const double2 v = *reinterpret_cast<const double2 *>(c0 + cc);
+          o.x += v.x;
+          o.y += v.y;
+        }
+        *reinterpret_cast<double2 *>(c + cc) = o;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    if (lane == 0) drain(fin_bar, 0u);   // no MMA may still write the accumulator
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+}
+
+std::once_flag g_once;
+bool g_ok = false;
+
+// ---------------------------------------------------------------------------
+// Digit planes of the rows of a matrix: block per row, the row read twice (the
+// second pass from L1 / L2), four neighbouring entries per thread and step.
+// Plane i, row r, entry k at dig[i * plane + r * ldk + k].
+// ---------------------------------------------------------------------------
+struct SplitParams {
+  OzSplitJob j[2 * kMaxBatch];
+  int cols, ld;
+};
+
+__device__ __forceinline__ void store_digits4(uint16_t *dst, int64_t plane, const uint2 (&y)[4]) {
+#define QSEL_OZ_STORE(I) \
+  *reinterpret_cast<uint2 *>(dst + (I) * plane) = make_uint2(digit_pair<I>(y[0], y[1]), digit_pair<I>(y[2], y[3]))
+  QSEL_OZ_STORE(0);
+  QSEL_OZ_STORE(1);
+  QSEL_OZ_STORE(2);
+  QSEL_OZ_STORE(3);
+  QSEL_OZ_STORE(4);
+  QSEL_OZ_STORE(5);
+  QSEL_OZ_STORE(6);
+  QSEL_OZ_STORE(7);
+#undef QSEL_OZ_STORE
+}
+
+constexpr int SPLIT_THREADS = 128;
+
+__global__ void __launch_bounds__(SPLIT_THREADS) k_oz_split_rows(const __grid_constant__ SplitParams p) {
+  __shared__ int red[SPLIT_THREADS / 32];
+  const OzSplitJob &job = p.j[blockIdx.y];
+  const int row = blockIdx.x;
+  if (row >= job.rows) return;
+  const double *src = job.src + (int64_t)row * p.ld;
+  int f = 0;
+  for (int k = 4 * threadIdx.x; k < p.cols; k += 4 * SPLIT_THREADS) {
+    const double2 a = *reinterpret_cast<const double2 *>(src + k), b = *reinterpret_cast<const double2 *>(src + k + 2);
+    f = max(f, max(max(exp_field(a.x), exp_field(a.y)), max(exp_field(b.x), exp_field(b.y))));
+  }
+  for (int o = 16; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < SPLIT_THREADS / 32; ++w) f = max(f, red[w]);
+  const int32_t E = row_exponent(f);
+  if (threadIdx.x == 0) job.exp[row] = E;
+  const int32_t Ef = E == kNonFinite ? 1025 : E;
+  const int64_t plane = (int64_t)job.rows * p.cols;
+  uint16_t *dst = job.dig + (int64_t)row * p.cols;
+  for (int k = 4 * threadIdx.x; k < p.cols; k += 4 * SPLIT_THREADS) {
+    const double2 a = *reinterpret_cast<const double2 *>(src + k), b = *reinterpret_cast<const double2 *>(src + k + 2);
+    const uint2 y[4] = {digit_bytes(fixed62(a.x, Ef)), digit_bytes(fixed62(a.y, Ef)), digit_bytes(fixed62(b.x, Ef)),
+                        digit_bytes(fixed62(b.y, Ef))};
+    store_digits4(dst + k, plane, y);
+  }
+}
+
+// Digit planes of the columns of a K x N block (row-major, leading dimension
+// ld): plane i, column c, entry k at dig[i * N * K + c * K + k].  Two passes: the
+// largest exponent field of every column (atomicMax into exp, which starts at
+// zero), then 64 (k) x 32 (columns) tiles transposed through shared memory.
+__global__ void __launch_bounds__(256) k_oz_colmax(const __grid_constant__ SplitParams p, int K) {
+  __shared__ int red[8][32];
+  const OzSplitJob &job = p.j[blockIdx.z];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int c = blockIdx.x * 32 + lane;
+  int f = 0;
+  const int k1 = min(K, (int)(blockIdx.y + 1) * 256);
+  for (int k = blockIdx.y * 256 + w; k < k1; k += 8) f = max(f, exp_field(job.src[(int64_t)k * p.ld + c]));
+  red[w][lane] = f;
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) f = max(f, red[q][lane]);
+    atomicMax(&job.exp[c], f);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_oz_split_cols(const __grid_constant__ SplitParams p, int K) {
+  __shared__ double S[64][33];
+  const OzSplitJob &job = p.j[blockIdx.z];
+  const int c0 = blockIdx.x * 32, k0 = blockIdx.y * 64;
+  for (int e = threadIdx.x; e < 64 * 32; e += 256)
+    S[e >> 5][e & 31] = job.src[(int64_t)(k0 + (e >> 5)) * p.ld + c0 + (e & 31)];
+  __syncthreads();
+  const int64_t plane = (int64_t)p.cols * K;
+  for (int e = threadIdx.x; e < 16 * 32; e += 256) {
+    const int k = 4 * (e & 15), c = e >> 4;
+    const int32_t E = row_exponent(job.exp[c0 + c]);
+    const int32_t Ef = E == kNonFinite ? 1025 : E;
+    const uint2 y[4] = {digit_bytes(fixed62(S[k][c], Ef)), digit_bytes(fixed62(S[k + 1][c], Ef)),
+                        digit_bytes(fixed62(S[k + 2][c], Ef)), digit_bytes(fixed62(S[k + 3][c], Ef))};
+    store_digits4(job.dig + (int64_t)(c0 + c) * K + k0 + k, plane, y);
+  }
+}
+// exponent fields to row exponents, once every column has been split
+__global__ void k_oz_exponents(const __grid_constant__ SplitParams p) {
+  const OzSplitJob &job = p.j[blockIdx.y];
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < p.cols) job.exp[c] = row_exponent(job.exp[c]);
+}
+
+// ---------------------------------------------------------------------------
+// One pivot of the binary64 symmetric sweep, off the update: for every row tile
+// i != k,  V_i = A_ik,  U_i = A_ik P,  A_ik <- U_i,  and A_kk <- -P; U and V leave
+// as digit planes (n_pad rows x 64) for the update A -= U V^T.  CTA per 128 rows.
+// The product takes 64 x 64 x 64 binary64 FMAs per row tile, 63 us on one SM's
+// binary64 pipe; as digit products it is 48 MMAs.  The digits of A_ik are formed
+// in registers and stored to shared memory in the MMA's swizzled layout and to
+// global memory as V's at once.
+// ---------------------------------------------------------------------------
+struct PanelParams {
+  double *A[kMaxBatch];
+  const double *P[kMaxBatch];
+  uint16_t *U[kMaxBatch], *V[kMaxBatch];
+  int32_t *Eu[kMaxBatch], *Ev[kMaxBatch];
+  int k, n_pad;
+  int32_t *err;
+  long long wait_cycles;
+};
+
+constexpr int P_ROWB = 128;                                // K = 64: 128-byte rows
+constexpr int PA_TILE = BM * P_ROWB, PB_TILE = 64 * P_ROWB;
+constexpr int PANEL_SMEM = kDigits * (PA_TILE + PB_TILE) + 1024;
+constexpr int PANEL_THREADS = 256;
+
+// Eight digits of eight neighbouring values: 16 bytes per digit plane to shared
+// (stride s_plane) and / or global memory (stride g_plane).
+template <bool SMEM>
+__device__ __forceinline__ void store_digits8(uint8_t *sdst, uint32_t s_plane, uint16_t *gdst, int64_t g_plane,
+                                              const double *x, int32_t E) {
+  uint2 y[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) y[c] = digit_bytes(fixed62(x[c], E));
+#define QSEL_OZ_STORE(I)                                                                                  \
+  {                                                                                                       \
+    const uint4 w = make_uint4(digit_pair<I>(y[0], y[1]), digit_pair<I>(y[2], y[3]),                      \
+                               digit_pair<I>(y[4], y[5]), digit_pair<I>(y[6], y[7]));                     \
+    if (SMEM) *reinterpret_cast<uint4 *>(sdst + (I) * s_plane) = w;                                       \
+    if (gdst) *reinterpret_cast<uint4 *>(gdst + (I) * g_plane) = w;                                       \
+  }
+  QSEL_OZ_STORE(0)
+  QSEL_OZ_STORE(1)
+  QSEL_OZ_STORE(2)
+  QSEL_OZ_STORE(3)
+  QSEL_OZ_STORE(4)
+  QSEL_OZ_STORE(5)
+  QSEL_OZ_STORE(6)
+  QSEL_OZ_STORE(7)
+#undef QSEL_OZ_STORE
+}
+__device__ __forceinline__ int32_t finite_exponent(int32_t E) { return E == kNonFinite ? 1025 : E; }
+
+__global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __grid_constant__ PanelParams p) {
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ int red[2][BM];
+  __shared__ int32_t ep[64];
+  __shared__ __align__(8) uint64_t bar_mem;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_mem;
+  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t *sa = base, *sb = base + kDigits * PA_TILE;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int z = blockIdx.y, k = p.k, ld = p.n_pad;
+  const uint32_t bar = smem_u32(&bar_mem);
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    abort_mem = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  const int q = warp & 3, half = warp >> 2;
+  const int r = 32 * q + lane, gi = blockIdx.x * BM + r;
+  const int i = gi >> 6;                        // this row's tile
+  const bool valid = gi < p.n_pad, on_pivot = i == k;
+  double *A = p.A[z];
+  const double *P = p.P[z];
+  double x[32];
+  if (!valid || on_pivot) {
+#pragma unroll
+    for (int c = 0; c < 32; ++c) x[c] = 0.0;
+  } else if (i > k) {
+    const double *src = A + (int64_t)gi * ld + 64 * k + 32 * half;
+#pragma unroll
+    for (int c = 0; c < 32; c += 2) {
+      const double2 v = *reinterpret_cast<const double2 *>(src + c);
+      x[c] = v.x;
+      x[c + 1] = v.y;
+    }
+  } else {
+    // A_ik = A_ki^T (lower tiles are stored): consecutive lanes, consecutive columns
+    const double *src = A + (int64_t)(64 * k + 32 * half) * ld + gi;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) x[c] = src[(int64_t)c * ld];
+  }
+  int f = 0;
+#pragma unroll
+  for (int c = 0; c < 32; ++c) f = max(f, exp_field(x[c]));
+  red[half][r] = f;
+  // P's digits: four threads per row, 16 entries each
+  {
+    const int pr = threadIdx.x >> 2, pq = threadIdx.x & 3;
+    double y[16];
+#pragma unroll
+    for (int c = 0; c < 16; c += 2) {
+      const double2 v = *reinterpret_cast<const double2 *>(P + pr * 64 + 16 * pq + c);
+      y[c] = v.x;
+      y[c + 1] = v.y;
+    }
+    int g = 0;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) g = max(g, exp_field(y[c]));
+    g = max(g, __shfl_xor_sync(0xffffffffu, g, 1));
+    g = max(g, __shfl_xor_sync(0xffffffffu, g, 2));
+    const int32_t E = row_exponent(g);
+    if (pq == 0) ep[pr] = E;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      store_digits8<true>(sb + pr * P_ROWB + (((2 * pq + c) ^ (pr & 7)) << 4), PB_TILE, nullptr, 0, y + 8 * c,
+                          finite_exponent(E));
+  }
+  __syncthreads();
+  const int64_t plane = (int64_t)p.n_pad * 64;
+  const int32_t Ea = row_exponent(max(red[0][r], red[1][r]));
+  {
+    uint16_t *gd = valid ? p.V[z] + (int64_t)gi * 64 + 32 * half : nullptr;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      store_digits8<true>(sa + r * P_ROWB + (((4 * half + c) ^ (r & 7)) << 4), PA_TILE, gd ? gd + 8 * c : nullptr, plane,
+                          x + 8 * c, finite_exponent(Ea));
+    if (valid && half == 0) p.Ev[z][gi] = Ea;
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      mma_digits<P_ROWB>(tmem, smem_u32(sa) + 32 * j, smem_u32(sb) + 32 * j, PA_TILE, PB_TILE, j == 0);
+    mma_commit(bar);
+  }
+  __syncwarp();
+  const bool okay = mbar_wait(bar, 0u, &abort_mem, p.err, p.wait_cycles);
+  tc_fence_after();
+  __syncwarp();
+  if (__all_sync(0xffffffffu, okay)) {
+    const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + 32u * half;
+    f = 0;
+#pragma unroll
+    for (int cb = 0; cb < 4; ++cb) {
+      int64_t hi[8], lo[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
+      accumulate8(t0 + 8u * cb, hi, lo);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        x[8 * cb + c] = value(hi[c], lo[c], Ea, ep[32 * half + 8 * cb + c], false);
+        f = max(f, exp_field(x[8 * cb + c]));
+      }
+    }
+  }
+  __syncthreads();   // red was read by every thread before the MMAs
+  red[half][r] = f;
+  __syncthreads();
+  const int32_t Eu = row_exponent(max(red[0][r], red[1][r]));
+  if (valid) {
+    uint16_t *gd = p.U[z] + (int64_t)gi * 64 + 32 * half;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) store_digits8<false>(nullptr, 0, gd + 8 * c, plane, x + 8 * c, finite_exponent(Eu));
+    if (half == 0) p.Eu[z][gi] = Eu;
+    if (on_pivot) {
+      double *dst = A + (int64_t)gi * ld + 64 * k + 32 * half;
+      const double *src = P + (gi & 63) * 64 + 32 * half;
+#pragma unroll
+      for (int c = 0; c < 32; ++c) dst[c] = -src[c];
+    } else if (i > k) {
+      double *dst = A + (int64_t)gi * ld + 64 * k + 32 * half;
+#pragma unroll
+      for (int c = 0; c < 32; c += 2) *reinterpret_cast<double2 *>(dst + c) = make_double2(x[c], x[c + 1]);
+    } else {
+      double *dst = A + (int64_t)(64 * k + 32 * half) * ld + gi;
+#pragma unroll
+      for (int c = 0; c < 32; ++c) dst[(int64_t)c * ld] = x[c];
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    if (lane == 0) drain(bar, 0u);   // no MMA may still write the accumulator
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+}
+
+}  // namespace oz
+
+int64_t oz_sweep_bytes(int n_pad) { return 2 * oz_digit_bytes(n_pad, 64) + 2 * (int64_t)n_pad * 4; }
+OzSweep oz_sweep_at(void *base, int n_pad) {
+  OzSweep o;
+  uint8_t *b = static_cast<uint8_t *>(base);
+  o.Ud = reinterpret_cast<uint16_t *>(b);
+  o.Vd = reinterpret_cast<uint16_t *>(b + oz_digit_bytes(n_pad, 64));
+  o.Eu = reinterpret_cast<int32_t *>(b + 2 * oz_digit_bytes(n_pad, 64));
+  o.Ev = o.Eu + n_pad;
+  return o;
+}
+
+int64_t oz_digit_bytes(int rows, int cols) { return (int64_t)oz::kDigits * rows * cols * 2; }
+
+bool launch_oz_split_rows(cudaStream_t s, const OzSplitJob *jobs, int count, int cols, int ld) {
+  if (count <= 0) return true;
+  oz::SplitParams p;
+  memset(&p, 0, sizeof(p));
+  int rows = 0;
+  for (int q = 0; q < count; ++q) {
+    p.j[q] = jobs[q];
+    rows = std::max(rows, jobs[q].rows);
+  }
+  p.cols = cols;
+  p.ld = ld;
+  ++g_launch_count;
+  oz::k_oz_split_rows<<<dim3(rows, count), oz::SPLIT_THREADS, 0, s>>>(p);
+  return true;
+}
+
+bool launch_oz_split_cols(cudaStream_t s, const OzSplitJob *jobs, int count, int K, int cols, int ld) {
+  if (count <= 0) return true;
+  oz::SplitParams p;
+  memset(&p, 0, sizeof(p));
+  for (int q = 0; q < count; ++q) {
+    p.j[q] = jobs[q];
+    if (cudaMemsetAsync(jobs[q].exp, 0, (size_t)cols * sizeof(int32_t), s) != cudaSuccess) return false;
+  }
+  p.cols = cols;
+  p.ld = ld;
+  g_launch_count += 3;
+  oz::k_oz_colmax<<<dim3(cols / 32, (K + 255) / 256, count), 256, 0, s>>>(p, K);
+  oz::k_oz_split_cols<<<dim3(cols / 32, K / 64, count), 256, 0, s>>>(p, K);
+  oz::k_oz_exponents<<<dim3((cols + 255) / 256, count), 256, 0, s>>>(p);
+  return true;
+}
+
+bool oz_available() {
+  if (!tc_gemm_available()) return false;
+  std::call_once(oz::g_once, [] {
+    oz::g_ok = cudaFuncSetAttribute(oz::k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM_BYTES) ==
+                   cudaSuccess &&
+               cudaFuncSetAttribute(oz::k_oz_sweep_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    oz::PANEL_SMEM) == cudaSuccess;
+    if (!oz::g_ok) cudaGetLastError();
+  });
+  return oz::g_ok;
+}
+
+bool launch_oz_gemm(cudaStream_t s, const OzGemmBatch &b, int M, int N, int K, int ldc, bool lower, int skip,
+                    int32_t *err) {
+  if (b.count <= 0) return true;
+  if (K % oz::KS != 0 || !oz_available()) return false;
+  oz::Params p;
+  memset(&p, 0, sizeof(p));
+  for (int q = 0; q < b.count; ++q) {
+    const OzGemmEntry &e = b.e[q];
+    if (!tc::encode_digits(&p.tm[q][0], e.A, M, K, oz::kDigits, oz::KS, tc::BM) ||
+        !tc::encode_digits(&p.tm[q][1], e.B, N, K, oz::kDigits, oz::KS, oz::BN_OZ))
+      return false;
+    p.Ea[q] = e.Ea;
+    p.Eb[q] = e.Eb;
+    p.C0[q] = e.C0;
+    p.C[q] = e.C;
+    p.negate[q] = e.negate;
+  }
+  p.M = M;
+  p.N = N;
+  p.K = K;
+  p.ldc = ldc;
+  p.lower = lower ? 1 : 0;
+  p.skip = skip;
+  p.tiles_m = (M + tc::BM - 1) / tc::BM;
+  p.tiles_n = (N + oz::BN_OZ - 1) / oz::BN_OZ;
+  if (lower) {
+    int t = 0;
+    for (int r = 0; r < p.tiles_m; ++r) t += std::min(p.tiles_n, 2 * r + 2);
+    p.per_matrix = t;
+  } else {
+    p.per_matrix = p.tiles_m * p.tiles_n;
+  }
+  p.total = p.per_matrix * b.count;
+  p.err = err;
+  p.wait_cycles = tc::wait_limit();
+  p.skip_loads = tc::skip_loads();
+  int sms = 152, dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  ++g_launch_count;
+  ProfScope ps_(s, PROF_GEMM, 2.0 * tc::BM * oz::BN_OZ * (double)K * p.total);
+  oz::k_oz_gemm<<<std::min(p.total, sms), oz::THREADS, oz::SMEM_BYTES, s>>>(p);
+  return true;
+}
+
+void launch_oz_sweep_panel(cudaStream_t s, const SweepBatch<double> &b, int k, int n_pad, int32_t *err) {
+  oz::PanelParams p;
+  memset(&p, 0, sizeof(p));
+  for (int q = 0; q < b.count; ++q) {
+    p.A[q] = b.e[q].A;
+    p.P[q] = b.e[q].P;
+    p.U[q] = b.e[q].oz.Ud;
+    p.V[q] = b.e[q].oz.Vd;
+    p.Eu[q] = b.e[q].oz.Eu;
+    p.Ev[q] = b.e[q].oz.Ev;
+  }
+  p.k = k;
+  p.n_pad = n_pad;
+  p.err = err;
+  p.wait_cycles = tc::wait_limit();
+  ++g_launch_count;
+  ProfScope ps_(s, PROF_PANEL);
+  oz::k_oz_sweep_panel<<<dim3((n_pad + tc::BM - 1) / tc::BM, b.count), oz::PANEL_THREADS, oz::PANEL_SMEM, s>>>(p);
+}
+
+}  // namespace qsel

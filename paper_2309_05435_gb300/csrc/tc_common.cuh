@@ -160,6 +160,10 @@ bool encode_4d(CUtensorMap *tm, const float *ptr, const uint64_t dims[4], const 
 // innermost, a multiple of 4): the layout of a staged store tile.
 bool encode_4d_plain(CUtensorMap *tm, const float *ptr, const uint64_t dims[4], const uint64_t strides[3],
                      const uint32_t box[4]);
+// Tensor map of `planes` stacked bf16 matrices (rows x cols each, contiguous):
+// boxes of box_cols columns (64-byte rows) x box_rows rows x all planes, 64B
+// swizzle, zero fill outside.
+bool encode_digits(CUtensorMap *tm, const uint16_t *ptr, int rows, int cols, int planes, int box_cols, int box_rows);
 // Limits of the bounded waits and the test hook's skip flag (tc_gemm.cu).
 long long wait_limit();
 int skip_loads();
