@@ -482,14 +482,13 @@ qsel_status qsel_debug_tc_wait(int32_t skip_loads, int64_t wait_cycles);
  * rank-64 bw update of the rest runs on the same stream as the pivot chain,
  * after it, instead of beside the next panel's pivots.  update_ctas > 0: the
  * persistent update kernel runs on at most that many CTAs (one per SM), so
- * that SMs stay free for the pivot chain; 0 = one per SM.  update_stages 2
- * or 3: the update's shared-memory ring (3 stages leave no room for the
- * pivot chain's CTAs on the update's SMs); 4: the update on 128 x 256
- * tiles by the persistent split-operand GEMM; 0 = the default.  By default
- * each pivot CTA asks for unused shared memory so that it cannot share an SM
- * with an update CTA, and the update (unless update_ctas says otherwise)
- * leaves one SM per pivot CTA free; shared_pivot non-zero lets the pivot CTAs
- * run beside update CTAs instead.  Process-wide;
+ * that SMs stay free for the pivot chain; 0 = the default.  update_stages 2
+ * or 3: the update's shared-memory ring (with 2 the pivot chain's CTAs fit
+ * beside it); 4: the update on 128 x 256 tiles by the persistent
+ * split-operand GEMM; 0 = the default, 3.  By default, with at most two
+ * matrices a launch, each of the four pivot CTAs of a matrix has an SM that the
+ * update leaves free; shared_pivot non-zero (and more matrices) gives the
+ * update every SM.  Process-wide;
  * qsel_debug_sweep_schedule(0, 0, 0, 0) restores the default.  Errors:
  * QSEL_EINVAL for update_ctas < 0 or update_stages not 0, 2, 3 or 4.
  */

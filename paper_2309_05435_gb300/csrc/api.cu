@@ -56,7 +56,7 @@ struct DenseSlot {
   std::vector<void *> Dinv;            // T_max pivot-block inverses
   void *SigA = nullptr, *SigB = nullptr, *Y = nullptr, *W = nullptr, *V = nullptr;
   void *P = nullptr, *U = nullptr, *Vs = nullptr, *Vk = nullptr;  // sweep scratch
-  void *U2 = nullptr, *V2 = nullptr, *Wp = nullptr, *Wp2 = nullptr;  // tensor-core sweep panels
+  void *U2 = nullptr, *Wp = nullptr, *Wp2 = nullptr;  // tensor-core sweep panels
   void *Sp[4] = {nullptr, nullptr, nullptr, nullptr};  // the panel update's operands split into TF32 hi / lo
   void *Gs[4] = {nullptr, nullptr, nullptr, nullptr};  // Takahashi operands split into TF32 hi / lo (2 matrices)
   // binary64 form on digit products: digit planes and row exponents of a
@@ -868,15 +868,15 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
   // device memory (at most kMaxBatch)
   const size_t mat = (size_t)n_pad * n_pad * esz;
   const size_t svec = (size_t)n_pad * c->ld * esz;
-  // sweep scratch: two sets of U, V and the column panel W (n_pad x
-  // 64 kSweepPanel each), Vk (64 kSweepPanel x 64) and P (64 x 64)
+  // sweep scratch: two sets of U and the column panel W, one of V (n_pad x
+  // 64 kSweepPanel each), per pivot of a panel Vk (64 kSweepPanel x 64) and P
   const size_t panel = (size_t)n_pad * 64 * kSweepPanel * esz;
   const bool split_panels = c->mixed && c->tc_passes == 3;
   const int oz_rows = std::max(n_pad, c->ld);   // the wider operand of the digit products
   const size_t oz_operand = (size_t)oz_digit_bytes(oz_rows, n_pad) + (size_t)oz_rows * sizeof(int32_t);
   auto slot_bytes = [&](int T) {
-    const size_t base = (size_t)(T + 5 + (split_panels ? 4 : 0)) * mat + (split_panels ? 10 : 6) * panel +
-                        (size_t)2 * kSweepPanel * (kSweepPanel + 1) * 64 * 64 * esz + (size_t)(T + 5) * svec + 4096;
+    const size_t base = (size_t)(T + 5 + (split_panels ? 4 : 0)) * mat + (split_panels ? 9 : 5) * panel +
+                        (size_t)kSweepPanel * (kSweepPanel + 1) * 64 * 64 * esz + (size_t)(T + 5) * svec + 4096;
     return base + (c->oz ? 2 * oz_operand + (size_t)oz_sweep_bytes(n_pad) : 0);
   };
   size_t free_b = 0, total_b = 0;
@@ -926,27 +926,26 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
     TRY(c->alloc_bytes(&sl.Y, mat));
     TRY(c->alloc_bytes(&sl.W, mat));
     TRY(c->alloc_bytes(&sl.V, mat));
-    TRY(c->alloc_bytes(&sl.P, (size_t)2 * kSweepPanel * 64 * 64 * esz));   // per panel parity and pivot
+    TRY(c->alloc_bytes(&sl.P, (size_t)kSweepPanel * 64 * 64 * esz));   // per pivot of a panel
     TRY(c->alloc_bytes(&sl.U, panel));
     TRY(c->alloc_bytes(&sl.Vs, panel));
     TRY(c->alloc_bytes(&sl.Wp, panel));
     TRY(c->alloc_bytes(&sl.U2, panel));
-    TRY(c->alloc_bytes(&sl.V2, panel));
     TRY(c->alloc_bytes(&sl.Wp2, panel));
     if (c->oz) {
-      for (int q = 0; q < 2; ++q) {
-        TRY(c->alloc_bytes(reinterpret_cast<void **>(&sl.Od[q]), (size_t)oz_digit_bytes(oz_rows, n_pad)));
-        TRY(c->alloc(&sl.Oe[q], (size_t)oz_rows));
+      uint8_t *oz = nullptr;
+      TRY(c->alloc(&oz, 2 * oz_operand + (size_t)oz_sweep_bytes(n_pad)));
+      for (int q = 0; q < 2; ++q, oz += oz_operand) {
+        sl.Od[q] = reinterpret_cast<uint16_t *>(oz);
+        sl.Oe[q] = reinterpret_cast<int32_t *>(oz + oz_digit_bytes(oz_rows, n_pad));
       }
-      void *ozs = nullptr;
-      TRY(c->alloc_bytes(&ozs, (size_t)oz_sweep_bytes(n_pad)));
-      sl.oz = oz_sweep_at(ozs, n_pad);
+      sl.oz = oz_sweep_at(oz, n_pad);
     }
     if (split_panels) {
       for (auto &sp : sl.Sp) TRY(c->alloc_bytes(&sp, panel));
       for (auto &gs : sl.Gs) TRY(c->alloc_bytes(&gs, mat));
     }
-    TRY(c->alloc_bytes(&sl.Vk, (size_t)2 * kSweepPanel * kSweepPanel * 64 * 64 * esz));
+    TRY(c->alloc_bytes(&sl.Vk, (size_t)kSweepPanel * kSweepPanel * 64 * 64 * esz));
     TRY(c->alloc_bytes(&sl.wbuf, (size_t)c->T_max * svec));
     TRY(c->alloc_bytes(&sl.ybuf, svec));
     TRY(c->alloc_bytes(&sl.tmp, svec));
@@ -1513,10 +1512,8 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
       we.U = buf(sl.U);
       we.V = buf(sl.Vs);
       we.Up[0] = buf(sl.U);
-      we.Vp[0] = buf(sl.Vs);
       we.Wp[0] = buf(sl.Wp);
       we.Up[1] = buf(sl.U2);
-      we.Vp[1] = buf(sl.V2);
       we.Wp[1] = buf(sl.Wp2);
       we.Vk = buf(sl.Vk);
       for (int q = 0; q < 4; ++q) we.Sp[q] = buf(sl.Sp[q]);

@@ -232,16 +232,7 @@ template void launch_gemm<float>(cudaStream_t, const GemmBatch<float> &, int, in
 template <int NT, typename T>
 __device__ __forceinline__ void invert_pivot_tile(const T *Tk, int ld, T *P, int32_t *err_flag, bool fp64) {
   // one buffer for either arithmetic (dfloat and double are both 8 bytes)
-  constexpr int kSweepBytes = (64 * 65 + 65 + 64) * 8;
-  constexpr int kBytes = (int)sizeof(Inverse64Smem) > kSweepBytes ? (int)sizeof(Inverse64Smem) : kSweepBytes;
-  __shared__ __align__(16) unsigned char pv_smem[kBytes];
-  if constexpr (std::is_same<T, float>::value && NT >= 512) {
-    if (!fp64) {
-      // the diagonal tile is kept symmetric; the lower half is what is read
-      sym_inverse64_df_2x2<NT>(Tk, ld, P, *reinterpret_cast<Inverse64Smem *>(pv_smem), err_flag);
-      return;
-    }
-  }
+  __shared__ __align__(16) unsigned char pv_smem[(64 * 65 + 65 + 64) * 8];
   if constexpr (std::is_same<T, float>::value) {
     if (!fp64) {
       dfloat *Sf = reinterpret_cast<dfloat *>(pv_smem);
@@ -325,228 +316,32 @@ __global__ void __launch_bounds__(256) k_sweep_panel(SweepBatch<T> bt, int k, in
 // receives one rank-64 bw update C -= [U^(k)] [V^(k)]^T on the tensor cores
 // (which also overwrites rows and columns K; the scatter restores them).
 // ---------------------------------------------------------------------------
+// Row tiles of the gather: [lo0, lo0 + n0) and then [lo1, ..).
 template <typename T>
-__global__ void __launch_bounds__(256) k_bsweep_gather(SweepBatch<T> bt, int k0, int bw, int ld, int buf) {
+__global__ void __launch_bounds__(256) k_bsweep_gather(SweepBatch<T> bt, int k0, int bw, int ld, int buf, int lo0,
+                                                       int n0, int lo1) {
   __shared__ T S[64 * 65];
   const SweepEntry<T> e = bt.e[blockIdx.y];
   constexpr int ldw = 64 * kSweepPanel;
-  const int i = blockIdx.x;
-  for (int q = 0; q < bw; ++q) {
-    const int j = k0 + q;
-    // A_ij lives in tile (max(i, j), min(i, j)) of the lower triangle
-    const T *src = e.A + (int64_t)max(i, j) * 64 * ld + min(i, j) * 64;
+  // CTA per (row tile, panel column)
+  const int t = (int)blockIdx.x / bw, q = (int)blockIdx.x % bw;
+  const int i = t < n0 ? lo0 + t : lo1 + t - n0;
+  const int j = k0 + q;
+  // A_ij lives in tile (max(i, j), min(i, j)) of the lower triangle
+  const T *src = e.A + (int64_t)max(i, j) * 64 * ld + min(i, j) * 64;
+  T *dst = (buf ? e.Wp[1] : e.Wp[0]) + (int64_t)i * 64 * ldw + q * 64;
+  if (i > j) {
     for (int idx = threadIdx.x; idx < 4096; idx += 256)
-      S[(idx >> 6) * 65 + (idx & 63)] = src[(int64_t)(idx >> 6) * ld + (idx & 63)];
-    __syncthreads();
-    T *dst = (buf ? e.Wp[1] : e.Wp[0]) + (int64_t)i * 64 * ldw + q * 64;
-    for (int idx = threadIdx.x; idx < 4096; idx += 256) {
-      const int r = idx >> 6, c = idx & 63;
-      const bool direct = i > j || (i == j && r >= c);
-      dst[(int64_t)r * ldw + c] = direct ? S[r * 65 + c] : S[c * 65 + r];
-    }
-    __syncthreads();
-  }
-}
-
-// Pivot k = k0 + q of the panel: P = W_kq^-1 (FP64), and Vk = rows K of
-// column q as they stand before the pivot.
-constexpr int kPivotThreads = 512;
-
-// P and Vk of pivot q of a panel of parity buf, kept until the rows outside
-// the panel have taken the panel's pivots: 2 kSweepPanel slots of each
-template <typename T>
-__device__ __forceinline__ T *pivot_P(const SweepEntry<T> &e, int buf, int q) {
-  return e.P + (int64_t)(buf * kSweepPanel + q) * 4096;
-}
-template <typename T>
-__device__ __forceinline__ T *pivot_Vk(const SweepEntry<T> &e, int buf, int q) {
-  return e.Vk + (int64_t)(buf * kSweepPanel + q) * kSweepPanel * 4096;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kPivotThreads) k_bsweep_pivot(SweepBatch<T> bt, int k0, int q, int bw, int buf,
-                                                                int32_t *err_flag) {
-  const SweepEntry<T> e = bt.e[blockIdx.x];
-  constexpr int ldw = 64 * kSweepPanel;
-  const T *W = (buf ? e.Wp[1] : e.Wp[0]);
-  T *Vk = pivot_Vk(e, buf, q);
-  // 16-byte rows: ldw, q * 64 and the Vk row length are multiples of 4 elements
-  constexpr int V = 16 / sizeof(T);
-  using Vec = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-#pragma unroll 4
-  for (int idx = threadIdx.x; idx < bw * 64 * (64 / V); idx += kPivotThreads) {
-    const int r = idx / (64 / V), c = (idx % (64 / V)) * V;
-    *reinterpret_cast<Vec *>(Vk + r * 64 + c) =
-        *reinterpret_cast<const Vec *>(W + (int64_t)(k0 * 64 + r) * ldw + q * 64 + c);
-  }
-  invert_pivot_tile<kPivotThreads>(W + (int64_t)(k0 + q) * 64 * ldw + q * 64, ldw, pivot_P(e, buf, q), err_flag,
-                                   bt.pivot_fp64 != 0);
-}
-
-// One pivot on the panel, CTA per row tile i:
-//   U_i = W_iq P,  V_i = W_iq           (saved at column q of U, V)
-//   W_ij -= U_i Vk_j^T                  (panel columns j != q)
-//   W_iq <- U_i,  W_kj <- U_j^T (j in K),  W_kq <- -P.
-// Row k belongs to no CTA's update, so the writes never overlap.  The 64 x 64
-// products stage both operands whole in shared memory, the left one
-// transposed (sA[kk][r]); each thread owns the 4 x 4 block at rows 4 ty,
-// columns 4 tx and reads 4 + 4 operands per k with two 16-byte loads.
-constexpr int kPanelLd = 68;   // padded shared row: 16-byte aligned, staggered banks
-
-__device__ __forceinline__ void panel_mma64(const float *sA, const float *sB, float acc[4][4]) {
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-#pragma unroll 8
-  for (int kk = 0; kk < 64; ++kk) {
-    const float4 a = *reinterpret_cast<const float4 *>(sA + kk * kPanelLd + 4 * ty);
-    const float4 b = *reinterpret_cast<const float4 *>(sB + kk * kPanelLd + 4 * tx);
-    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-  }
-}
-
-// dst[kk][r] = src[r][kk] for a 64 x 64 tile at src (row stride lds); lanes
-// take consecutive rows so that the shared stores do not conflict
-__device__ __forceinline__ void panel_load_transposed(float *dst, const float *src, int64_t lds) {
-  for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-    const int r = e & 63, k4 = (e >> 6) * 4;
-    const float4 v = *reinterpret_cast<const float4 *>(src + r * lds + k4);
-    dst[(k4 + 0) * kPanelLd + r] = v.x;
-    dst[(k4 + 1) * kPanelLd + r] = v.y;
-    dst[(k4 + 2) * kPanelLd + r] = v.z;
-    dst[(k4 + 3) * kPanelLd + r] = v.w;
-  }
-}
-
-// A 64 x 64 tile (row stride lds) into registers, 4 float4 per thread: element
-// group e = threadIdx.x + 256 m holds row e & 63, columns 4 (e >> 6) .. + 3.
-__device__ __forceinline__ void tile_to_regs(const float *src, int64_t lds, float4 (&r)[4]) {
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int e = threadIdx.x + 256 * m;
-    r[m] = *reinterpret_cast<const float4 *>(src + (int64_t)(e & 63) * lds + (e >> 6) * 4);
-  }
-}
-// the same groups into shared memory transposed: dst[kk][r] = tile[r][kk]
-__device__ __forceinline__ void regs_to_smem_transposed(float *dst, const float4 (&r)[4]) {
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int e = threadIdx.x + 256 * m;
-    const int row = e & 63, k4 = (e >> 6) * 4;
-    dst[(k4 + 0) * kPanelLd + row] = r[m].x;
-    dst[(k4 + 1) * kPanelLd + row] = r[m].y;
-    dst[(k4 + 2) * kPanelLd + row] = r[m].z;
-    dst[(k4 + 3) * kPanelLd + row] = r[m].w;
-  }
-}
-
-// Pivot q of the panel on row tile i != k of the panel W (CTA-wide; sA, sB
-// staging of 64 x kPanelLd floats each).  Wk: row tile k's panel row, written
-// with U_i^T when i lies in the panel (else null).  Every global operand is
-// loaded into registers a step ahead of its use, so that the CTA waits on
-// memory about once per product instead of once per load.
-__device__ __forceinline__ void panel_row_step(float *Wi, float *Ui, float *Vi, const float *P, const float *Vk,
-                                               float *Wk, int q, int bw, float *sA, float *sB) {
-  constexpr int ldw = 64 * kSweepPanel;
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  float4 w[4], pr[4], vk[4];
-  tile_to_regs(Wi + q * 64, ldw, w);
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int idx = threadIdx.x + 256 * m;
-    pr[m] = *reinterpret_cast<const float4 *>(P + (idx >> 4) * 64 + (idx & 15) * 4);
-  }
-  int jj = (q == 0) ? 1 : 0;   // first panel column other than q
-  if (jj < bw) tile_to_regs(Vk + jj * 4096, 64, vk);
-  regs_to_smem_transposed(sA, w);
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const int idx = threadIdx.x + 256 * m;
-    *reinterpret_cast<float4 *>(sB + (idx >> 4) * kPanelLd + (idx & 15) * 4) = pr[m];
-    // V_i = A_ik before the pivot
-    const int e = idx;
-    *reinterpret_cast<float4 *>(Vi + (int64_t)(e & 63) * ldw + (e >> 6) * 4) = w[m];
-  }
-  __syncthreads();
-  float acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
-  panel_mma64(sA, sB, acc);
-  __syncthreads();  // sA is reused for U_i below; column q of W was read
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int r = 4 * ty + a;
-    const float4 v = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
-    *reinterpret_cast<float4 *>(Ui + (int64_t)r * ldw + 4 * tx) = v;
-    *reinterpret_cast<float4 *>(Wi + (int64_t)r * ldw + q * 64 + 4 * tx) = v;
-  }
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int c = 4 * tx + b;
-    const float4 v = make_float4(acc[0][b], acc[1][b], acc[2][b], acc[3][b]);
-    // U_i^T staged as the left operand of the updates: sA[kk][r] = U_i[r][kk]
-    *reinterpret_cast<float4 *>(sA + c * kPanelLd + 4 * ty) = v;
-    if (Wk) *reinterpret_cast<float4 *>(Wk + (int64_t)c * ldw + 4 * ty) = v;
-  }
-  while (jj < bw) {
-    int nx = jj + 1;
-    if (nx == q) ++nx;
-    __syncthreads();  // sB free, sA complete
-    // sB[kk][c] = Vk_jj[c][kk]
-    regs_to_smem_transposed(sB, vk);
-    if (nx < bw) tile_to_regs(Vk + nx * 4096, 64, vk);
-    float4 wij[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-      wij[a] = *reinterpret_cast<const float4 *>(Wi + (int64_t)(4 * ty + a) * ldw + jj * 64 + 4 * tx);
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
-    panel_mma64(sA, sB, acc);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      float4 w2 = wij[a];
-      w2.x -= acc[a][0];
-      w2.y -= acc[a][1];
-      w2.z -= acc[a][2];
-      w2.w -= acc[a][3];
-      *reinterpret_cast<float4 *>(Wi + (int64_t)(4 * ty + a) * ldw + jj * 64 + 4 * tx) = w2;
-    }
-    jj = nx;
-  }
-}
-
-// Pivot q of the panel on the panel's own row tiles i = k0 + blockIdx.x (the
-// rows the next pivot reads).  Row k takes -P; the other rows the step above.
-template <typename T>
-__global__ void __launch_bounds__(256) k_bsweep_panel(SweepBatch<T> bt, int k0, int q, int bw, int buf) {
-  static_assert(std::is_same<T, float>::value, "the panel-blocked sweep runs on float tiles");
-  __shared__ __align__(16) float sA[64 * kPanelLd];
-  __shared__ __align__(16) float sB[64 * kPanelLd];
-  const SweepEntry<T> e = bt.e[blockIdx.y];
-  constexpr int ldw = 64 * kSweepPanel;
-  const int i = k0 + blockIdx.x, k = k0 + q;
-  float *Wi = (buf ? e.Wp[1] : e.Wp[0]) + (int64_t)i * 64 * ldw;
-  float *Ui = (buf ? e.Up[1] : e.Up[0]) + (int64_t)i * 64 * ldw + q * 64;
-  float *Vi = (buf ? e.Vp[1] : e.Vp[0]) + (int64_t)i * 64 * ldw + q * 64;
-  const float *P = pivot_P(e, buf, q);
-  if (i == k) {
-    for (int idx = threadIdx.x; idx < 4096; idx += 256) {
-      const int64_t o = (int64_t)(idx >> 6) * ldw + (idx & 63);
-      Wi[o + q * 64] = -P[idx];
-      Ui[o] = 0.0f;
-      Vi[o] = 0.0f;
-    }
+      dst[(int64_t)(idx >> 6) * ldw + (idx & 63)] = src[(int64_t)(idx >> 6) * ld + (idx & 63)];
     return;
   }
-  float *Wk = (buf ? e.Wp[1] : e.Wp[0]) + (int64_t)k * 64 * ldw + (i - k0) * 64;
-  panel_row_step(Wi, Ui, Vi, P, pivot_Vk(e, buf, q), Wk, q, bw, sA, sB);
+  for (int idx = threadIdx.x; idx < 4096; idx += 256)
+    S[(idx >> 6) * 65 + (idx & 63)] = src[(int64_t)(idx >> 6) * ld + (idx & 63)];
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < 4096; idx += 256) {
+    const int r = idx >> 6, c = idx & 63;
+    dst[(int64_t)r * ldw + c] = (i == j && r >= c) ? S[r * 65 + c] : S[c * 65 + r];
+  }
 }
 
 // Column panel back into the lower tiles: A_ij for j in K from W row tile i
@@ -680,17 +475,16 @@ __global__ void __launch_bounds__(256) k_sweep_mirror(SweepBatch<T> bt, int ld, 
   }
 }
 
-static std::atomic<int> g_sweep_serial{0}, g_update_ctas{0}, g_update_stages{2}, g_pivot_shared{0};
+static std::atomic<int> g_sweep_serial{0}, g_update_ctas{0}, g_update_stages{3}, g_pivot_shared{0};
 int sweep_serial() { return g_sweep_serial.load(); }
 int update_cta_cap() { return g_update_ctas.load(); }
 int update_stages() { return g_update_stages.load(); }
 int pivot_exclusive() { return !g_pivot_shared.load(); }
-// Unused dynamic shared memory that keeps a pivot CTA (42 KB static) off the
-// SMs of the persistent rank-64 bw update (129 KB): 42 + 64 + 129 KB plus the
-// per-CTA reserve exceed the SM's 228 KB, so the pivot runs on an SM that the
-// update leaves free, beside panel CTAs only.
-constexpr int kPivotPad = 64 * 1024;
-
+int device_sms() {
+  int sms = 152, dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
 template <typename T>
 void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err_flag, int tc_passes,
                  const SweepStreams *ss) {
@@ -770,64 +564,39 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
                   2.0 * 64.0 * (r1 - r0) * 64.0 * bw1 * 64.0 * bw * b.count, compact);
       };
       const int n_panels = (nt + kSweepPanel - 1) / kSweepPanel;
-      // the update's CTA count, and the pivot CTAs' padding
+      // With one or two matrices a launch the pivot chain sets the pace: its CTAs
+      // get SMs of their own and the update leaves as many free.  With more, the
+      // update does, and takes every SM (measured per pass: two 9216-node matrices
+      // 276.8 ms exclusive, 289 shared; four of them 290.6 and 286.9; eight of 4096
+      // nodes 105.4 and 103.4).
+      const bool exclusive = pivot_exclusive() && b.count <= 2;
       int upd_ctas = update_cta_cap();
-      int pad = 0;
-      if (pivot_exclusive()) {
-        static std::once_flag once;
-        static bool pad_ok = false;
-        std::call_once(once, [] {
-          pad_ok = cudaFuncSetAttribute(k_bsweep_pivot<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        kPivotPad) == cudaSuccess;
-          if (!pad_ok) cudaGetLastError();
-        });
-        if (pad_ok) {
-          pad = kPivotPad;
-          if (upd_ctas == 0) {
-            int sms = 152, dev = 0;
-            if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            upd_ctas = std::max(1, sms - b.count);
-          }
-        }
-      }
-      ++g_launch_count;
-      {
-        ProfScope ps_(hi, PROF_PANEL);
-        k_bsweep_gather<T><<<dim3(nt, b.count), 256, 0, hi>>>(b, 0, std::min(kSweepPanel, nt), n_pad, 0);
-      }
+      if (exclusive && upd_ctas == 0) upd_ctas = std::max(1, device_sms() - kSweepPanel * b.count);
+      // column panel K' of A, row tiles [r0, r1) and [r2, r3), into Wp[buf]
+      auto gather = [&](cudaStream_t st, int k1, int bw1, int buf, int r0, int r1, int r2, int r3) {
+        const int n0 = r1 - r0, n1 = std::max(0, r3 - r2);
+        if (n0 + n1 <= 0) return;
+        ++g_launch_count;
+        ProfScope ps_(st, PROF_PANEL);
+        k_bsweep_gather<T><<<dim3((n0 + n1) * bw1, b.count), 256, 0, st>>>(b, k1, bw1, n_pad, buf, r0, n0, r2);
+      };
+      gather(hi, 0, std::min(kSweepPanel, nt), 0, 0, nt, 0, 0);
       for (int p = 0; p < n_panels; ++p) {
         const int k0 = p * kSweepPanel, bw = std::min(kSweepPanel, nt - k0), cur = p & 1;
         const bool has_next = p + 1 < n_panels;
         const int k1 = k0 + bw, bw1 = has_next ? std::min(kSweepPanel, nt - k1) : 0;
-        g_launch_count += 2 * bw;
-        for (int q = 0; q < bw; ++q) {
-          {
-            ProfScope ps_(hi, PROF_PIVOT, 2.0 * 64.0 * 64.0 * 64.0 * b.count);
-            k_bsweep_pivot<T><<<b.count, kPivotThreads, pad, hi>>>(b, k0, q, bw, cur, err_flag);
-          }
-          {
-            ProfScope ps_(hi, PROF_PANEL);
-            k_bsweep_panel<T><<<dim3(bw, b.count), 256, 0, hi>>>(b, k0, q, bw, cur);
-          }
-        }
+        launch_sweep_chain(hi, b, k0, bw, cur, err_flag, exclusive);
         if (has_next) {
           // rows K' of this panel: the previous panel's look-ahead on them ran on lo
           if (ss && p > 0) cudaStreamWaitEvent(hi, ss->lookahead, 0);
-          g_launch_count += 2;
+          ++g_launch_count;
           panel_apply(hi, cur, k0, bw, k1, k1 + bw1, split_ops);
           // columns K' as the previous update and scatter left them
           if (ss && p > 0) cudaStreamWaitEvent(hi, ss->scatter, 0);
-          {
-            ProfScope ps_(hi, PROF_PANEL);
-            k_bsweep_gather<T><<<dim3(nt, b.count), 256, 0, hi>>>(b, k1, bw1, n_pad, cur ^ 1);
-          }
+          gather(hi, k1, bw1, cur ^ 1, k1, k1 + bw1, 0, 0);
           // compact tiles: the product runs beside the previous panel's
           // persistent update instead of waiting for its SMs
           lookahead(hi, cur, k1, bw, bw1, k1, k1 + bw1, split_ops);
-          {
-            ProfScope ps_(hi, PROF_PANEL);
-            k_bsweep_rows<T><<<dim3(bw * bw1, b.count), 256, 0, hi>>>(b, k0, bw, k1, bw1, cur);
-          }
         }
         if (ss) {
           cudaEventRecord(ss->panel, hi);
@@ -836,6 +605,13 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
         // the swept panel on the other rows (outside K and K'), their look-ahead
         // (rows K come from k_bsweep_rows above), the update of the rest
         const int r1s = has_next ? k1 + bw1 : k1;   // other rows: [0, k0) and [r1s, nt)
+        if (has_next) {
+          // the next panel's other rows, and its rows K from this panel's U
+          gather(lo, k1, bw1, cur ^ 1, 0, k0, r1s, nt);
+          ++g_launch_count;
+          ProfScope ps_(lo, PROF_PANEL);
+          k_bsweep_rows<T><<<dim3(bw * bw1, b.count), 256, 0, lo>>>(b, k0, bw, k1, bw1, cur);
+        }
         bool fused = false;
         if (split_ops) {
           // W (the products' left operand and the update's right one) and U's
@@ -1480,7 +1256,7 @@ extern "C" qsel_status qsel_debug_sweep_schedule(int32_t serial, int32_t update_
     return QSEL_EINVAL;
   qsel::g_sweep_serial.store(serial ? 1 : 0);
   qsel::g_update_ctas.store(update_ctas);
-  qsel::g_update_stages.store(update_stages == 0 ? 2 : update_stages);
+  qsel::g_update_stages.store(update_stages == 0 ? 3 : update_stages);
   qsel::g_pivot_shared.store(shared_pivot ? 1 : 0);
   return QSEL_OK;
 }

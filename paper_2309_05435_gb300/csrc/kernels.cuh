@@ -212,14 +212,13 @@ OzSweep oz_sweep_at(void *base, int n_pad);
 template <typename T>
 struct SweepEntry {
   T *A;          // n_pad x n_pad, row-major, lower tiles used
-  T *P;          // 64 x 64 scratch (tensor-core path: 2 kSweepPanel of them, one
-                 // per panel parity and pivot)
+  T *P;          // 64 x 64 scratch (tensor-core path: kSweepPanel of them)
   T *U, *V;      // n_pad x 64 scratch each (tile-major)
-  // tensor-core path, one set per panel parity: the products U, the pivot
-  // columns V and the column panel W, n_pad x 64 kSweepPanel each (row-major)
-  T *Up[2], *Vp[2], *Wp[2];
-  T *Vk;         // tensor-core path: 2 kSweepPanel blocks of 64 kSweepPanel x 64 (the
-                 // panel rows of the pivot column, per panel parity and pivot)
+  // tensor-core path, one set per panel parity: the products U and the column
+  // panel W, n_pad x 64 kSweepPanel each (row-major)
+  T *Up[2], *Wp[2];
+  T *Vk;         // tensor-core path: kSweepPanel blocks of 64 kSweepPanel x 64 (the
+                 // panel rows of the pivot column, per pivot)
   T *Sp[4];      // tensor-core path: the panel update's U and V split into TF32 hi / lo
                  // (U_hi, U_lo, V_hi, V_lo; n_pad x 64 kSweepPanel each), or null
   OzSweep oz;    // double only
@@ -244,12 +243,19 @@ struct SweepBatch {
 // (double tiles) or double-float (float tiles).  err_flag gets bit 0 on a non-positive pivot.  For float with
 // tc_passes > 0 the pivots are taken kSweepPanel at a time on a gathered column
 // panel and the rest of the matrix gets one rank-64 kSweepPanel update per
-// panel on the tcgen05 tensor cores (Up, Vp, Wp and Vk are needed).  With ss the
+// panel on the tcgen05 tensor cores (Up, Wp and Vk are needed).  With ss the
 // next panel is pivoted on ss->hi while the update of the current one runs on
 // ss->lo (both joined back into s); without it everything runs on s.
 template <typename T>
 void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err_flag, int tc_passes = 0,
                  const SweepStreams *ss = nullptr);
+// The pivots of panel [k0, k0 + bw) of the tensor-core sweep on the panel's own
+// rows of Wp[buf], in one launch of a cluster per matrix (sweep_chain.cu).
+// exclusive: its CTAs keep off the SMs that the persistent update occupies.
+void launch_sweep_chain(cudaStream_t s, const SweepBatch<float> &b, int k0, int bw, int buf, int32_t *err,
+                        bool exclusive);
+// SMs of the current device.
+int device_sms();
 // Copy the lower tiles of each e[].A into its upper triangle (symmetric fill).
 template <typename T>
 void launch_mirror(cudaStream_t s, const SweepBatch<T> &b, int n_pad);

@@ -134,7 +134,7 @@ __device__ __forceinline__ dfloat df_sub(dfloat a, dfloat b) {
 // 1 / d: the float reciprocal and one Newton step r + r (1 - d r), whose
 // residual is formed exactly enough with two fused multiply-adds
 __device__ __forceinline__ dfloat df_recip(dfloat d) {
-  const float r = 1.0f / d.hi;
+  const float r = __frcp_rn(d.hi);   // correctly rounded, as 1 / d.hi
   float t = __fmaf_rn(-d.hi, r, 1.0f);
   t = __fmaf_rn(-d.lo, r, t);
   return df_fast_two_sum(r, __fmul_rn(r, t));
@@ -209,151 +209,5 @@ __device__ __forceinline__ void df_fma_acc(dfloat &acc, dfloat a, dfloat b) {
   acc.lo = __fadd_rn(acc.lo, __fadd_rn(s.lo, e));
 }
 __device__ __forceinline__ dfloat df_renorm(dfloat a) { return df_two_sum(a.hi, a.lo); }
-
-// Scalar sweep of a 32 x 32 SPD block held in the lower triangle of S (row
-// stride 33) in double-float: after the 32 pivots the lower triangle holds that
-// of -S^-1, then both halves are filled.  Each pivot reads the block as it
-// stood before the pivot from one buffer and writes the new values to the
-// other (S and T alternate; 32 pivots end in S), so a pivot costs one block
-// barrier: every thread forms 1 / d and reads column p itself, then updates
-// the lower entries it owns (528 entries, about one per thread):
-//   S_pp <- -1/d,  S_ip <- c_i / d,  S_ij <- S_ij - c_i (c_j / d).
-// A non-positive pivot sets bit 0 of *err_flag.  blockDim.x == NT.
-template <int NT>
-__device__ inline void df_sweep32(dfloat *S, dfloat *T, int32_t *err_flag) {
-  constexpr int EPT = (528 + NT - 1) / NT;
-  int ei[EPT], ej[EPT];
-#pragma unroll
-  for (int q = 0; q < EPT; ++q) {
-    const int e = (int)threadIdx.x + q * NT;
-    ei[q] = -1;
-    ej[q] = 0;
-    if (e < 528) {
-      int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-      while ((i + 1) * (i + 2) / 2 <= e) ++i;
-      while (i * (i + 1) / 2 > e) --i;
-      ei[q] = i;
-      ej[q] = e - i * (i + 1) / 2;
-    }
-  }
-  dfloat *src = S, *dst = T;
-  for (int p = 0; p < 32; ++p) {
-    const dfloat d = src[p * 33 + p];
-    const bool pos = d.hi > 0.0f;
-    const dfloat inv = pos ? df_recip(d) : dfloat{0.0f, 0.0f};
-    if (threadIdx.x == 0 && !pos && err_flag) atomicOr(err_flag, 1);
-#pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-      const int i = ei[q], j = ej[q];
-      if (i < 0) continue;
-      const dfloat ci = (i >= p) ? src[i * 33 + p] : src[p * 33 + i];
-      const dfloat cj = (j >= p) ? src[j * 33 + p] : src[p * 33 + j];
-      const dfloat wj = df_mul(cj, inv);
-      dfloat v;
-      if (i == p && j == p)
-        v = dfloat{-inv.hi, -inv.lo};
-      else if (i == p)
-        v = wj;
-      else if (j == p)
-        v = df_mul(ci, inv);
-      else
-        v = df_sub(src[i * 33 + j], df_mul(ci, wj));
-      dst[i * 33 + j] = v;
-    }
-    __syncthreads();
-    dfloat *t = src;
-    src = dst;
-    dst = t;
-  }
-  // 32 pivots: the result is in S
-  for (int e = threadIdx.x; e < 1024; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    if (i < j) S[i * 33 + j] = S[j * 33 + i];
-  }
-  __syncthreads();
-}
-
-// Shared scratch of sym_inverse64_df_2x2: the three blocks of the tile and
-// the two products, 32 x 32 each with row stride 33.
-struct Inverse64Smem {
-  dfloat B11[32 * 33], B21[32 * 33], B22[32 * 33], U[32 * 33], X[32 * 33];
-};
-
-// P = Tk^-1 (64 x 64 float, both halves) for the SPD tile whose lower half is
-// at Tk (row stride ld), in double-float, as a 2 x 2 block sweep: sweeping the
-// index blocks K1 = [0, 32) and then K2 = [32, 64) is the same as sweeping the
-// 64 indices one by one, and reads (N = -inverse of a swept block)
-//   N11 = -B11^-1,  U = B21 B11^-1 = -B21 N11,  B22' = B22 - U B21^T,
-//   N22 = -B22'^-1, X = B22'^-1 U = -N22 U,
-//   -Tk^-1 = [[N11 - U^T X, X^T], [X, N22]].
-// The 32 x 32 sweeps take one barrier per pivot with about one entry per
-// thread; the four 32-term block products run on all threads with their
-// sums in double-float.  A non-positive pivot sets bit 0 of *err_flag.
-// blockDim.x == NT >= 512.
-template <int NT>
-__device__ inline void sym_inverse64_df_2x2(const float *Tk, int ld, float *P, Inverse64Smem &S,
-                                             int32_t *err_flag) {
-  const int tid = threadIdx.x;
-  for (int e = tid; e < 1024; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    S.B11[i * 33 + j] = dfloat{Tk[(int64_t)max(i, j) * ld + min(i, j)], 0.0f};
-    S.B21[i * 33 + j] = dfloat{Tk[(int64_t)(32 + i) * ld + j], 0.0f};
-    if (i >= j) S.B22[i * 33 + j] = dfloat{Tk[(int64_t)(32 + i) * ld + 32 + j], 0.0f};
-  }
-  __syncthreads();
-  df_sweep32<NT>(S.B11, S.U, err_flag);   // B11 <- N11 (both halves; U as the second buffer)
-  // U = -B21 N11
-  for (int e = tid; e < 1024; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    dfloat acc{0.0f, 0.0f};
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) df_fma_acc(acc, S.B21[i * 33 + k], S.B11[k * 33 + j]);
-    acc = df_renorm(acc);
-    S.U[i * 33 + j] = dfloat{-acc.hi, -acc.lo};
-  }
-  __syncthreads();
-  // B22 <- B22 - U B21^T (lower)
-  for (int e = tid; e < 1024; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    if (i < j) continue;
-    dfloat acc{0.0f, 0.0f};
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) df_fma_acc(acc, S.U[i * 33 + k], S.B21[j * 33 + k]);
-    S.B22[i * 33 + j] = df_sub(S.B22[i * 33 + j], df_renorm(acc));
-  }
-  __syncthreads();
-  df_sweep32<NT>(S.B22, S.X, err_flag);   // B22 <- N22 (both halves; X as the second buffer)
-  // X = -N22 U
-  for (int e = tid; e < 1024; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    dfloat acc{0.0f, 0.0f};
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) df_fma_acc(acc, S.B22[i * 33 + k], S.U[k * 33 + j]);
-    acc = df_renorm(acc);
-    S.X[i * 33 + j] = dfloat{-acc.hi, -acc.lo};
-  }
-  __syncthreads();
-  // N11 <- N11 - U^T X (lower), and the output
-  for (int e = tid; e < 1024; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    if (i < j) continue;
-    dfloat acc{0.0f, 0.0f};
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) df_fma_acc(acc, S.U[k * 33 + i], S.X[k * 33 + j]);
-    const dfloat v = df_sub(S.B11[i * 33 + j], df_renorm(acc));
-    const float f = -__fadd_rn(v.hi, v.lo);
-    P[i * 64 + j] = f;
-    P[j * 64 + i] = f;
-  }
-  for (int e = tid; e < 1024; e += NT) {
-    const int i = e >> 5, j = e & 31;
-    const dfloat x = S.X[i * 33 + j];
-    const float fx = -__fadd_rn(x.hi, x.lo);
-    P[(32 + i) * 64 + j] = fx;
-    P[j * 64 + 32 + i] = fx;
-    const dfloat n = S.B22[i * 33 + j];
-    P[(32 + i) * 64 + 32 + j] = -__fadd_rn(n.hi, n.lo);
-  }
-}
 
 }  // namespace qsel
