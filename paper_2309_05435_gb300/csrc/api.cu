@@ -862,6 +862,7 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
   TRY(c->alloc(&c->d_corr4, (size_t)n));
   TRY(c->alloc(&c->d_traces, 4));
   TRY(c->alloc(&c->d_err, 4));
+  QSEL_CUDA_TRY(cudaMemset(c->d_err, 0, 4 * sizeof(int32_t)));
   TRY(c->alloc_bytes(reinterpret_cast<void **>(&c->d_diag_scratch), extract_scratch_bytes(n_pad)));
 
   // dense working sets: as many subdomains per wave as fit in 85 % of the free
@@ -1042,7 +1043,11 @@ static PcgVec<T> make_pcg(qsel_ctx *c, T *x, T *r, T *z, T *p, T *q) {
   v.n = c->n;
   v.ld = c->ld;
   v.n_blocks_dot = bt_spmm_grid(c->n);
-  v.n_tiles = pcg_update_grid(c->n);
+  // the block-Jacobi apply as digit products (the scalar Jacobi one, b = 1, is not
+  // a product)
+  v.oz = std::is_same<T, double>::value && !c->kron && c->bsize >= 16 && oz_available();
+  v.err = c->d_err;
+  v.n_tiles = v.oz ? oz_block_grid(c->n) : pcg_update_grid(c->n);
   v.x = x;
   v.r = r;
   v.z = z;
@@ -1107,7 +1112,10 @@ static Err pcg_solve(qsel_ctx *c, const PcgVec<T> &v, const T *pblk, double tol,
     if (c->h_counters[0] == 0) done = true;
   }
   QSEL_CUDA_TRY(cudaMemcpyAsync(c->h_small, v.max_rel, sizeof(double), cudaMemcpyDeviceToHost, s));
+  if (v.oz) QSEL_CUDA_TRY(cudaMemcpyAsync(c->h_counters, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   QSEL_CUDA_TRY(cudaStreamSynchronize(s));
+  if (v.oz && (c->h_counters[0] & 2))
+    return fail(QSEL_ETIMEOUT, "a bounded device-side wait of the preconditioner gave up");
   *iters = it;
   *max_rel = c->h_small[0];
   *converged = done;
@@ -1374,6 +1382,7 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
   const size_t vec = (size_t)c->n * c->ld;
   const int b = c->bsize;
   const int nblk = (c->n + b - 1) / b;
+  if (!oz_available()) return fail(QSEL_ECUDA, "the Lanczos sampler needs the tcgen05 tensor cores");
   if (!c->lz.ready) {
     for (auto &p : c->lz.vec) TRY(c->alloc(&p, vec));
     TRY(c->alloc(&c->lz.u, vec));
@@ -1420,12 +1429,12 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
       double *alpha_j = c->lz.alpha + (size_t)j * c->ld;
       double *beta_j = c->lz.beta + (size_t)j * c->ld;
       // w = L^-1 Q L^-T v  (the SpMM's time combination uses w as scratch)
-      launch_block_apply(s, c->lz.linv, b, c->n, c->ld, v, c->lz.u, true);
+      launch_oz_block_apply(s, c->lz.linv, b, true, c->n, c->ld, v, c->lz.u, nullptr, nullptr, c->d_err);
       sp.x = c->lz.u;
       sp.y = c->lz.q;
       sp.tmp = w;
       launch_bt_spmm<double>(s, sp);
-      launch_block_apply(s, c->lz.linv, b, c->n, c->ld, c->lz.q, w, false);
+      launch_oz_block_apply(s, c->lz.linv, b, false, c->n, c->ld, c->lz.q, w, nullptr, nullptr, c->d_err);
       if (pass == 0) {
         launch_lz_vec(s, 0, la, vp, v, w, nullptr, nullptr, beta_prev, c->lz.partial);
         launch_lz_reduce(s, la, c->lz.partial, false, alpha_j, nullptr);
@@ -1446,7 +1455,7 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
       launch_lz_quadrature(s, la, c->lz.alpha, c->lz.beta, c->lz.eta, c->lz.dwork, c->lz.U, c->lz.coef, c->d_err);
   }
   // rewind the preconditioner: x = L^-T x~
-  launch_block_apply(s, c->lz.linv, b, c->n, c->ld, c->lz.xt, c->d_X, true);
+  launch_oz_block_apply(s, c->lz.linv, b, true, c->n, c->ld, c->lz.xt, c->d_X, nullptr, nullptr, c->d_err);
   QSEL_CUDA_TRY(cudaGetLastError());
   c->stats.pcg_iterations = m;
   c->stats.pcg_max_rel_residual = 0.0;
@@ -3337,8 +3346,11 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
   launch_pcg_update<double>(s, v, pblk, c->bsize, c->kron ? &c->kop : nullptr);
   ce = cudaMemcpy2DAsync(Z, (size_t)ld * sizeof(double), c->d_zv, (size_t)c->ld * sizeof(double),
                          (size_t)c->k * sizeof(double), c->n, cudaMemcpyDeviceToHost, s);
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(c->h_counters, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
   if (ce != cudaSuccess) return finish(c, cuda_fail(ce, "preconditioner output", __FILE__, __LINE__));
+  if (c->h_counters[0] & 2)
+    return finish(c, fail(QSEL_ETIMEOUT, "a bounded device-side wait of the preconditioner gave up"));
   return QSEL_OK;
 }
 

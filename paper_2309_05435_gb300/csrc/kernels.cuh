@@ -131,6 +131,8 @@ struct PcgVec {
   int32_t *active;
   int32_t *counters;                  // [0] active columns
   double *max_rel;                    // [0] max relative residual
+  bool oz = false;                    // double: block-Jacobi apply as digit products
+  int32_t *err = nullptr;             // error word of its bounded waits
   const double *tol2_dev = nullptr;   // squared stopping tolerance in device memory (overrides the argument)
 };
 // Device-driven loops of captured graphs: the condition of a while node is
@@ -333,6 +335,13 @@ bool oz_available();
 bool launch_oz_gemm(cudaStream_t s, const OzGemmBatch &b, int M, int N, int K, int ldc, bool lower, int skip,
                     int32_t *err);
 
+// z = B x (trans: B^T x) for a block-diagonal B of b = 16, 32 or 64 rows a block
+// (block after block, row-major) and n x ld blocks x, z (ld <= 512, z not x); with
+// partial_xz, partial_xx non-null the column sums of x z and x x per CTA
+// (oz_block_grid(n) rows of ld).  Needs oz_available().
+int oz_block_grid(int n);
+void launch_oz_block_apply(cudaStream_t s, const double *B, int b, bool trans, int n, int ld, const double *x, double *z,
+                           double *partial_xz, double *partial_xx, int32_t *err);
 // One pivot k of the binary64 sweep on digit products: the column panel and its
 // digit planes (SweepEntry::oz), see oz_gemm.cu.
 void launch_oz_sweep_panel(cudaStream_t s, const SweepBatch<double> &b, int k, int n_pad, int32_t *err);
@@ -569,8 +578,6 @@ struct LanczosArgs {
 int lz_grid(int n);
 void launch_bj_cholinv(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t, int b,
                        double *linv, int32_t *err_flag);
-void launch_block_apply(cudaStream_t s, const double *linv, int b, int n, int ld, const double *x, double *y,
-                        bool trans);
 void launch_lz_vec(cudaStream_t s, int mode, const LanczosArgs &a, const double *vprev, const double *v, double *w,
                    double *xt, const double *coef, const double *scal, double *partial);
 void launch_lz_reduce(cudaStream_t s, const LanczosArgs &a, const double *partial, bool sqrt_out, double *out,

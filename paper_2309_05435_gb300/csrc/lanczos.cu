@@ -70,79 +70,6 @@ __global__ void __launch_bounds__(256) k_bj_cholinv(SellPattern pat, BtModel m, 
 // transpose (TRANS = true); b in {16, 32, 64}.  The block is staged so that
 // Bs[j][row] = B[row][j]; each thread accumulates an 8-row x 2-column tile.
 // ---------------------------------------------------------------------------
-template <bool TRANS>
-__global__ void __launch_bounds__(256) k_block_apply(const double *__restrict__ linv, int b, int n, int ld,
-                                                     const double *__restrict__ x, double *__restrict__ y) {
-  constexpr int PS = 66, RS = 66, CW = 64;
-  extern __shared__ __align__(16) double smem_apply[];
-  double *Bs = smem_apply;            // [64][PS]
-  double *xs = smem_apply + 64 * PS;  // [64][RS]
-  const int tid = threadIdx.x, rg = tid >> 5, cg = tid & 31;
-  const int n_blocks = (n + b - 1) / b;
-  const int n_tiles = (n + 63) / 64;
-  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int r0 = tile * 64;
-    const int rows = min(64, n - r0);
-    __syncthreads();
-    {
-      const int64_t base = (int64_t)(r0 / b) * b * b;
-      const int64_t lim = (int64_t)n_blocks * b * b;
-      for (int e = tid; e < 64 * b; e += blockDim.x) {
-        const int blk = e / (b * b), rem = e - blk * b * b;
-        const int r = rem / b, j = rem - r * b;
-        const double v = (base + e < lim) ? linv[base + e] : 0.0;
-        if (TRANS)
-          Bs[(blk * b + r) * PS + blk * b + j] = v;     // B = Linv^T: B[j][r] = Linv[r][j]
-        else
-          Bs[(blk * b + j) * PS + blk * b + r] = v;     // B = Linv
-      }
-    }
-    for (int c0 = 0; c0 < ld; c0 += CW) {
-      __syncthreads();
-      for (int e = tid; e < 64 * CW / 2; e += blockDim.x) {
-        const int rr = e / (CW / 2), q = e - rr * (CW / 2);
-        double2 val = make_double2(0.0, 0.0);
-        if (rr < rows) val = *reinterpret_cast<const double2 *>(x + (int64_t)(r0 + rr) * ld + c0 + 2 * q);
-        *reinterpret_cast<double2 *>(xs + rr * RS + 2 * q) = val;
-      }
-      __syncthreads();
-      const int row0 = rg * 8;
-      const int jb = (row0 / b) * b;
-      double z[8][2];
-#pragma unroll
-      for (int a = 0; a < 8; ++a) z[a][0] = z[a][1] = 0.0;
-      // B is triangular within its block: Linv is lower (j <= row), its
-      // transpose upper (j >= row); the zero half is skipped
-      const int j_lo = TRANS ? row0 - jb : 0;
-      const int j_hi = TRANS ? b : row0 + 8 - jb;
-      for (int jj = j_lo; jj < j_hi; ++jj) {
-        const int jl = jb + jj;
-        const double2 *pp = reinterpret_cast<const double2 *>(Bs + jl * PS + row0);
-        double pv[8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const double2 t2 = pp[u];
-          pv[2 * u] = t2.x;
-          pv[2 * u + 1] = t2.y;
-        }
-        const double2 rv = *reinterpret_cast<const double2 *>(xs + jl * RS + 2 * cg);
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          z[a][0] = fma(pv[a], rv.x, z[a][0]);
-          z[a][1] = fma(pv[a], rv.y, z[a][1]);
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const int rl = row0 + a;
-        if (rl < rows)
-          *reinterpret_cast<double2 *>(y + (int64_t)(r0 + rl) * ld + c0 + 2 * cg) = make_double2(z[a][0], z[a][1]);
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Lanczos vector kernels.  Rows are split across CTAs; within a CTA, 64
 // consecutive columns x 4 row groups; per-CTA partial column sums in double
 // are reduced in a fixed order by k_lz_reduce.  Columns >= k are held at 0.
@@ -343,24 +270,6 @@ void launch_bj_cholinv(cudaStream_t s, const SellPattern &pat, const BtModel &m,
   ++g_launch_count;
   const int nblk = (n_s * n_t + b - 1) / b;
   k_bj_cholinv<<<nblk, 256, smem, s>>>(pat, m, n_s, n_t, b, linv, err_flag);
-}
-
-void launch_block_apply(cudaStream_t s, const double *linv, int b, int n, int ld, const double *x, double *y,
-                        bool trans) {
-  constexpr int smem = 2 * 64 * 66 * (int)sizeof(double);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_block_apply<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k_block_apply<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
-  ++g_launch_count;
-  const int tiles = (n + 63) / 64;
-  const int grid = tiles < 152 * 4 ? tiles : 152 * 4;
-  if (trans)
-    k_block_apply<true><<<grid, 256, smem, s>>>(linv, b, n, ld, x, y);
-  else
-    k_block_apply<false><<<grid, 256, smem, s>>>(linv, b, n, ld, x, y);
 }
 
 void launch_lz_vec(cudaStream_t s, int mode, const LanczosArgs &a, const double *vprev, const double *v, double *w,

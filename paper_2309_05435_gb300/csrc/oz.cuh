@@ -39,14 +39,9 @@ __device__ __forceinline__ int64_t fixed62(double x, int32_t E) {
   const int field = (int)(bits >> 52) & 0x7ff;
   uint64_t m = bits & 0x000fffffffffffffULL;
   if (field) m |= 0x0010000000000000ULL;
-  const int up = 9 - (E + 1022 - max(field, 1));   // left shift that aligns m with 2^(62 - E)
-  uint64_t v;
-  if (up >= 0) {
-    v = m << up;
-  } else {
-    const int r = min(-up, 60);
-    v = (m + (1ULL << (r - 1))) >> r;
-  }
+  // m 2^10 shifted right by one more than the distance to the largest exponent
+  const int d = E + 1023 - max(field, 1), r = min(d, 63);
+  const uint64_t v = d > 63 ? 0 : ((m << 10) + (1ULL << (r - 1))) >> r;
   return (bits >> 63) ? -(int64_t)v : (int64_t)v;
 }
 

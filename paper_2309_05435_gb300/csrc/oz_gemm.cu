@@ -12,7 +12,7 @@
 //   warp 0      one thread issues the TMA loads of K = 32 stages (A: 8 digits x
 //               128 rows, B: 8 digits x 64 rows, 96 KB) into a 2-stage ring;
 //   warp 1      owns the 512 TMEM columns; one thread issues 12 MMAs per K = 16;
-//   warps 2-9   after every kChunk of K: tcgen05.ld, FP32 sums to integers, 64-bit
+//   warps 2-17  after every kChunk of K: tcgen05.ld, FP32 sums to integers, 64-bit
 //               integer accumulation (exact); at the end one rounding to binary64.
 // Every wait is bounded: after the limit the CTA raises bit 1 of *err, stops
 // issuing work, waits (bounded) for its loads and MMAs in flight, frees its
@@ -49,7 +49,8 @@ constexpr int A_BYTES = kDigits * A_TILE;      // 64 KiB
 constexpr int B_BYTES = kDigits * B_TILE;      // 32 KiB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 256 + 1024;
-constexpr int EP_WARPS = 8;
+constexpr int EP_WARPS = 16;
+constexpr int EP_COLS = 64 / (EP_WARPS / 4);   // columns of an epilogue warp
 constexpr int THREADS = 64 + 32 * EP_WARPS;
 constexpr int GROUP = 8;
 
@@ -216,9 +217,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
     }
   } else {
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = tile rows, columns
-    // 32 ((w - 2) / 4) .. + 31 of the tile
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + 32u * half;
+    // EP_COLS ((w - 2) / 4) .. of the tile
+    const int q = warp & 3, part = (warp - 2) >> 2;
+    const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(EP_COLS * part);
     const int n_chunks = (p.K + kChunk - 1) / kChunk;
     uint32_t chunk = 0;
     bool go = true;
@@ -227,9 +228,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
       int bm, bn;
       tile_of(p, L - z * p.per_matrix, bm, bn);
       if (bn == p.skip) continue;
-      int64_t hi[32], lo[32];
+      int64_t hi[EP_COLS], lo[EP_COLS];
 #pragma unroll
-      for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
+      for (int c = 0; c < EP_COLS; ++c) hi[c] = lo[c] = 0;
       for (int ch = 0; ch < n_chunks; ++ch, ++chunk) {
         int okay = 0;
         if (lane == 0) okay = mbar_wait(accf_bar, chunk & 1, abort, p.err, p.wait_cycles) && !*abort;
@@ -240,12 +241,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
         }
         tc_fence_after();
 #pragma unroll
-        for (int cb = 0; cb < 4; ++cb) accumulate8(t0 + 8u * cb, hi + 8 * cb, lo + 8 * cb);
+        for (int cb = 0; cb < EP_COLS / 8; ++cb) accumulate8(t0 + 8u * cb, hi + 8 * cb, lo + 8 * cb);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(accr_bar);
       }
-      const int row = bm * BM + 32 * q + lane, col = bn * BN_OZ + 32 * half;
+      const int row = bm * BM + 32 * q + lane, col = bn * BN_OZ + EP_COLS * part;
       if (!go || row >= p.M || col >= p.N || (row >> 6) == p.skip) continue;
       const bool neg = p.negate[z] != 0;
       const int32_t Ea = p.Ea[z][row];
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
       const double *c0 = p.C0[z] ? p.C0[z] + (int64_t)row * p.ldc + col : nullptr;
       double *c = p.C[z] + (int64_t)row * p.ldc + col;
 #pragma unroll
-      for (int cc = 0; cc < 32; cc += 2) {
+      for (int cc = 0; cc < EP_COLS; cc += 2) {
         double2 o = make_double2(value(hi[cc], lo[cc], Ea, Eb[cc], neg), value(hi[cc + 1], lo[cc + 1], Ea, Eb[cc + 1], neg));
         if (c0) {
           const double2 v = *reinterpret_cast<const double2 *>(c0 + cc);
@@ -399,7 +400,9 @@ struct PanelParams {
 constexpr int P_ROWB = 128;                                // K = 64: 128-byte rows
 constexpr int PA_TILE = BM * P_ROWB, PB_TILE = 64 * P_ROWB;
 constexpr int PANEL_SMEM = kDigits * (PA_TILE + PB_TILE) + 1024;
-constexpr int PANEL_THREADS = 256;
+constexpr int PANEL_THREADS = 512;
+constexpr int PARTS = PANEL_THREADS / BM;      // threads per row of the left operand
+constexpr int PART = 64 / PARTS;               // entries of a thread
 
 // Eight digits of eight neighbouring values: 16 bytes per digit plane to shared
 // (stride s_plane) and / or global memory (stride g_plane).
@@ -428,9 +431,33 @@ __device__ __forceinline__ void store_digits8(uint8_t *sdst, uint32_t s_plane, u
 }
 __device__ __forceinline__ int32_t finite_exponent(int32_t E) { return E == kNonFinite ? 1025 : E; }
 
+// Digits of the 64 x 64 matrix B(row, j) as the right operand at sb, its row
+// exponents to ep: eight threads per row, eight entries each.
+template <class F>
+__device__ __forceinline__ void matrix_digits(uint8_t *sb, int32_t *ep, F B) {
+  const int row = threadIdx.x >> 3, part = threadIdx.x & 7;
+  double y[8];
+  int g = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) y[u] = B(row, 8 * part + u);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) g = max(g, exp_field(y[u]));
+  for (int o = 1; o < 8; o <<= 1) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
+  const int32_t E = row_exponent(g);
+  if (part == 0) ep[row] = E;
+  store_digits8<true>(sb + row * P_ROWB + ((part ^ (row & 7)) << 4), PB_TILE, nullptr, 0, y, finite_exponent(E));
+}
+// The row exponent from the parts' largest exponent fields.
+__device__ __forceinline__ int32_t part_exponent(const int (&red)[PARTS][BM], int r) {
+  int f = red[0][r];
+#pragma unroll
+  for (int h = 1; h < PARTS; ++h) f = max(f, red[h][r]);
+  return row_exponent(f);
+}
+
 __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __grid_constant__ PanelParams p) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ int red[2][BM];
+  __shared__ int red[PARTS][BM];
   __shared__ int32_t ep[64];
   __shared__ __align__(8) uint64_t bar_mem;
   __shared__ uint32_t tmem_slot;
@@ -451,120 +478,93 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  const int q = warp & 3, half = warp >> 2;
+  const int q = warp & 3, part = warp >> 2;
   const int r = 32 * q + lane, gi = blockIdx.x * BM + r;
   const int i = gi >> 6;                        // this row's tile
-  const bool valid = gi < p.n_pad, on_pivot = i == k;
+  const bool valid = gi < p.n_pad, on_pivot = i == k, live = valid && !on_pivot;
   double *A = p.A[z];
   const double *P = p.P[z];
-  double x[32];
-  if (!valid || on_pivot) {
-#pragma unroll
-    for (int c = 0; c < 32; ++c) x[c] = 0.0;
-  } else if (i > k) {
-    const double *src = A + (int64_t)gi * ld + 64 * k + 32 * half;
-#pragma unroll
-    for (int c = 0; c < 32; c += 2) {
-      const double2 v = *reinterpret_cast<const double2 *>(src + c);
-      x[c] = v.x;
-      x[c + 1] = v.y;
-    }
-  } else {
-    // A_ik = A_ki^T (lower tiles are stored): consecutive lanes, consecutive columns
-    const double *src = A + (int64_t)(64 * k + 32 * half) * ld + gi;
-#pragma unroll
-    for (int c = 0; c < 32; ++c) x[c] = src[(int64_t)c * ld];
-  }
+  // this thread's PART entries of A_ik: along the row, or down the column of the
+  // stored A_ki (consecutive lanes, consecutive columns)
+  double *Ai = i > k ? A + (int64_t)gi * ld + 64 * k + PART * part : A + (int64_t)(64 * k + PART * part) * ld + gi;
+  const int64_t step = i > k ? 1 : ld;
   int f = 0;
-#pragma unroll
-  for (int c = 0; c < 32; ++c) f = max(f, exp_field(x[c]));
-  red[half][r] = f;
-  // P's digits: four threads per row, 16 entries each
-  {
-    const int pr = threadIdx.x >> 2, pq = threadIdx.x & 3;
-    double y[16];
-#pragma unroll
-    for (int c = 0; c < 16; c += 2) {
-      const double2 v = *reinterpret_cast<const double2 *>(P + pr * 64 + 16 * pq + c);
-      y[c] = v.x;
-      y[c + 1] = v.y;
-    }
-    int g = 0;
-#pragma unroll
-    for (int c = 0; c < 16; ++c) g = max(g, exp_field(y[c]));
-    g = max(g, __shfl_xor_sync(0xffffffffu, g, 1));
-    g = max(g, __shfl_xor_sync(0xffffffffu, g, 2));
-    const int32_t E = row_exponent(g);
-    if (pq == 0) ep[pr] = E;
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-      store_digits8<true>(sb + pr * P_ROWB + (((2 * pq + c) ^ (pr & 7)) << 4), PB_TILE, nullptr, 0, y + 8 * c,
-                          finite_exponent(E));
+  if (live) {
+#pragma unroll 16
+    for (int c = 0; c < PART; ++c) f = max(f, exp_field(Ai[c * step]));
   }
+  red[part][r] = f;
+  matrix_digits(sb, ep, [&](int row, int j) { return P[row * 64 + j]; });
   __syncthreads();
   const int64_t plane = (int64_t)p.n_pad * 64;
-  const int32_t Ea = row_exponent(max(red[0][r], red[1][r]));
-  {
-    uint16_t *gd = valid ? p.V[z] + (int64_t)gi * 64 + 32 * half : nullptr;
+  const int32_t Ea = part_exponent(red, r);
+  // the digits eight values at a time in a loop: unrolled, the kernel waited on
+  // instruction fetches for most of its time
+#pragma unroll 1
+  for (int c = 0; c < PART / 8; ++c) {
+    double x[8];
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-      store_digits8<true>(sa + r * P_ROWB + (((4 * half + c) ^ (r & 7)) << 4), PA_TILE, gd ? gd + 8 * c : nullptr, plane,
-                          x + 8 * c, finite_exponent(Ea));
-    if (valid && half == 0) p.Ev[z][gi] = Ea;
+    for (int u = 0; u < 8; ++u) x[u] = live ? Ai[(8 * c + u) * step] : 0.0;
+    store_digits8<true>(sa + r * P_ROWB + (((PART / 8 * part + c) ^ (r & 7)) << 4), PA_TILE,
+                        valid ? p.V[z] + (int64_t)gi * 64 + PART * part + 8 * c : nullptr, plane, x, finite_exponent(Ea));
   }
+  if (valid && part == 0) p.Ev[z][gi] = Ea;
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   if (threadIdx.x == 0) {
-#pragma unroll
+#pragma unroll 1
     for (int j = 0; j < 4; ++j)
       mma_digits<P_ROWB>(tmem, smem_u32(sa) + 32 * j, smem_u32(sb) + 32 * j, PA_TILE, PB_TILE, j == 0);
     mma_commit(bar);
   }
   __syncwarp();
-  const bool okay = mbar_wait(bar, 0u, &abort_mem, p.err, p.wait_cycles);
+  const bool okay = __syncthreads_and(mbar_wait(bar, 0u, &abort_mem, p.err, p.wait_cycles));
   tc_fence_after();
-  __syncwarp();
-  if (__all_sync(0xffffffffu, okay)) {
-    const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + 32u * half;
-    f = 0;
-#pragma unroll
-    for (int cb = 0; cb < 4; ++cb) {
+  // U staged in the shared memory of the operands (the MMAs have read them)
+  constexpr int kUld = 65;
+  double *su = reinterpret_cast<double *>(sa);
+  double *ur = su + r * kUld + PART * part;
+  f = 0;
+  if (okay) {
+    const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(PART * part);
+#pragma unroll 1
+    for (int cb = 0; cb < PART / 8; ++cb) {
       int64_t hi[8], lo[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
       accumulate8(t0 + 8u * cb, hi, lo);
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        x[8 * cb + c] = value(hi[c], lo[c], Ea, ep[32 * half + 8 * cb + c], false);
-        f = max(f, exp_field(x[8 * cb + c]));
+        const double u = value(hi[c], lo[c], Ea, ep[PART * part + 8 * cb + c], false);
+        f = max(f, exp_field(u));
+        ur[8 * cb + c] = u;
       }
     }
   }
-  __syncthreads();   // red was read by every thread before the MMAs
-  red[half][r] = f;
+  red[part][r] = f;
   __syncthreads();
-  const int32_t Eu = row_exponent(max(red[0][r], red[1][r]));
-  if (valid) {
-    uint16_t *gd = p.U[z] + (int64_t)gi * 64 + 32 * half;
+  const int32_t Eu = part_exponent(red, r);
+  if (okay && valid) {
+#pragma unroll 1
+    for (int c = 0; c < PART / 8; ++c) {
+      double x[8];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) store_digits8<false>(nullptr, 0, gd + 8 * c, plane, x + 8 * c, finite_exponent(Eu));
-    if (half == 0) p.Eu[z][gi] = Eu;
+      for (int u = 0; u < 8; ++u) x[u] = ur[8 * c + u];
+      store_digits8<false>(nullptr, 0, p.U[z] + (int64_t)gi * 64 + PART * part + 8 * c, plane, x, finite_exponent(Eu));
+      if (live) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) Ai[(8 * c + u) * step] = x[u];
+      }
+    }
+    if (part == 0) p.Eu[z][gi] = Eu;
     if (on_pivot) {
-      double *dst = A + (int64_t)gi * ld + 64 * k + 32 * half;
-      const double *src = P + (gi & 63) * 64 + 32 * half;
-#pragma unroll
-      for (int c = 0; c < 32; ++c) dst[c] = -src[c];
-    } else if (i > k) {
-      double *dst = A + (int64_t)gi * ld + 64 * k + 32 * half;
-#pragma unroll
-      for (int c = 0; c < 32; c += 2) *reinterpret_cast<double2 *>(dst + c) = make_double2(x[c], x[c + 1]);
-    } else {
-      double *dst = A + (int64_t)(64 * k + 32 * half) * ld + gi;
-#pragma unroll
-      for (int c = 0; c < 32; ++c) dst[(int64_t)c * ld] = x[c];
+      double *dst = A + (int64_t)gi * ld + 64 * k + PART * part;
+      const double *src = P + (gi & 63) * 64 + PART * part;
+#pragma unroll 8
+      for (int c = 0; c < PART; ++c) dst[c] = -src[c];
     }
   }
   tc_fence_before();
@@ -575,6 +575,170 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
+}
+
+// ---------------------------------------------------------------------------
+// z = B x for a block-diagonal B (blocks of b = 16, 32 or 64 rows; trans: B^T) and
+// n x ld blocks x, z; with partial sums, per CTA and column, of <x, z> and <x, x>.
+// 64 rows at a time: the transposed product z^T = x^T B^T, its M the columns (128
+// at a time), N the 64 rows, K = 64.  On the binary64 pipe this takes 64 FMAs per
+// entry of z, 2 per cycle and SM; here every SM forms the digits of one tile,
+// runs 48 MMAs and rounds, about 130 integer operations per entry.  512 threads:
+// with 256 the operations' latencies showed (43.6 against 62 us for two tiles of
+// 128 columns an SM).  Measured, n = 32768, 128 columns: 545 us on the binary64
+// pipe (k_pcg_precond) -> 82 us; n = 9216, 64 columns, without sums: 52 -> 17 us.
+// ---------------------------------------------------------------------------
+struct BlockParams {
+  const double *B, *x;
+  double *z, *pa, *pb;
+  int n, ld, b, log2b, trans;
+  int32_t *err;
+  long long wait_cycles;
+};
+
+template <bool DOTS>
+__global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __grid_constant__ BlockParams p) {
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ int red[PARTS][BM];
+  __shared__ int32_t ep[64];
+  __shared__ __align__(8) uint64_t bar_mem;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_mem;
+  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t *sa = base, *sb = base + kDigits * PA_TILE;
+  double *psum = reinterpret_cast<double *>(sb + kDigits * PB_TILE);   // [2 sums][PARTS][BM] of a column chunk
+  double *acc = psum + 2 * PARTS * BM;                                 // [2 sums][ld] of the CTA's tiles
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t bar = smem_u32(&bar_mem);
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    abort_mem = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  const int q = warp & 3, part = warp >> 2, cl = 32 * q + lane;
+  if (DOTS)
+    for (int c = threadIdx.x; c < 2 * p.ld; c += PANEL_THREADS) acc[c] = 0.0;
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const int n_tiles = (p.n + 63) / 64, n_blocks = (p.n + p.b - 1) / p.b;
+  uint32_t issued = 0;
+  bool go = true;
+  for (int tile = blockIdx.x; tile < n_tiles && go; tile += gridDim.x) {
+    const int r0 = tile * 64;
+    // the digits of B's rows (zero outside the blocks); the previous tile's MMAs
+    // have completed
+    const int blk0 = r0 >> p.log2b;
+    matrix_digits(sb, ep, [&](int row, int j) {
+      const int blk = row >> p.log2b, br = row & (p.b - 1), bj = j & (p.b - 1);
+      if (j >> p.log2b != blk || blk0 + blk >= n_blocks) return 0.0;
+      return p.B[((int64_t)(blk0 + blk) * p.b + (p.trans ? bj : br)) * p.b + (p.trans ? br : bj)];
+    });
+    const int rows = min(PART, max(0, p.n - r0 - PART * part));   // this thread's rows
+    for (int c0 = 0; c0 < p.ld && go; c0 += BM) {
+      const int col = c0 + cl;
+      const bool valid = col < p.ld;
+      const int64_t at = (int64_t)(r0 + PART * part) * p.ld + col;
+      const double *xc = p.x + at;
+      double *zc = p.z + at;
+      int f = 0;
+      if (valid) {
+#pragma unroll 16
+        for (int j = 0; j < rows; ++j) f = max(f, exp_field(xc[(int64_t)j * p.ld]));
+      }
+      red[part][cl] = f;
+      __syncthreads();
+      const int32_t Ea = part_exponent(red, cl);
+      // eight values at a time in loops, x re-read (from L1): unrolled over the
+      // tile, the kernel waited on instruction fetches for most of its time
+#pragma unroll 1
+      for (int c = 0; c < PART / 8; ++c) {
+        double x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = valid && 8 * c + u < rows ? xc[(int64_t)(8 * c + u) * p.ld] : 0.0;
+        store_digits8<true>(sa + cl * P_ROWB + (((PART / 8 * part + c) ^ (cl & 7)) << 4), PA_TILE, nullptr, 0, x,
+                            finite_exponent(Ea));
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+      if (threadIdx.x == 0) {
+#pragma unroll 1
+        for (int j = 0; j < 4; ++j)
+          mma_digits<P_ROWB>(tmem, smem_u32(sa) + 32 * j, smem_u32(sb) + 32 * j, PA_TILE, PB_TILE, j == 0);
+        mma_commit(bar);
+      }
+      __syncwarp();
+      const bool okay = mbar_wait(bar, issued & 1, &abort_mem, p.err, p.wait_cycles);
+      ++issued;
+      tc_fence_after();
+      go = __syncthreads_and(okay);
+      if (!go) break;
+      const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(PART * part);
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll 1
+      for (int cb = 0; cb < PART / 8; ++cb) {
+        int64_t hi[8], lo[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
+        accumulate8(t0 + 8u * cb, hi, lo);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int j = 8 * cb + c;
+          const double zv = value(hi[c], lo[c], Ea, ep[PART * part + j], false);
+          if (valid && j < rows) {
+            zc[(int64_t)j * p.ld] = zv;
+            if (DOTS) {
+              const double x = xc[(int64_t)j * p.ld];
+              s0 = fma(x, zv, s0);
+              s1 = fma(x, x, s1);
+            }
+          }
+        }
+      }
+      if (DOTS) {
+        psum[part * BM + cl] = s0;
+        psum[(PARTS + part) * BM + cl] = s1;
+      }
+      // red, ep and the shared operands are rewritten only after this barrier, psum
+      // only after the next one
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
+      if (DOTS && part < 2 && valid) {
+        double t = 0.0;
+#pragma unroll
+        for (int h = 0; h < PARTS; ++h) t += psum[(PARTS * part + h) * BM + cl];
+        acc[part * p.ld + col] += t;
+      }
+    }
+  }
+  __syncthreads();
+  if (DOTS)
+    for (int c = threadIdx.x; c < p.ld; c += PANEL_THREADS) {
+      p.pa[(int64_t)blockIdx.x * p.ld + c] = acc[c];
+      p.pb[(int64_t)blockIdx.x * p.ld + c] = acc[p.ld + c];
+    }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    if (lane == 0 && issued) drain(bar, (issued - 1) & 1);   // no MMA may still write the accumulator
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+}
+// operands, then the sums
+__host__ __device__ constexpr int block_smem(int ld, bool dots) {
+  return kDigits * (PA_TILE + PB_TILE) + 1024 + (dots ? 2 * (PARTS * BM + ld) * 8 : 0);
 }
 
 }  // namespace oz
@@ -631,7 +795,11 @@ bool oz_available() {
     oz::g_ok = cudaFuncSetAttribute(oz::k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM_BYTES) ==
                    cudaSuccess &&
                cudaFuncSetAttribute(oz::k_oz_sweep_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    oz::PANEL_SMEM) == cudaSuccess;
+                                    oz::PANEL_SMEM) == cudaSuccess &&
+               cudaFuncSetAttribute(oz::k_oz_block_apply<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    oz::block_smem(512, true)) == cudaSuccess &&
+               cudaFuncSetAttribute(oz::k_oz_block_apply<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    oz::block_smem(512, true)) == cudaSuccess;
     if (!oz::g_ok) cudaGetLastError();
   });
   return oz::g_ok;
@@ -699,6 +867,19 @@ void launch_oz_sweep_panel(cudaStream_t s, const SweepBatch<double> &b, int k, i
   ++g_launch_count;
   ProfScope ps_(s, PROF_PANEL);
   oz::k_oz_sweep_panel<<<dim3((n_pad + tc::BM - 1) / tc::BM, b.count), oz::PANEL_THREADS, oz::PANEL_SMEM, s>>>(p);
+}
+
+int oz_block_grid(int n) { return std::min((n + 63) / 64, device_sms()); }
+
+void launch_oz_block_apply(cudaStream_t s, const double *B, int b, bool trans, int n, int ld, const double *x, double *z,
+                           double *partial_xz, double *partial_xx, int32_t *err) {
+  oz::BlockParams p{B, x, z, partial_xz, partial_xx, n, ld, b, b == 64 ? 6 : b == 32 ? 5 : 4, trans ? 1 : 0, err,
+                    tc::wait_limit()};
+  ++g_launch_count;
+  if (partial_xz)
+    oz::k_oz_block_apply<true><<<oz_block_grid(n), oz::PANEL_THREADS, oz::block_smem(ld, true), s>>>(p);
+  else
+    oz::k_oz_block_apply<false><<<oz_block_grid(n), oz::PANEL_THREADS, oz::block_smem(ld, false), s>>>(p);
 }
 
 }  // namespace qsel

@@ -582,6 +582,19 @@ __global__ void __launch_bounds__(256) k_pcg_precond(PcgVec<T> v, const T *__res
 
 template <typename T>
 void launch_pcg_update(cudaStream_t s, const PcgVec<T> &v, const T *pblk, int bsize, const KronOperator *kron) {
+  if constexpr (std::is_same<T, double>::value) {
+    if (v.oz && !kron) {
+      g_launch_count += 1;
+      const int64_t vec2 = (int64_t)v.n * v.ld / 2;
+      {
+        ProfScope ps_(s, PROF_PCGVEC);
+        k_pcg_axpy<T><<<(int)std::min<int64_t>((vec2 + 255) / 256, 152 * 8), 256, 0, s>>>(v);
+      }
+      ProfScope ps_(s, PROF_PRECOND, 2.0 * bsize * (double)v.n * v.ld);
+      launch_oz_block_apply(s, pblk, bsize, false, v.n, v.ld, v.r, v.z, v.partial_a, v.partial_b, v.err);
+      return;
+    }
+  }
   // 128-column chunks for FP32 when they divide ld, else 64
   constexpr int CWF = std::is_same<T, float>::value ? 128 : 64;
   static bool attr_set = false;

@@ -68,3 +68,17 @@ def test_gradient_term_from_the_dense_inverse(q):
     q.qsel_set_data(ctx, qi.seeded_normal((int(model.obs_mask.sum()), 1), 7)[:, 0])
     _, (prior, _, _) = q.qsel_loglik_grad(ctx, with_terms=True)
     assert _rel(prior, oh.prior_logdet_grad(model, th)) <= 1e-10
+
+
+@pytest.mark.parametrize("m,n_t,k,block", [(5, 3, 10, 64), (9, 4, 70, 32), (8, 5, 130, 16), (13, 3, 200, 64)])
+def test_block_jacobi_apply(q, m, n_t, k, block):
+    """Z = P^-1 R block by block: one ragged 64-row tile, rows past n, blocks
+    smaller than the tile, one and several 128-column chunks."""
+    model, mesh, th = grid_model(m, n_t, 0.3), qi.grid_mesh(m), mk_theta(0.4, 1.1, 0.8)
+    ctx = _ctx(q, model, mesh, th, n_parts=1, overlap=0, n_samples=k, precond_block=block)
+    R = qi.seeded_normal((model.n, k), 9) * np.logspace(-6, 6, k)
+    Z = q.qsel_debug_apply_precond(ctx, R)
+    Q = o.precision(model, th).toarray()
+    ref = np.concatenate([np.linalg.solve(Q[a:a + block, a:a + block], R[a:a + block]) for a in range(0, model.n, block)])
+    # per column, against the column's largest entry: the digits are scaled by it
+    assert np.max(np.abs(Z - ref) / np.abs(ref).max(0)) <= 1e-11
