@@ -256,6 +256,8 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
 // exclusive: its CTAs keep off the SMs that the persistent update occupies.
 void launch_sweep_chain(cudaStream_t s, const SweepBatch<float> &b, int k0, int bw, int buf, int32_t *err,
                         bool exclusive);
+// P = A_kk^-1 for the 64 x 64 pivot tile of every entry, in binary64 (sweep_f64.cu).
+void launch_sweep_pivot_f64(cudaStream_t s, const SweepBatch<double> &b, int k, int ld, int32_t *err_flag);
 // SMs of the current device.
 int device_sms();
 // Copy the lower tiles of each e[].A into its upper triangle (symmetric fill).

@@ -48,9 +48,9 @@ constexpr int B_TILE = BN_OZ * ROWB;
 constexpr int A_BYTES = kDigits * A_TILE;      // 64 KiB
 constexpr int B_BYTES = kDigits * B_TILE;      // 32 KiB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 256 + 1024;
 constexpr int EP_WARPS = 16;
 constexpr int EP_COLS = 64 / (EP_WARPS / 4);   // columns of an epilogue warp
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 256 + 1024;
 constexpr int THREADS = 64 + 32 * EP_WARPS;
 constexpr int GROUP = 8;
 
@@ -253,6 +253,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
       const int32_t *Eb = p.Eb[z] + col;
       const double *c0 = p.C0[z] ? p.C0[z] + (int64_t)row * p.ldc + col : nullptr;
       double *c = p.C[z] + (int64_t)row * p.ldc + col;
+      // rows straight from the registers: staging them for whole-sector stores made
+      // no difference (39.6 against 37.4 us an update)
 #pragma unroll
       for (int cc = 0; cc < EP_COLS; cc += 2) {
         double2 o = make_double2(value(hi[cc], lo[cc], Ea, Eb[cc], neg), value(hi[cc + 1], lo[cc + 1], Ea, Eb[cc + 1], neg));
@@ -385,7 +387,8 @@ __global__ void k_oz_exponents(const __grid_constant__ SplitParams p) {
 // The product takes 64 x 64 x 64 binary64 FMAs per row tile, 63 us on one SM's
 // binary64 pipe; as digit products it is 48 MMAs.  The digits of A_ik are formed
 // in registers and stored to shared memory in the MMA's swizzled layout and to
-// global memory as V's at once.
+// global memory as V's at once.  70 us a pivot on the CUDA cores, 40 with a row per
+// thread, 25 with eight threads a row (whole sectors) at 1024 and 1600 nodes.
 // ---------------------------------------------------------------------------
 struct PanelParams {
   double *A[kMaxBatch];
@@ -457,8 +460,7 @@ __device__ __forceinline__ int32_t part_exponent(const int (&red)[PARTS][BM], in
 
 __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __grid_constant__ PanelParams p) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ int red[PARTS][BM];
-  __shared__ int32_t ep[64];
+  __shared__ int32_t ea[BM], ep[64];
   __shared__ __align__(8) uint64_t bar_mem;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_mem;
@@ -478,37 +480,38 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  const int q = warp & 3, part = warp >> 2;
-  const int r = 32 * q + lane, gi = blockIdx.x * BM + r;
-  const int i = gi >> 6;                        // this row's tile
-  const bool valid = gi < p.n_pad, on_pivot = i == k, live = valid && !on_pivot;
   double *A = p.A[z];
   const double *P = p.P[z];
-  // this thread's PART entries of A_ik: along the row, or down the column of the
-  // stored A_ki (consecutive lanes, consecutive columns)
-  double *Ai = i > k ? A + (int64_t)gi * ld + 64 * k + PART * part : A + (int64_t)(64 * k + PART * part) * ld + gi;
-  const int64_t step = i > k ? 1 : ld;
-  int f = 0;
-  if (live) {
-#pragma unroll 16
-    for (int c = 0; c < PART; ++c) f = max(f, exp_field(Ai[c * step]));
-  }
-  red[part][r] = f;
-  matrix_digits(sb, ep, [&](int row, int j) { return P[row * 64 + j]; });
-  __syncthreads();
   const int64_t plane = (int64_t)p.n_pad * 64;
-  const int32_t Ea = part_exponent(red, r);
-  // the digits eight values at a time in a loop: unrolled, the kernel waited on
-  // instruction fetches for most of its time
+  // Eight neighbouring entries of a row per thread and eight threads per row, so
+  // that rows, columns (of the stored A_ki, for i < k) and digit planes move in
+  // whole sectors: 64 rows at a time.
+  const int sub = threadIdx.x & 7;
+  auto entries = [&](int gi) {
+    return (gi >> 6) > k ? A + (int64_t)gi * ld + 64 * k + 8 * sub : A + (int64_t)(64 * k + 8 * sub) * ld + gi;
+  };
+  matrix_digits(sb, ep, [&](int row, int j) { return P[row * 64 + j]; });
 #pragma unroll 1
-  for (int c = 0; c < PART / 8; ++c) {
+  for (int r = threadIdx.x >> 3; r < BM; r += PANEL_THREADS / 8) {
+    const int gi = blockIdx.x * BM + r;
+    const bool valid = gi < p.n_pad, live = valid && (gi >> 6) != k;
+    const double *src = entries(gi);
+    const int64_t step = (gi >> 6) > k ? 1 : ld;
     double x[8];
+    int f = 0;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = live ? Ai[(8 * c + u) * step] : 0.0;
-    store_digits8<true>(sa + r * P_ROWB + (((PART / 8 * part + c) ^ (r & 7)) << 4), PA_TILE,
-                        valid ? p.V[z] + (int64_t)gi * 64 + PART * part + 8 * c : nullptr, plane, x, finite_exponent(Ea));
+    for (int u = 0; u < 8; ++u) x[u] = live ? src[u * step] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) f = max(f, exp_field(x[u]));
+    for (int o = 1; o < 8; o <<= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
+    const int32_t E = row_exponent(f);
+    if (sub == 0) {
+      ea[r] = E;
+      if (valid) p.Ev[z][gi] = E;
+    }
+    store_digits8<true>(sa + r * P_ROWB + ((sub ^ (r & 7)) << 4), PA_TILE,
+                        valid ? p.V[z] + (int64_t)gi * 64 + 8 * sub : nullptr, plane, x, finite_exponent(E));
   }
-  if (valid && part == 0) p.Ev[z][gi] = Ea;
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   tc_fence_before();
   __syncthreads();
@@ -526,10 +529,11 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
   // U staged in the shared memory of the operands (the MMAs have read them)
   constexpr int kUld = 65;
   double *su = reinterpret_cast<double *>(sa);
-  double *ur = su + r * kUld + PART * part;
-  f = 0;
   if (okay) {
+    const int q = warp & 3, part = warp >> 2, r = 32 * q + lane;
     const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(PART * part);
+    const int32_t Ea = ea[r];
+    double *ur = su + r * kUld + PART * part;
 #pragma unroll 1
     for (int cb = 0; cb < PART / 8; ++cb) {
       int64_t hi[8], lo[8];
@@ -537,34 +541,38 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
       for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
       accumulate8(t0 + 8u * cb, hi, lo);
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const double u = value(hi[c], lo[c], Ea, ep[PART * part + 8 * cb + c], false);
-        f = max(f, exp_field(u));
-        ur[8 * cb + c] = u;
-      }
+      for (int c = 0; c < 8; ++c)
+        ur[8 * cb + c] = value(hi[c], lo[c], Ea, ep[PART * part + 8 * cb + c], false);
     }
   }
-  red[part][r] = f;
   __syncthreads();
-  const int32_t Eu = part_exponent(red, r);
-  if (okay && valid) {
+  if (okay) {
 #pragma unroll 1
-    for (int c = 0; c < PART / 8; ++c) {
+    for (int r = threadIdx.x >> 3; r < BM; r += PANEL_THREADS / 8) {
+      const int gi = blockIdx.x * BM + r;
+      const bool valid = gi < p.n_pad, on_pivot = (gi >> 6) == k;
       double x[8];
+      int f = 0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = ur[8 * c + u];
-      store_digits8<false>(nullptr, 0, p.U[z] + (int64_t)gi * 64 + PART * part + 8 * c, plane, x, finite_exponent(Eu));
-      if (live) {
+      for (int u = 0; u < 8; ++u) x[u] = su[r * kUld + 8 * sub + u];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) Ai[(8 * c + u) * step] = x[u];
+      for (int u = 0; u < 8; ++u) f = max(f, exp_field(x[u]));
+      for (int o = 1; o < 8; o <<= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
+      const int32_t E = row_exponent(f);
+      if (!valid) continue;
+      if (sub == 0) p.Eu[z][gi] = E;
+      store_digits8<false>(nullptr, 0, p.U[z] + (int64_t)gi * 64 + 8 * sub, plane, x, finite_exponent(E));
+      if (on_pivot) {
+        double *dst = A + (int64_t)gi * ld + 64 * k + 8 * sub;
+        const double *src = P + (gi & 63) * 64 + 8 * sub;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) dst[u] = -src[u];
+      } else {
+        double *dst = entries(gi);
+        const int64_t step = (gi >> 6) > k ? 1 : ld;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) dst[u * step] = x[u];
       }
-    }
-    if (part == 0) p.Eu[z][gi] = Eu;
-    if (on_pivot) {
-      double *dst = A + (int64_t)gi * ld + 64 * k + PART * part;
-      const double *src = P + (gi & 63) * 64 + PART * part;
-#pragma unroll 8
-      for (int c = 0; c < PART; ++c) dst[c] = -src[c];
     }
   }
   tc_fence_before();
