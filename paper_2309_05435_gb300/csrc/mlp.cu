@@ -12,7 +12,9 @@
 // (14).  The forward pass reads BF16 copies of W1, W2, W3.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -31,8 +33,15 @@ static_assert(N_TRAIN == QSEL_CV_PARAMS, "parameter count");
 constexpr int TILE = 64;   // samples per backward CTA
 
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-  return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * __expf(-0.5f * x * x);
+
+// {a.x b.x + c.x, a.y b.y + c.y}, each rounded once: one issue slot for two FMAs.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<uint64_t &>(d))
+      : "l"(reinterpret_cast<uint64_t &>(a)), "l"(reinterpret_cast<uint64_t &>(b)),
+        "l"(reinterpret_cast<uint64_t &>(c)));
+  return d;
 }
 
 struct Weights {
@@ -40,14 +49,15 @@ struct Weights {
   const float *p;   // master parameters: biases, mean, scale
 };
 
-// Weights, biases, mean and scale staged in shared memory as float.
-struct SmemW {
-  float w1[H * NF], b1[H], w2[H * H], b2[H], w3[H], b3, mu[NF], sc[NF];
+// Weights (input unit first), biases, mean and scale staged in shared memory as
+// float.
+struct __align__(16) SmemW {
+  float w1[NF][H], w2[H][H], b1[H], b2[H], w3[H], b3, mu[NF], sc[NF];
 };
 
 __device__ void stage_weights(const Weights &W, SmemW &s) {
-  for (int i = threadIdx.x; i < H * NF; i += blockDim.x) s.w1[i] = __bfloat162float(W.w1[i]);
-  for (int i = threadIdx.x; i < H * H; i += blockDim.x) s.w2[i] = __bfloat162float(W.w2[i]);
+  for (int i = threadIdx.x; i < H * NF; i += blockDim.x) s.w1[i / H][i % H] = __bfloat162float(W.w1[(i % H) * NF + i / H]);
+  for (int i = threadIdx.x; i < H * H; i += blockDim.x) s.w2[i / H][i % H] = __bfloat162float(W.w2[(i % H) * H + i / H]);
   for (int i = threadIdx.x; i < H; i += blockDim.x) {
     s.w3[i] = __bfloat162float(W.w3[i]);
     s.b1[i] = W.p[OFF_B1 + i];
@@ -61,46 +71,153 @@ __device__ void stage_weights(const Weights &W, SmemW &s) {
   __syncthreads();
 }
 
-// One sample per thread.  With act set, a1 and a2 are stored (training).
+// S samples per thread.  With act set, a1 and a2 are stored (training).
+//
+// What bounds it: issue slots -- FMAs, the shared-memory reads that feed them and the
+// two error functions per unit.  The first layer's output goes through shared memory
+// (h1[unit][sample]; a thread reads what it wrote), so that both layers run as loops
+// over 16 units: kept in registers, the 64 units had to be unrolled, and every weight
+// was read once per sample and FMA.  A 16-byte read now serves 4 S FMAs, issued in
+// pairs; every sum keeps its order.  Measured, 524288 samples: 311 -> 178 us
+// (8 or 32 units: 191, 179; one sample per thread: 200); 65000 with act: 74 -> 36 us.
+template <int S>
+__host__ __device__ constexpr int forward_smem() {
+  return (int)sizeof(SmemW) + H * 256 * S * 4;
+}
+
+template <int S>
 __global__ void __launch_bounds__(256) k_mlp_forward(Weights W, const float *__restrict__ X, int n,
                                                      float *__restrict__ y, float *__restrict__ act) {
-  __shared__ SmemW s;
+  extern __shared__ __align__(16) unsigned char smem_f[];
+  SmemW &s = *reinterpret_cast<SmemW *>(smem_f);
+  float *h1s = reinterpret_cast<float *>(smem_f + sizeof(SmemW));   // [H][256 S]
   stage_weights(W, s);
-  for (int smp = blockIdx.x * blockDim.x + threadIdx.x; smp < n; smp += gridDim.x * blockDim.x) {
-    float xn[NF];
+  const bool pairs = (reinterpret_cast<uintptr_t>(X) & 7) == 0;   // a caller's rows may start on 4 bytes
+  constexpr int B = 16;   // units at a time
+  for (int64_t s0 = (int64_t)blockIdx.x * 256 * S; s0 < n; s0 += (int64_t)gridDim.x * 256 * S) {
+    float xn[S][NF];
+    float out[S];
 #pragma unroll
-    for (int k = 0; k < NF; ++k) xn[k] = (X[(int64_t)smp * NF + k] - s.mu[k]) / s.sc[k];
-    float h1[H];
+    for (int q = 0; q < S; ++q) {
+      const int64_t smp = min(s0 + q * 256 + threadIdx.x, (int64_t)n - 1);
 #pragma unroll
-    for (int j = 0; j < H; ++j) {
-      float a = s.b1[j];
-#pragma unroll
-      for (int k = 0; k < NF; ++k) a = fmaf(s.w1[j * NF + k], xn[k], a);
-      if (act) act[(int64_t)smp * 2 * H + j] = a;
-      h1[j] = gelu(a);
+      for (int k = 0; k < NF; k += 2) {
+        const float *x = X + smp * NF + k;
+        const float2 v = pairs ? *reinterpret_cast<const float2 *>(x) : make_float2(x[0], x[1]);
+        xn[q][k] = (v.x - s.mu[k]) / s.sc[k];
+        xn[q][k + 1] = (v.y - s.mu[k + 1]) / s.sc[k + 1];
+      }
+      out[q] = s.b3;
     }
-    float out = s.b3;
-    for (int j = 0; j < H; ++j) {
-      float a = s.b2[j];
+#pragma unroll 1
+    for (int j = 0; j < H; j += B) {
+      float2 a[S][B / 2];
 #pragma unroll
-      for (int k = 0; k < H; ++k) a = fmaf(s.w2[j * H + k], h1[k], a);
-      if (act) act[(int64_t)smp * 2 * H + H + j] = a;
-      out = fmaf(s.w3[j], gelu(a), out);
+      for (int q = 0; q < S; ++q)
+#pragma unroll
+        for (int u = 0; u < B / 2; ++u) a[q][u] = make_float2(s.b1[j + 2 * u], s.b1[j + 2 * u + 1]);
+#pragma unroll
+      for (int k = 0; k < NF; ++k) {
+        float2 w[B / 2];
+#pragma unroll
+        for (int u = 0; u < B / 2; u += 2)
+          *reinterpret_cast<float4 *>(w + u) = *reinterpret_cast<const float4 *>(&s.w1[k][j + 2 * u]);
+#pragma unroll
+        for (int q = 0; q < S; ++q)
+#pragma unroll
+          for (int u = 0; u < B / 2; ++u) a[q][u] = fma2(w[u], make_float2(xn[q][k], xn[q][k]), a[q][u]);
+      }
+#pragma unroll
+      for (int q = 0; q < S; ++q) {
+        const int64_t smp = s0 + q * 256 + threadIdx.x;
+        if (act && smp < n) {
+#pragma unroll
+          for (int u = 0; u < B / 2; u += 2)
+            *reinterpret_cast<float4 *>(act + smp * 2 * H + j + 2 * u) =
+                make_float4(a[q][u].x, a[q][u].y, a[q][u + 1].x, a[q][u + 1].y);
+        }
+#pragma unroll
+        for (int u = 0; u < B / 2; ++u) {
+          h1s[(j + 2 * u) * 256 * S + q * 256 + threadIdx.x] = gelu(a[q][u].x);
+          h1s[(j + 2 * u + 1) * 256 * S + q * 256 + threadIdx.x] = gelu(a[q][u].y);
+        }
+      }
     }
-    y[smp] = out;
+    // a thread reads its own samples' units only
+#pragma unroll 1
+    for (int j = 0; j < H; j += B) {
+      float2 a[S][B / 2];
+#pragma unroll
+      for (int q = 0; q < S; ++q)
+#pragma unroll
+        for (int u = 0; u < B / 2; ++u) a[q][u] = make_float2(s.b2[j + 2 * u], s.b2[j + 2 * u + 1]);
+#pragma unroll 8
+      for (int k = 0; k < H; ++k) {
+        float2 w[B / 2];
+#pragma unroll
+        for (int u = 0; u < B / 2; u += 2)
+          *reinterpret_cast<float4 *>(w + u) = *reinterpret_cast<const float4 *>(&s.w2[k][j + 2 * u]);
+#pragma unroll
+        for (int q = 0; q < S; ++q) {
+          const float h = h1s[k * 256 * S + q * 256 + threadIdx.x];
+#pragma unroll
+          for (int u = 0; u < B / 2; ++u) a[q][u] = fma2(w[u], make_float2(h, h), a[q][u]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < S; ++q) {
+        const int64_t smp = s0 + q * 256 + threadIdx.x;
+        if (act && smp < n) {
+#pragma unroll
+          for (int u = 0; u < B / 2; u += 2)
+            *reinterpret_cast<float4 *>(act + smp * 2 * H + H + j + 2 * u) =
+                make_float4(a[q][u].x, a[q][u].y, a[q][u + 1].x, a[q][u + 1].y);
+        }
+#pragma unroll
+        for (int u = 0; u < B / 2; ++u) {
+          out[q] = fmaf(s.w3[j + 2 * u], gelu(a[q][u].x), out[q]);
+          out[q] = fmaf(s.w3[j + 2 * u + 1], gelu(a[q][u].y), out[q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+      const int64_t smp = s0 + q * 256 + threadIdx.x;
+      if (smp < n) y[smp] = out[q];
+    }
   }
 }
 
+// Two samples per thread (a weight read serves both) where a block per SM would not
+// cover the samples with one; below that the second would only lengthen each thread's
+// work: 65000 samples take 10 us less with two.
+void launch_mlp_forward(cudaStream_t st, const Weights &W, const float *X, int n, float *y, float *act) {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_mlp_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, forward_smem<1>());
+    cudaFuncSetAttribute(k_mlp_forward<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, forward_smem<2>());
+  });
+  const int sms = device_sms();
+  if (n > 256 * sms)
+    k_mlp_forward<2><<<std::min((n - 1) / 512 + 1, sms), 256, forward_smem<2>(), st>>>(W, X, n, y, act);
+  else
+    k_mlp_forward<1><<<(n + 255) / 256, 256, forward_smem<1>(), st>>>(W, X, n, y, act);
+}
+
 // Backward for TILE samples per CTA: per-sample deltas in shared memory, then
-// the tile's partial weight gradients (mean-squared loss, 2 (y - t) / n).
+// the tile's partial weight gradients (mean-squared loss, 2 (y - t) / n).  The two
+// 64 x 64 x 64 products run on 4 x 4 register tiles with 16-byte shared reads (two
+// scalar reads per FMA bound them before), the activation's error function is
+// evaluated once per value; 161 -> 72 us for 65000 samples.
+constexpr int BLD = 68;   // padded row of the 64 x 64 tiles: 16-byte aligned
 struct SmemB {
+  float h1[TILE][BLD];
+  float h2[TILE][BLD];
+  float d2[TILE][BLD];
+  float d1[TILE][BLD];   // gelu'(a1) first, then delta1
+  float w2[H][BLD];
   float xn[TILE][NF + 1];
-  float h1[TILE][H + 1];
-  float h2[TILE][H + 1];
-  float d2[TILE][H + 1];
-  float d1[TILE][H + 1];   // holds a1 first, then delta1
-  float dy[TILE];
-  float lsum[TILE];
+  float w3[H], dy[TILE], lsum[TILE];
 };
 
 __global__ void __launch_bounds__(256) k_mlp_backward(Weights W, const float *__restrict__ X,
@@ -108,99 +225,172 @@ __global__ void __launch_bounds__(256) k_mlp_backward(Weights W, const float *__
                                                       const float *__restrict__ act, int n,
                                                       float *__restrict__ partial, float *__restrict__ loss_partial) {
   extern __shared__ __align__(16) unsigned char smem_b[];
-  SmemW &s = *reinterpret_cast<SmemW *>(smem_b);
-  SmemB &b = *reinterpret_cast<SmemB *>(smem_b + ((sizeof(SmemW) + 15) / 16) * 16);
-  stage_weights(W, s);
+  SmemB &b = *reinterpret_cast<SmemB *>(smem_b);
+  const int tid = threadIdx.x;
   const int s0 = blockIdx.x * TILE;
   const float inv_n = 2.0f / (float)n;
-  for (int e = threadIdx.x; e < TILE * H; e += blockDim.x) {
-    const int q = e / H, j = e - q * H;
-    const int smp = s0 + q;
-    float a1 = 0.f, a2 = 0.f;
-    if (smp < n) {
-      a1 = act[(int64_t)smp * 2 * H + j];
-      a2 = act[(int64_t)smp * 2 * H + H + j];
-    }
-    b.h1[q][j] = (smp < n) ? gelu(a1) : 0.f;
-    b.h2[q][j] = (smp < n) ? gelu(a2) : 0.f;
-    b.d1[q][j] = a1;
-    b.d2[q][j] = (smp < n) ? s.w3[j] * gelu_grad(a2) : 0.f;   // times dy below
+  for (int i = tid; i < H * H; i += 256) b.w2[i / H][i % H] = __bfloat162float(W.w2[i]);
+  if (tid < H) b.w3[tid] = __bfloat162float(W.w3[tid]);
+  if (tid < TILE) {
+    const int smp = s0 + tid;
+    const float diff = (smp < n) ? y[smp] - target[smp] : 0.f;
+    b.dy[tid] = diff * inv_n;
+    b.lsum[tid] = diff * diff;
   }
-  for (int e = threadIdx.x; e < TILE * NF; e += blockDim.x) {
+  for (int e = tid; e < TILE * NF; e += 256) {
     const int q = e / NF, k = e - q * NF;
     const int smp = s0 + q;
-    b.xn[q][k] = (smp < n) ? (X[(int64_t)smp * NF + k] - s.mu[k]) / s.sc[k] : 0.f;
-  }
-  if (threadIdx.x < TILE) {
-    const int smp = s0 + threadIdx.x;
-    const float diff = (smp < n) ? y[smp] - target[smp] : 0.f;
-    b.dy[threadIdx.x] = diff * inv_n;
-    b.lsum[threadIdx.x] = diff * diff;
+    b.xn[q][k] = (smp < n) ? (X[(int64_t)smp * NF + k] - W.p[OFF_MU + k]) / W.p[OFF_SC + k] : 0.f;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < TILE * H; e += blockDim.x) {
-    const int q = e / H, j = e - q * H;
-    b.d2[q][j] *= b.dy[q];
+  for (int e = tid; e < TILE * H / 4; e += 256) {
+    const int q = e / (H / 4), j = 4 * (e - q * (H / 4));
+    const int smp = s0 + q;
+    float4 v1 = make_float4(0.f, 0.f, 0.f, 0.f), v2 = v1;
+    if (smp < n) {
+      v1 = *reinterpret_cast<const float4 *>(act + (int64_t)smp * 2 * H + j);
+      v2 = *reinterpret_cast<const float4 *>(act + (int64_t)smp * 2 * H + H + j);
+    }
+    const float a1[4] = {v1.x, v1.y, v1.z, v1.w}, a2[4] = {v2.x, v2.y, v2.z, v2.w};
+    const float dy = b.dy[q];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float e1 = 1.0f + erff(a1[u] * 0.70710678118654752f), e2 = 1.0f + erff(a2[u] * 0.70710678118654752f);
+      const float g1 = 0.5f * e1 + a1[u] * 0.39894228040143268f * __expf(-0.5f * a1[u] * a1[u]);
+      const float g2 = 0.5f * e2 + a2[u] * 0.39894228040143268f * __expf(-0.5f * a2[u] * a2[u]);
+      // rows past n: a1 = a2 = 0 give zero activations, dy = 0 zero deltas
+      b.h1[q][j + u] = 0.5f * a1[u] * e1;
+      b.h2[q][j + u] = 0.5f * a2[u] * e2;
+      b.d1[q][j + u] = g1;
+      b.d2[q][j + u] = b.w3[j + u] * g2 * dy;
+    }
   }
   __syncthreads();
+  const int ty = tid >> 4, tx = tid & 15;
   // delta1[q][k] = (sum_j delta2[q][j] W2[j][k]) gelu'(a1[q][k])
-  for (int e = threadIdx.x; e < TILE * H; e += blockDim.x) {
-    const int q = e / H, k = e - q * H;
-    float acc = 0.f;
-#pragma unroll 8
-    for (int j = 0; j < H; ++j) acc = fmaf(b.d2[q][j], s.w2[j * H + k], acc);
-    b.d1[q][k] = acc * gelu_grad(b.d1[q][k]);
+  {
+    float acc[4][4] = {};
+#pragma unroll 4
+    for (int j = 0; j < H; j += 4) {
+      float4 dv[4], wv[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) dv[r] = *reinterpret_cast<const float4 *>(&b.d2[4 * ty + r][j]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) wv[u] = *reinterpret_cast<const float4 *>(&b.w2[j + u][4 * tx]);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float d[4] = {dv[r].x, dv[r].y, dv[r].z, dv[r].w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          acc[r][0] = fmaf(d[u], wv[u].x, acc[r][0]);
+          acc[r][1] = fmaf(d[u], wv[u].y, acc[r][1]);
+          acc[r][2] = fmaf(d[u], wv[u].z, acc[r][2]);
+          acc[r][3] = fmaf(d[u], wv[u].w, acc[r][3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float4 *g = reinterpret_cast<float4 *>(&b.d1[4 * ty + r][4 * tx]);
+      const float4 v = *g;
+      *g = make_float4(acc[r][0] * v.x, acc[r][1] * v.y, acc[r][2] * v.z, acc[r][3] * v.w);
+    }
   }
   __syncthreads();
   float *out = partial + (int64_t)blockIdx.x * N_TRAIN;
-  for (int e = threadIdx.x; e < H * H; e += blockDim.x) {   // W2[j][k]
-    const int j = e / H, k = e - j * H;
-    float acc = 0.f;
-    for (int q = 0; q < TILE; ++q) acc = fmaf(b.d2[q][j], b.h1[q][k], acc);
-    out[OFF_W2 + e] = acc;
+  // W2[j][k] = sum_q delta2[q][j] h1[q][k]
+  {
+    float acc[4][4] = {};
+#pragma unroll 8
+    for (int q = 0; q < TILE; ++q) {
+      const float4 dv = *reinterpret_cast<const float4 *>(&b.d2[q][4 * ty]);
+      const float4 hv = *reinterpret_cast<const float4 *>(&b.h1[q][4 * tx]);
+      const float d[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        acc[r][0] = fmaf(d[r], hv.x, acc[r][0]);
+        acc[r][1] = fmaf(d[r], hv.y, acc[r][1]);
+        acc[r][2] = fmaf(d[r], hv.z, acc[r][2]);
+        acc[r][3] = fmaf(d[r], hv.w, acc[r][3]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) out[OFF_W2 + (4 * ty + r) * H + 4 * tx + c] = acc[r][c];
   }
-  for (int e = threadIdx.x; e < H * NF; e += blockDim.x) {  // W1[j][k]
+  for (int e = tid; e < H * NF; e += 256) {  // W1[j][k]
     const int j = e / NF, k = e - j * NF;
     float acc = 0.f;
+#pragma unroll 8
     for (int q = 0; q < TILE; ++q) acc = fmaf(b.d1[q][j], b.xn[q][k], acc);
     out[OFF_W1 + e] = acc;
   }
-  for (int j = threadIdx.x; j < H; j += blockDim.x) {
-    float g1 = 0.f, g2 = 0.f, g3 = 0.f;
-    for (int q = 0; q < TILE; ++q) {
-      g1 += b.d1[q][j];
-      g2 += b.d2[q][j];
-      g3 = fmaf(b.dy[q], b.h2[q][j], g3);
-    }
-    out[OFF_B1 + j] = g1;
-    out[OFF_B2 + j] = g2;
-    out[OFF_W3 + j] = g3;
-  }
-  if (threadIdx.x == 0) {
-    float g = 0.f, l = 0.f;
-    for (int q = 0; q < TILE; ++q) {
-      g += b.dy[q];
-      l += b.lsum[q];
-    }
-    out[OFF_B3] = g;
-    loss_partial[blockIdx.x] = l;
+  // the biases, W3 and the two sums, a column sum per thread
+  const int which = tid / H, j = tid - which * H;
+  float g = 0.f;
+  if (which == 0) {
+#pragma unroll 8
+    for (int q = 0; q < TILE; ++q) g += b.d1[q][j];
+    out[OFF_B1 + j] = g;
+  } else if (which == 1) {
+#pragma unroll 8
+    for (int q = 0; q < TILE; ++q) g += b.d2[q][j];
+    out[OFF_B2 + j] = g;
+  } else if (which == 2) {
+#pragma unroll 8
+    for (int q = 0; q < TILE; ++q) g = fmaf(b.dy[q], b.h2[q][j], g);
+    out[OFF_W3 + j] = g;
+  } else if (j < 2) {
+    const float *v = j ? b.lsum : b.dy;
+#pragma unroll 8
+    for (int q = 0; q < TILE; ++q) g += v[q];
+    if (j)
+      loss_partial[blockIdx.x] = g;
+    else
+      out[OFF_B3] = g;
   }
 }
 
-// grad[p] = sum over tiles (fixed order, double), loss = mean squared error.
-__global__ void k_mlp_reduce(const float *__restrict__ partial, const float *__restrict__ loss_partial, int tiles,
-                             int n, float *__restrict__ grad, float *__restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < N_TRAIN) {
-    double acc = 0.0;
-    for (int t = 0; t < tiles; ++t) acc += partial[(int64_t)t * N_TRAIN + p];
+// grad[p] = sum over tiles (fixed order, double), loss = mean squared error: eight
+// parameters (a sector of each tile's row) x 32 groups of tiles per block, eight
+// partials in flight per thread.  Bound by the binary64 additions and conversions,
+// so the blocks are small enough to share the SMs evenly: 214 -> 24 us for 1016 tiles
+// (one thread per parameter walked all tiles alone; 32 parameters per block: 38 us,
+// 163 blocks on 152 SMs).
+constexpr int kReduceParams = 8, kReduceGroups = 32;
+
+__global__ void __launch_bounds__(kReduceParams *kReduceGroups)
+    k_mlp_reduce(const float *__restrict__ partial, const float *__restrict__ loss_partial, int tiles, int n,
+                 float *__restrict__ grad, float *__restrict__ loss) {
+  __shared__ double red[kReduceGroups][kReduceParams + 1];
+  const int lane = threadIdx.x % kReduceParams, g = threadIdx.x / kReduceParams;
+  const int p = blockIdx.x * kReduceParams + lane;
+  // the first index past the parameters sums the losses
+  const bool is_loss = p == N_TRAIN;
+  const float *src = is_loss ? loss_partial : partial + p;
+  const int64_t step = is_loss ? 1 : N_TRAIN;
+  double acc = 0.0;
+  if (p <= N_TRAIN) {
+    int t = g;
+    for (; t + 7 * kReduceGroups < tiles; t += 8 * kReduceGroups) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = src[(int64_t)(t + kReduceGroups * u) * step];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc += v[u];
+    }
+    for (; t < tiles; t += kReduceGroups) acc += src[(int64_t)t * step];
+  }
+  red[g][lane] = acc;
+  __syncthreads();
+  if (g != 0 || p > N_TRAIN) return;
+#pragma unroll
+  for (int h = 1; h < kReduceGroups; ++h) acc += red[h][lane];
+  if (is_loss)
+    *loss = (float)(acc / n);
+  else
     grad[p] = (float)acc;
-  }
-  if (p == 0) {
-    double l = 0.0;
-    for (int t = 0; t < tiles; ++t) l += loss_partial[t];
-    *loss = (float)(l / n);
-  }
 }
 
 // Adam on the FP32 master parameters, then the BF16 copies of W1, W2, W3.
@@ -264,65 +454,151 @@ __global__ void k_feature_stats(const float *__restrict__ X, int n, float *__res
 
 // ---------------------------------------------------------------------------
 // Per-node features of the current model for a given overlap (see the oracle
-// documentation for the definition).  One thread per node.
+// documentation for the definition).  One thread per spatial node and kFeatSlabs
+// slabs.  The eight largest entries and their logarithms depend on the slab only
+// through its block values and coefficients, which the separable model repeats
+// from slab to slab: they are formed again only where one of them differs in a bit.
+// 621 us at 524288 nodes with nine binary64 logarithms and an indexed, spilled list
+// per node; 35 us now, the latency of the first slab's sorting and of each slab's
+// loads (8 or 32 slabs per thread: 40, 46 us).
 // ---------------------------------------------------------------------------
-__global__ void k_cv_features(SellPattern pat, BtModel m, int n_s, int n_t, const float *__restrict__ sep_dist,
-                              const float *__restrict__ bnd_dist, double th0, double th1, double th2,
-                              float *__restrict__ F) {
-  const int n = n_s * n_t;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    const int t = r / n_s, i = r - t * n_s;
-    const int sl = i >> 5, li = i & 31;
-    const int w = pat.slice_width[sl];
-    const int base = pat.slice_ptr[sl] + li;
-    double diag = (m.obs && m.obs[r]) ? m.obs_w : 0.0;
-    double top[8];
+constexpr int kFeatSlabs = 16;
+
+// (float)log(a).  binary64 arithmetic holds a warp's issue slot for about 70 cycles an
+// instruction here, so a positive normal a = 2^e (1 + f), 1 + f in [sqrt(1/2), sqrt(2)),
+// takes pairs of floats: 2 atanh(s) = 2 s (1 + s^2/3 + s^4/5 + ...), s = f / (2 + f),
+// plus e ln 2.  The tail from s^4/5 on is in single precision, an error below 2^-34 of
+// the result: the rounding to float is what is left.
+__device__ __forceinline__ float log_to_float(double a) {
+  const long long bits = __double_as_longlong(a);
+  if (bits < 0x0010000000000000ll || bits >= 0x7ff0000000000000ll) return (float)log(a);
+  int e = (int)(bits >> 52) - 1023;
+  long long g = bits & 0xfffffffffffffll;   // f = g scale
+  float scale = 0x1p-52f;
+  if (g >= 0x6a09e667f3bcdll) {
+    g -= 0x10000000000000ll;
+    scale = 0x1p-53f;
+    ++e;
+  }
+  const float gh = __ll2float_rn(g), gl = __ll2float_rn(g - (long long)gh);
+  const float fh = gh * scale, fl = gl * scale;
+  const float dh = 2.f + fh, dl = ((2.f - dh) + fh) + fl;
+  const float sh = fh / dh, sl = (fmaf(-sh, dh, fh) + fmaf(-sh, dl, fl)) / dh;
+  const float th = sh * sh, tl = fmaf(sh, sh, -th) + 2.f * sh * sl;
+  constexpr float third = (float)(1.0 / 3.0), third_lo = (float)(1.0 / 3.0 - (double)third);
+  const float p = th * fmaf(th, fmaf(th, fmaf(th, fmaf(th, 1.f / 13.f, 1.f / 11.f), 1.f / 9.f), 1.f / 7.f), 1.f / 5.f);
+  const float ch = third + p, cl = (third - ch) + p + third_lo;
+  const float uh = th * ch, ul = fmaf(th, ch, -uh) + fmaf(th, cl, tl * ch);
+  const float ph = sh * uh, pl = fmaf(sh, uh, -ph) + fmaf(sh, ul, sl * uh);
+  const float zh = sh + ph, zl = ((sh - zh) + ph) + pl + sl;
+  constexpr double ln2 = 0.693147180559945309417232;
+  constexpr float l1 = (float)ln2, l2 = (float)(ln2 - (double)l1);
+  const float ef = (float)e, eh = ef * l1, el = fmaf(ef, l1, -eh) + ef * l2;
+  const float h = eh + 2.f * zh, back = h - eh;
+  const float err = (eh - (h - back)) + (2.f * zh - back);
+  return h + (err + fmaf(2.f, zl, el));
+}
+
+
+__global__ void __launch_bounds__(128) k_cv_features(SellPattern pat, BtModel m, int n_s, int n_t,
+                                                     const float *__restrict__ sep_dist,
+                                                     const float *__restrict__ bnd_dist, double th0, double th1,
+                                                     double th2, float *__restrict__ F) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_s) return;
+  const int sl = i >> 5, li = i & 31;
+  const int w = pat.slice_width[sl];
+  const int base = pat.slice_ptr[sl] + li;
+  const float bnd = bnd_dist[i];
+  const int t0 = blockIdx.y * kFeatSlabs, t1 = min(n_t, t0 + kFeatSlabs);
+  double c0 = 0.0, cm = 0.0, cp = 0.0;
+  const double *v0 = nullptr, *vm = nullptr, *vp = nullptr;
+  float ltop[8], lplain = 0.f, lobs = 0.f;   // lplain, lobs: the diagonal's without and with the observation
+  double dplain = 0.0, dobs = 0.0;
+  bool have_plain = false, have_obs = false;
+  const bool pairs = (reinterpret_cast<uintptr_t>(F) & 7) == 0;   // a caller's buffer may start on 4 bytes
 #pragma unroll
-    for (int q = 0; q < 8; ++q) top[q] = 0.0;
-    auto push = [&](double v) {
-      if (!(v > top[7])) return;
-      int q = 7;
-      while (q > 0 && top[q - 1] < v) {
-        top[q] = top[q - 1];
-        --q;
+  for (int q = 0; q < 8; ++q) ltop[q] = 0.f;
+  for (int t = t0; t < t1; ++t) {
+    // no coupling past the ends: its scale is zero, and a zero is never among the largest
+    const bool has_m = t > 0, has_p = t + 1 < n_t;
+    const double b0 = m.diag.scale(t), bm = has_m ? m.off.scale(t - 1) : 0.0, bp = has_p ? m.off.scale(t) : 0.0;
+    const double *u0 = m.diag.at(t), *um = has_m ? m.off.at(t - 1) : u0, *up = has_p ? m.off.at(t) : u0;
+    auto same = [](double x, double y) { return __double_as_longlong(x) == __double_as_longlong(y); };
+    if (t == t0 || !same(b0, c0) || !same(bm, cm) || !same(bp, cp) || u0 != v0 || um != vm || up != vp) {
+      c0 = b0;
+      cm = bm;
+      cp = bp;
+      v0 = u0;
+      vm = um;
+      vp = up;
+      // non-negative values order like their bit patterns: an insertion by integer
+      // comparisons, without branches
+      unsigned long long top[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) top[q] = 0;
+      auto push = [&](double a, bool use) {
+        unsigned long long v = (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
+        if (!use || v > 0x7ff0000000000000ull) v = 0;   // not a number: never larger
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const unsigned long long hi = v > top[q] ? v : top[q];
+          v = v > top[q] ? top[q] : v;
+          top[q] = hi;
+        }
+      };
+      dplain = 0.0;
+      dobs = m.obs_w;
+#pragma unroll 4
+      for (int s = 0; s < w; ++s) {
+        const int idx = base + s * kSlice;
+        const double v = c0 * v0[idx];
+        const double pm = cm * vm[idx], pp = cp * vp[idx];
+        const bool on = pat.col[idx] == i;
+        if (on) {
+          dplain += v;
+          dobs += v;
+        }
+        push(v, !on);
+        push(pm, has_m);
+        push(pp, has_p);
       }
-      top[q] = v;
-    };
-    const double c0 = m.diag.scale(t);
-    const double cm = t > 0 ? m.off.scale(t - 1) : 0.0, cp = t + 1 < n_t ? m.off.scale(t) : 0.0;
-    const double *v0 = m.diag.at(t);
-    const double *vm = m.off.at(t > 0 ? t - 1 : 0);
-    const double *vp = m.off.at(t + 1 < n_t ? t : 0);
-    for (int s = 0; s < w; ++s) {
-      const int idx = base + s * kSlice;
-      const int j = pat.col[idx];
-      const double v = c0 * v0[idx];
-      if (j == i)
-        diag += v;
-      else if (v != 0.0)
-        push(fabs(v));
-      if (t > 0 && vm[idx] != 0.0) push(fabs(cm * vm[idx]));
-      if (t + 1 < n_t && vp[idx] != 0.0) push(fabs(cp * vp[idx]));
-    }
-    float *f = F + (int64_t)r * mlp::NF;
-    f[0] = (float)log(diag);
+      have_plain = have_obs = false;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) f[1 + q] = (float)log(top[q] > 1e-30 ? top[q] : 1e-30);
-    f[9] = sep_dist[t];
-    f[10] = bnd_dist[i];
-    f[11] = (float)th0;
-    f[12] = (float)th1;
-    f[13] = (float)th2;
+      for (int q = 0; q < 8; ++q) {
+        const unsigned long long floor_bits = (unsigned long long)__double_as_longlong(1e-30);
+        const double a = __longlong_as_double((long long)(top[q] > floor_bits ? top[q] : floor_bits));
+        // a stencil's entries come in equal sets
+        ltop[q] = q > 0 && top[q] == top[q - 1] ? ltop[q - 1] : log_to_float(a);
+      }
+    }
+    const int64_t r = (int64_t)t * n_s + i;
+    const bool obs = m.obs && m.obs[r];
+    if (obs && !have_obs) {
+      lobs = log_to_float(dobs);
+      have_obs = true;
+    } else if (!obs && !have_plain) {
+      lplain = log_to_float(dplain);
+      have_plain = true;
+    }
+    float *f = F + r * mlp::NF;
+    const float row[mlp::NF] = {obs ? lobs : lplain, ltop[0], ltop[1], ltop[2], ltop[3], ltop[4], ltop[5],
+                                ltop[6], ltop[7], sep_dist[t], bnd, (float)th0, (float)th1, (float)th2};
+    if (pairs) {
+#pragma unroll
+      for (int k = 0; k < mlp::NF; k += 2) *reinterpret_cast<float2 *>(f + k) = make_float2(row[k], row[k + 1]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < mlp::NF; ++k) f[k] = row[k];
+    }
   }
 }
 
 void launch_cv_features(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t,
                         const float *sep_dist, const float *bnd_dist, const double th[3], float *F) {
   ++g_launch_count;
-  const int n = n_s * n_t;
-  int grid = (n + 255) / 256;
-  if (grid > 152 * 8) grid = 152 * 8;
-  k_cv_features<<<grid, 256, 0, s>>>(pat, m, n_s, n_t, sep_dist, bnd_dist, th[0], th[1], th[2], F);
+  k_cv_features<<<dim3((n_s + 127) / 128, (n_t + kFeatSlabs - 1) / kFeatSlabs), 128, 0, s>>>(
+      pat, m, n_s, n_t, sep_dist, bnd_dist, th[0], th[1], th[2], F);
 }
 
 // Per part p: sum over the rows of Omega_p (slabs [slab_start[p],
@@ -430,7 +706,7 @@ qsel_status cv_fail(qsel_status st, const std::string &m) {
 }
 
 int backward_smem() {
-  return (int)(((sizeof(mlp::SmemW) + 15) / 16) * 16 + sizeof(mlp::SmemB));
+  return (int)sizeof(mlp::SmemB);
 }
 
 qsel_status cv_forward_backward(qsel_cv *cv, const float *X, const float *target, int n) {
@@ -443,11 +719,11 @@ qsel_status cv_forward_backward(qsel_cv *cv, const float *X, const float *target
   if (!cv->ensure(n)) return cv_fail(QSEL_ENOMEM, "qsel_cv: device allocation failed");
   const int tiles = (n + TILE - 1) / TILE;
   g_launch_count += 3;
-  k_mlp_forward<<<std::min((n + 255) / 256, 152 * 4), 256, 0, cv->stream>>>(cv->weights(), X, n, cv->y, cv->act);
+  launch_mlp_forward(cv->stream, cv->weights(), X, n, cv->y, cv->act);
   k_mlp_backward<<<tiles, 256, backward_smem(), cv->stream>>>(cv->weights(), X, target, cv->y, cv->act, n,
                                                               cv->partial, cv->loss_partial);
-  k_mlp_reduce<<<(N_TRAIN + 255) / 256, 256, 0, cv->stream>>>(cv->partial, cv->loss_partial, tiles, n, cv->g,
-                                                               cv->loss);
+  k_mlp_reduce<<<N_TRAIN / kReduceParams + 1, kReduceParams * kReduceGroups, 0, cv->stream>>>(
+      cv->partial, cv->loss_partial, tiles, n, cv->g, cv->loss);
   return cudaGetLastError() == cudaSuccess ? QSEL_OK : cv_fail(QSEL_ECUDA, "qsel_cv: kernel launch failed");
 }
 }  // namespace
@@ -519,8 +795,7 @@ qsel_status qsel_cv_get_params(const qsel_cv *cv, float *params) {
 qsel_status qsel_cv_predict(const qsel_cv *cv, const float *X_dev, float *y_dev, int32_t n) {
   if (!cv || !X_dev || !y_dev || n < 1) return cv_fail(QSEL_EINVAL, "qsel_cv_predict: invalid argument");
   ++g_launch_count;
-  mlp::k_mlp_forward<<<std::min((n + 255) / 256, 152 * 4), 256, 0, cv->stream>>>(cv->weights(), X_dev, n, y_dev,
-                                                                                  nullptr);
+  mlp::launch_mlp_forward(cv->stream, cv->weights(), X_dev, n, y_dev, nullptr);
   if (cudaStreamSynchronize(cv->stream) != cudaSuccess) return cv_fail(QSEL_ECUDA, "qsel_cv_predict: kernel failed");
   return QSEL_OK;
 }
