@@ -37,7 +37,7 @@
  *   - Work is issued on the CUDA stream given in qsel_options (NULL = the
  *     legacy default stream); every call returns after the stream has reached
  *     the end of its work (results are ready on return).  Inside a call the
- *     context may fork work onto non-blocking streams of its own (the PCG
+ *     context may fork work onto non-blocking streams of its own (the sampler
  *     beside the first wave's factorisation, the sweep's look-ahead) and
  *     joins them back into that stream before it returns.
  *   - One context must not be used from two threads at the same time.
@@ -222,7 +222,8 @@ typedef struct {
 typedef struct {
   int32_t pcg_iterations;     /* iterations until every column met pcg_tol         */
   double pcg_max_rel_residual;/* max over columns of ||b - Q x|| / ||b|| at exit   */
-  double ms_rhs;              /* device time of each phase, milliseconds           */
+  double ms_rhs;              /* device time of each phase, milliseconds; those of
+                                 the sampler and of the first wave may overlap     */
   double ms_pcg;
   double ms_factor;           /* forward block factorisation (all subdomains)      */
   double ms_takahashi;        /* backward selected inversion (all subdomains)      */

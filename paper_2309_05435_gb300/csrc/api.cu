@@ -186,7 +186,7 @@ struct qsel_ctx {
   double *h_small = nullptr;
   cudaEvent_t ev[4]{};
   SweepStreams sweep_ss;               // look-ahead of the tensor-core sweep (mixed path)
-  cudaStream_t pcg_stream = nullptr;   // the PCG sampler, beside the first wave's dense part
+  cudaStream_t pcg_stream = nullptr;   // the sampler, beside the first wave's dense part
   cudaEvent_t ev_fork = nullptr, ev_samples = nullptr;
   std::vector<cudaEvent_t> phase_ev;   // pairs per (wave, phase)
   size_t phase_used = 0;
@@ -2046,19 +2046,27 @@ static Err run_pipeline_body(qsel_ctx *c) {
     return c->mixed ? run_wave<float>(c, p0, p1, marks, stages) : run_wave<double>(c, p0, p1, marks, stages);
   };
   int first = 0;   // first wave still to run in full
-  if (c->mixed && !c->injected && need_samples && c->opt.sampler == QSEL_SAMPLER_PCG) {
+  const bool beside = (c->mixed && c->opt.sampler == QSEL_SAMPLER_PCG) ||
+                      ((c->mixed || c->oz) && !c->opt.profile_kernels);
+  if (beside && !c->injected && need_samples) {
     // The samples are needed only by the correction: the first wave's
     // factorisation and Takahashi recursion are enqueued on the context's
-    // stream and run while the PCG (whose host loop synchronises only its
-    // own stream) runs on pcg_stream.  Mixed form only: in FP64 both parts
-    // run on the FP64 pipe, and sequential phases keep its phase times
-    // (which the plain-FP64 time-to-target model scales) additive.
+    // stream and run while the sampler (the PCG's host loop synchronises only
+    // its own stream) runs on pcg_stream.  In binary64 this takes the digit
+    // products: the sampler's SpMM holds the FP64 pipe and the Lanczos
+    // quadrature two SMs, the dense part the tensor cores.  Dense products on the
+    // FP64 pipe would only take turns with it, and a profiled pass of these forms
+    // stays sequential, so that its launches are timed alone.  Measured in
+    // binary64: 64 samples on 16 x 16 x 8 16.7 -> 13.3 ms, Lanczos on 24 x 24 x 16
+    // 38.7 -> 29.2 ms, 32 x 32 x 32 with 128 samples 120 -> 115 ms (the PCG's
+    // blocks leave little room; a stream of higher priority for the dense part
+    // changed nothing).
     QSEL_CUDA_TRY(cudaEventRecord(c->ev_fork, s));
     first = std::min(np, c->wave);
     TRY(wave(0, first, 1));
     QSEL_CUDA_TRY(cudaStreamWaitEvent(c->pcg_stream, c->ev_fork, 0));
     c->stream = c->pcg_stream;
-    Err e = run_sampler(c);
+    Err e = c->opt.sampler == QSEL_SAMPLER_LANCZOS ? run_sampler_lanczos(c) : run_sampler(c);
     if (e.code == 0 && cudaEventRecord(c->ev[2], c->pcg_stream) != cudaSuccess)
       e = fail(QSEL_ECUDA, "event record failed");
     if (e.code == 0 && cudaEventRecord(c->ev_samples, c->pcg_stream) != cudaSuccess)
