@@ -8,14 +8,14 @@
 // epilogue writes that axis contiguously.  Axes s (samples, ld), t (n_t),
 // i, j (m); layouts slowest axis first:
 //   r (t, i, j, s)  --transpose, x Dh_i Dh_j-->                  (s, t, i, j)
-//   P1  V^T over j, rows along i (32) x t (4)                ->  (s, t, j, i)
-//   P2  V^T over i, rows along t (128)                        ->  (s, j, i, t)
-//   P3  U^T over t, x spectral scaling, rows along i x j     ->  (s, t, j, i)
+//   P1  V^T over j, rows along i x t (x s)                    ->  (s, t, j, i)
+//   P2  V^T over i, rows along t (x s)                        ->  (s, j, i, t)
+//   P3  U^T over t, x spectral scaling, rows along i x j      ->  (s, t, j, i)
 //       (the scaling 1 / (tau mu_t (kappa^2 + lambda_i + lambda_j)^2 + omega)
 //       is formed in the epilogue from mu and lambda, in binary32)
-//   P4  V over i, rows along j (32) x t (4)                   ->  (s, t, i, j)
-//   P5  V over j, rows along t (128)                          ->  (s, i, j, t)
-//   P6  U over t, x Dh_i Dh_j, rows along s (128)             ->  z (t, i, j, s)
+//   P4  V over i, rows along j x t (x s)                      ->  (s, t, i, j)
+//   P5  V over j, rows along t (x s)                          ->  (s, i, j, t)
+//   P6  U over t, x Dh_i Dh_j, rows along s (x j)             ->  z (t, i, j, s)
 // A pass computes D[row][o] = sum_k X[row][k] op(B)[o][k] for every tile of
 // 128 rows, N = dim rounded up to 16, 3xTF32 (hi*hi + hi*lo + lo*hi, FP32
 // accumulation): the tables are split into TF32 parts once per theta, the
@@ -30,6 +30,12 @@
 //              staging tile laid out as the output box (double-buffered), and
 //              one TMA tensor store per 32 columns (the TMA writes full lines
 //              and leaves out what lies outside the tensor).
+// A last chunk of at most 16 columns is split and multiplied only that far, and a
+// table of an odd number of 16s stores only its columns.  64 x 64 x 16 with 256
+// samples (67 MB in, 67 MB out a pass): spatial passes over j 36 us, over i 36 (about 280
+// with tiles of 128 slabs along t), temporal ones 67 and 64 (82 and 71 with whole
+// chunks).  Longer rings, two groups of converter and epilogue warps, or op(B) kept in
+// shared memory change none of them by more than 2 us.
 // Every wait is bounded: after the limit the CTA raises bit 1 of *err, stops
 // issuing work, waits (bounded) for its loads and MMAs in flight, frees its
 // tensor memory and returns.
@@ -222,8 +228,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_kron_tc(const __grid_constant__ 
           tc_fence_after();
           const uint32_t st = smem_u32(base + s * SB);
           const uint32_t a_hi = st, a_lo = st + ATILE, b_hi = st + 2 * ATILE, b_lo = b_hi + BT;
-#pragma unroll
-          for (int j = 0; j < BK / 8; ++j) {
+          // steps past the contracted axis would add zeros
+          const int steps = min(BK, p.K - kc * BK + 7) / 8;
+          for (int j = 0; j < steps; ++j) {
             const uint32_t off = j * 32;
             mma_tf32_n(d, smem_desc(a_hi + off), smem_desc(b_hi + off), idesc, (kc | j) != 0);
             mma_tf32_n(d, smem_desc(a_hi + off), smem_desc(b_lo + off), idesc, 1u);
@@ -254,8 +261,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_kron_tc(const __grid_constant__ 
         }
         float4 *raw = reinterpret_cast<float4 *>(base + s * SB);
         float4 *lo = reinterpret_cast<float4 *>(base + s * SB + ATILE);
-#pragma unroll 4
-        for (int e = ct; e < ATILE / 16; e += 128) {
+        auto split = [&](int e) {
           const float4 v = raw[e];
           float4 h;
           h.x = tf32_rn(v.x);
@@ -264,6 +270,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_kron_tc(const __grid_constant__ 
           h.w = tf32_rn(v.w);
           raw[e] = h;
           lo[e] = make_float4(tf32_rn(v.x - h.x), tf32_rn(v.y - h.y), tf32_rn(v.z - h.z), tf32_rn(v.w - h.w));
+        };
+        if (p.K - kc * BK > BK / 2) {
+#pragma unroll 4
+          for (int e = ct; e < ATILE / 16; e += 128) split(e);
+        } else {
+          // the lower half of the columns only: 16-byte pieces c ^ (row % 8), c < 4, of
+          // rows r and r + 4 in eight lanes, which fall on different banks
+#pragma unroll
+          for (int e = ct; e < ATILE / 32; e += 128) {
+            const int c = e & 3, row = (e >> 5) * 8 + ((e >> 3) & 3) + (e & 4);
+            split(row * 8 + (c ^ (row & 7)));
+          }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         conv_sync();
@@ -310,16 +328,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_kron_tc(const __grid_constant__ 
         // the store that last used this staging tile has read it
         if (ec >= 2 && et == 0) bulk_wait_read<1>();
         epi_sync();
+        // the last 16 columns of a table with an odd number of 16s are not there
+        const bool wide = oc + OCH <= p.np;
         if (p.smode == 1) {
 #pragma unroll
           for (int jj = 0; jj < 32; ++jj) {
+            if (jj == 16 && !wide) break;
             // a preconditioner's scaling: the fast divide (a few ulp) suffices
             const float den = fmaf(__shfl_sync(0xffffffffu, tmu, jj), s2sq, p.omega);
             yt[yrow + jj * ycol] = __fdividef(__uint_as_float(v[jj]), den);
           }
         } else {
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj) yt[yrow + jj * ycol] = __uint_as_float(v[jj]) * rs;
+          for (int jj = 0; jj < 32; ++jj) {
+            if (jj == 16 && !wide) break;
+            yt[yrow + jj * ycol] = __uint_as_float(v[jj]) * rs;
+          }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         epi_sync();
@@ -373,10 +397,31 @@ bool g_attr_ok = false;
 enum Axis { AS = 0, AT = 1, AI = 2, AJ = 3 };
 struct PassSpec {
   int in[4], out[4];    // layouts, slowest axis first; in[3] is contracted
-  int box[4];           // tile rows per axis (product 128), indexed by axis
+  int fill[3];          // axes that fill a tile's 128 rows, in this order (the output's contiguous axis first)
   int table;            // KronOperator::split index of op(B)
   int scale;            // 0 none, 1 spectral, 2 dh_i dh_j
 };
+
+// Rows of a tile along each axis (product 128).  The first axis, which the output
+// has contiguous, takes a power of two of 16 .. 128 (64 to 512 bytes a line; a
+// shorter axis all of it) that pads it least, the larger one where several do;
+// the others then take the largest powers of two that divide them.
+void tile_box(const int *fill, const int64_t *sz, int *box) {
+  for (int a = 0; a < 4; ++a) box[a] = 1;
+  auto padded = [](int64_t n, int b) { return (n + b - 1) / b * b; };
+  const int64_t n0 = sz[fill[0]];
+  int b0 = MR;
+  for (int b = MR / 2; b >= 4 && (b >= 16 || 2 * b > n0); b /= 2)
+    if (padded(n0, b) < padded(n0, b0)) b0 = b;
+  box[fill[0]] = b0;
+  int left = MR / b0;
+  for (int f = 1; f < 3 && left > 1; ++f)
+    while (left > 1 && sz[fill[f]] % (2 * box[fill[f]]) == 0) {
+      box[fill[f]] *= 2;
+      left /= 2;
+    }
+  box[fill[1]] *= left;
+}
 
 }  // namespace ktc
 
@@ -400,14 +445,14 @@ bool launch_kron_apply_tc(cudaStream_t s, const KronOperator &op, const float *r
       acc *= sz[lay[a]];
     }
   };
-  // the chain of the header, P1 .. P6; box[] is indexed by axis (s, t, i, j)
+  // the chain of the header, P1 .. P6
   static const PassSpec chain[6] = {
-      {{AS, AT, AI, AJ}, {AS, AT, AJ, AI}, {1, 4, 32, 1}, 1, 0},
-      {{AS, AT, AJ, AI}, {AS, AJ, AI, AT}, {1, 128, 1, 1}, 1, 0},
-      {{AS, AJ, AI, AT}, {AS, AT, AJ, AI}, {1, 1, 32, 4}, 3, 1},
-      {{AS, AT, AJ, AI}, {AS, AT, AI, AJ}, {1, 4, 1, 32}, 0, 0},
-      {{AS, AT, AI, AJ}, {AS, AI, AJ, AT}, {1, 128, 1, 1}, 0, 0},
-      {{AS, AI, AJ, AT}, {AT, AI, AJ, AS}, {128, 1, 1, 1}, 2, 2},
+      {{AS, AT, AI, AJ}, {AS, AT, AJ, AI}, {AI, AT, AS}, 1, 0},
+      {{AS, AT, AJ, AI}, {AS, AJ, AI, AT}, {AT, AS, AJ}, 1, 0},
+      {{AS, AJ, AI, AT}, {AS, AT, AJ, AI}, {AI, AJ, AS}, 3, 1},
+      {{AS, AT, AJ, AI}, {AS, AT, AI, AJ}, {AJ, AT, AS}, 0, 0},
+      {{AS, AT, AI, AJ}, {AS, AI, AJ, AT}, {AT, AS, AI}, 0, 0},
+      {{AS, AI, AJ, AT}, {AT, AI, AJ, AS}, {AS, AJ, AI}, 2, 2},
   };
   Params ps[6];
   for (int k = 0; k < 6; ++k) {
@@ -415,6 +460,8 @@ bool launch_kron_apply_tc(cudaStream_t s, const KronOperator &op, const float *r
     Params &p = ps[k];
     memset(&p, 0, sizeof(p));
     int64_t sin[4], sout[4];
+    int tbox[4];
+    tile_box(sp.fill, sz, tbox);
     strides(sp.in, sin);
     strides(sp.out, sout);
     // tensor dims innermost first: d0 = contracted axis, d1 = in[2], d2 = in[1], d3 = in[0]
@@ -426,7 +473,7 @@ bool launch_kron_apply_tc(cudaStream_t s, const KronOperator &op, const float *r
     for (int a = 0; a < 4; ++a) {
       dims[a] = (uint64_t)sz[dax[a]];
       p.size[a] = (int)sz[dax[a]];
-      box[a] = a == 0 ? (uint32_t)BK : (uint32_t)sp.box[dax[a]];
+      box[a] = a == 0 ? (uint32_t)BK : (uint32_t)tbox[dax[a]];
       if (a > 0) {
         bst[a - 1] = (uint64_t)sin[dax[a]] * sizeof(float);
         p.box[a] = (int)box[a];
