@@ -174,7 +174,7 @@ struct qsel_ctx {
     double *vec[3] = {nullptr, nullptr, nullptr};   // v_{j-1}, v_j, w (rotated)
     double *u = nullptr, *q = nullptr, *xt = nullptr, *linv = nullptr;
     double *alpha = nullptr, *beta = nullptr, *coef = nullptr, *eta = nullptr, *zero = nullptr;
-    double *partial = nullptr, *dwork = nullptr, *U = nullptr;
+    double *partial = nullptr, *U = nullptr;
     bool ready = false, ran = false;
   } lz;
   double *d_partials = nullptr, *d_diag_scratch = nullptr;
@@ -1395,7 +1395,6 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
     TRY(c->alloc(&c->lz.eta, (size_t)c->ld));
     TRY(c->alloc(&c->lz.zero, (size_t)c->ld));
     TRY(c->alloc(&c->lz.partial, (size_t)lz_grid(c->n) * c->ld));
-    TRY(c->alloc(&c->lz.dwork, (size_t)2 * m * c->ld));
     TRY(c->alloc(&c->lz.U, (size_t)m * m * c->ld));
     QSEL_CUDA_TRY(cudaMemset(c->lz.zero, 0, (size_t)c->ld * sizeof(double)));
     c->lz.ready = true;
@@ -1452,7 +1451,7 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
       w = t;
     }
     if (pass == 0)
-      launch_lz_quadrature(s, la, c->lz.alpha, c->lz.beta, c->lz.eta, c->lz.dwork, c->lz.U, c->lz.coef, c->d_err);
+      launch_lz_quadrature(s, la, c->lz.alpha, c->lz.beta, c->lz.eta, c->lz.U, c->lz.coef, c->d_err);
   }
   // rewind the preconditioner: x = L^-T x~
   launch_oz_block_apply(s, c->lz.linv, b, true, c->n, c->ld, c->lz.xt, c->d_X, nullptr, nullptr, c->d_err);

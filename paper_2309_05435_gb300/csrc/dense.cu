@@ -16,6 +16,8 @@
 // (n_pad = n_s rounded up to 64, identity on the padded diagonal).
 #include <atomic>
 #include <mutex>
+#include <cooperative_groups.h>
+
 #include "qsel.h"
 #include "kernels.cuh"
 #include "sweep.cuh"
@@ -1156,10 +1158,13 @@ template void launch_schur_assemble<float>(cudaStream_t, const SchurBatch<float>
 
 // ---------------------------------------------------------------------------
 // diag(S) and the pattern inner products <M_j, S> with the entry's spatial
-// derivative blocks M_j (j < n_sums) in double (one block per entry, fixed
-// reduction order).  With D0 set, the diagonal is
-// instead diag(D0) + diag(D0 V) accumulated in double over column chunks
-// (k_diag64), D0 symmetric so that D0[i, l] = D0[l, i] reads coalesce.
+// derivative blocks M_j (j < n_sums) in double, in a fixed order: a cluster of
+// kExtractCtas blocks per entry, whose sums meet in the first one.  Each row's
+// entries lie in lines of their own, so the time is the loads' latency: eight of a
+// row in flight, and a row per thread up to 4096 of them (one block per entry,
+// an entry at a time: 52 us at 2304 rows in single precision, 24 at 1024 in double;
+// 14 and 19 us, the latter beside a sampler).  With D0 set, the diagonal is instead
+// diag(D0) + diag(D0 V) accumulated in double over column chunks (k_diag64), D0 symmetric so that D0[i, l] = D0[l, i] reads coalesce.
 // ---------------------------------------------------------------------------
 constexpr int kDiagChunks = 16;
 
@@ -1175,18 +1180,26 @@ __global__ void __launch_bounds__(256) k_diag64(ExtractBatch<T> bt, int n_s, int
   partial[((int64_t)blockIdx.z * kDiagChunks + blockIdx.y) * n_pad + i] = acc;
 }
 
+constexpr int kExtractCtas = 8, kExtractThreads = 512;
+
 template <typename T>
-__global__ void __launch_bounds__(1024) k_extract(ExtractBatch<T> bt, SellPattern pat, int n_sums, int n_s, int n_pad,
-                                                  const double *__restrict__ diag_partial) {
-  __shared__ double red[kMaxTheta][32];
-  const ExtractEntry<T> e = bt.e[blockIdx.x];
+__global__ void __cluster_dims__(kExtractCtas, 1, 1) __launch_bounds__(kExtractThreads)
+    k_extract(ExtractBatch<T> bt, SellPattern pat, int n_sums, int n_s, int n_pad,
+              const double *__restrict__ diag_partial) {
+  __shared__ double red[kMaxTheta][kExtractThreads / 32];
+  __shared__ double mine[kMaxTheta];
+  const int entry = blockIdx.x / kExtractCtas, rank = blockIdx.x % kExtractCtas;
+  const ExtractEntry<T> e = bt.e[entry];
   double acc[kMaxTheta] = {0.0, 0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < n_s; i += blockDim.x) {
+  // a block takes a run of whole slices, so that short ones spread over the blocks
+  const int run = ((n_s + kExtractCtas - 1) / kExtractCtas + 31) / 32 * 32;
+  const int end = min(n_s, (rank + 1) * run);
+  for (int i = rank * run + threadIdx.x; i < end; i += kExtractThreads) {
     const T *Si = e.S + (int64_t)i * n_pad;
     if (e.diag_out) {
       if (e.D0) {
         double d = (double)e.D0[(int64_t)i * n_pad + i];
-        for (int c = 0; c < kDiagChunks; ++c) d += diag_partial[((int64_t)blockIdx.x * kDiagChunks + c) * n_pad + i];
+        for (int c = 0; c < kDiagChunks; ++c) d += diag_partial[((int64_t)entry * kDiagChunks + c) * n_pad + i];
         e.diag_out[i] = d;
       } else {
         e.diag_out[i] = (double)Si[i];
@@ -1196,16 +1209,20 @@ __global__ void __launch_bounds__(1024) k_extract(ExtractBatch<T> bt, SellPatter
       const int sl = i >> 5, li = i & 31;
       const int w = pat.slice_width[sl];
       const int base = pat.slice_ptr[sl] + li;
-      for (int s = 0; s < w; ++s) {
-        const int idx = base + s * kSlice;
-        const double sv = (double)Si[pat.col[idx]];
+      constexpr int D = 8;
+      for (int s0 = 0; s0 < w; s0 += D) {
+        T sv[D];
 #pragma unroll
-        for (int j = 0; j < kMaxTheta; ++j)
-          if (j < n_sums) acc[j] = fma(e.sv[j][idx], sv, acc[j]);
+        for (int u = 0; u < D; ++u) sv[u] = s0 + u < w ? Si[pat.col[base + (s0 + u) * kSlice]] : T(0);
+#pragma unroll
+        for (int u = 0; u < D; ++u)
+#pragma unroll
+          for (int j = 0; j < kMaxTheta; ++j)
+            if (j < n_sums && s0 + u < w) acc[j] = fma(e.sv[j][base + (s0 + u) * kSlice], (double)sv[u], acc[j]);
       }
     }
   }
-  if (!e.sums) return;
+  if (!e.sums) return;   // the whole cluster
 #pragma unroll
   for (int j = 0; j < kMaxTheta; ++j) {
     for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_down_sync(0xffffffffu, acc[j], o);
@@ -1214,9 +1231,17 @@ __global__ void __launch_bounds__(1024) k_extract(ExtractBatch<T> bt, SellPatter
   __syncthreads();
   if (threadIdx.x < n_sums) {
     double a = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += red[threadIdx.x][w];
+    for (int w = 0; w < kExtractThreads / 32; ++w) a += red[threadIdx.x][w];
+    mine[threadIdx.x] = a;
+  }
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  cl.sync();
+  if (rank == 0 && threadIdx.x < n_sums) {
+    double a = 0.0;
+    for (int q = 0; q < kExtractCtas; ++q) a += *cl.map_shared_rank(&mine[threadIdx.x], q);
     e.sums[threadIdx.x] = a;
   }
+  cl.sync();   // the others' shared memory is read until here
 }
 
 // Scratch for the FP64 diagonal partials (per device, grown on demand by the
@@ -1239,7 +1264,7 @@ void launch_extract(cudaStream_t s, const ExtractBatch<T> &b, const SellPattern 
   ++g_launch_count;
   {
     ProfScope ps_(s, PROF_EXTRACT);
-    k_extract<T><<<b.count, 1024, 0, s>>>(b, pat, n_sums, n_s, n_pad, diag_scratch);
+    k_extract<T><<<b.count * kExtractCtas, kExtractThreads, 0, s>>>(b, pat, n_sums, n_s, n_pad, diag_scratch);
   }
 }
 template void launch_extract<double>(cudaStream_t, const ExtractBatch<double> &, const SellPattern &, int, int, int,

@@ -586,7 +586,7 @@ void launch_lz_reduce(cudaStream_t s, const LanczosArgs &a, const double *partia
                       double *store);
 void launch_lz_scale(cudaStream_t s, const LanczosArgs &a, double *w, const double *scal);
 void launch_lz_quadrature(cudaStream_t s, const LanczosArgs &a, const double *alpha, const double *beta,
-                          const double *eta, double *dwork, double *U, double *coef, int32_t *err_flag);
+                          const double *eta, double *U, double *coef, int32_t *err_flag);
 
 // ---------------------------------------------------------------- mlp.cu
 void launch_cv_features(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t,

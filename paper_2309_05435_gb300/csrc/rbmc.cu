@@ -108,30 +108,46 @@ template void launch_correction_terms<float>(cudaStream_t, const CorrBatch<float
 //   <dA_j(t), Sigma_tt> - <dB_j(t), Y_t> - <dB_j(t-1), Y_{t-1}>
 // (Sigma_{t,t+1} = -Y_t^T, Sigma_{t,t-1} = -Y_{t-1}, the blocks symmetric;
 // sums hold the pattern inner products without the scales) plus the
-// correction partials.  One thread, fixed order.
-__global__ void k_trace_combine(const TraceSlab *__restrict__ slabs, int n_slabs,
-                                const double *__restrict__ sums, const double *__restrict__ partials,
-                                int n_partials, DerivModels dm, double *out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// correction partials.  One block, fixed order: a thread takes every 256th slab and
+// every 256th partial, then a tree (one thread alone took 143 us for 12 slabs and
+// 475 us with four parts' partials; 6 and 7 us).
+__global__ void __launch_bounds__(256) k_trace_combine(const TraceSlab *__restrict__ slabs, int n_slabs,
+                                                       const double *__restrict__ sums,
+                                                       const double *__restrict__ partials, int n_partials,
+                                                       DerivModels dm, double *out) {
+  __shared__ double red[kMaxTheta][256];
   double acc[kMaxTheta] = {0.0, 0.0, 0.0, 0.0};
-  for (int q = 0; q < n_slabs; ++q) {
+  for (int q = threadIdx.x; q < n_slabs; q += 256) {
     const TraceSlab sl = slabs[q];
     const int t = sl.t;
-    for (int j = 0; j < dm.n; ++j) {
+#pragma unroll
+    for (int j = 0; j < kMaxTheta; ++j) {
+      if (j >= dm.n) break;
       acc[j] += dm.diag[j].scale(t) * sums[kMaxTheta * sl.sd + j];
       if (sl.sy >= 0) acc[j] -= dm.off[j].scale(t) * sums[kMaxTheta * sl.sy + j];
       if (sl.sym >= 0) acc[j] -= dm.off[j].scale(t - 1) * sums[kMaxTheta * sl.sym + j];
     }
   }
-  for (int q = 0; q < n_partials; ++q)
-    for (int j = 0; j < dm.n; ++j) acc[j] += partials[kMaxTheta * q + j];
-  for (int j = 0; j < dm.n; ++j) out[j] = acc[j];
+  for (int q = threadIdx.x; q < n_partials; q += 256)
+#pragma unroll
+    for (int j = 0; j < kMaxTheta; ++j)
+      if (j < dm.n) acc[j] += partials[kMaxTheta * q + j];
+#pragma unroll
+  for (int j = 0; j < kMaxTheta; ++j) red[j][threadIdx.x] = acc[j];
+  for (int o = 128; o > 0; o >>= 1) {
+    __syncthreads();
+    if (threadIdx.x < o)
+#pragma unroll
+      for (int j = 0; j < kMaxTheta; ++j) red[j][threadIdx.x] += red[j][threadIdx.x + o];
+  }
+  if (threadIdx.x == 0)
+    for (int j = 0; j < dm.n; ++j) out[j] = red[j][0];
 }
 
 void launch_trace_combine(cudaStream_t s, const TraceSlab *slabs_dev, int n_slabs, const double *sums,
                           const double *partials, int n_partials, const DerivModels &dm, double *out) {
   ++g_launch_count;
-  k_trace_combine<<<1, 32, 0, s>>>(slabs_dev, n_slabs, sums, partials, n_partials, dm, out);
+  k_trace_combine<<<1, 256, 0, s>>>(slabs_dev, n_slabs, sums, partials, n_partials, dm, out);
 }
 
 template <typename T>

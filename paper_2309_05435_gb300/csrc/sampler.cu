@@ -304,8 +304,10 @@ __global__ void __launch_bounds__(256) k_bt_spmm(BtSpmmArgs<T> a) {
         x0 = xv.x;
         x1 = xv.y;
       }
-      ax[v] = fma(ow, x0, ax[v]);
-      ay[v] = fma(ow, x1, ay[v]);
+      if (ow != T(0)) {   // uniform in the warp
+        ax[v] = fma(ow, x0, ax[v]);
+        ay[v] = fma(ow, x1, ay[v]);
+      }
       store2(yr + 64 * v, ax[v], ay[v]);
       if (dot) {
         red[warp][coff + 64 * v] = fma(x0, ax[v], red[warp][coff + 64 * v]);
@@ -630,27 +632,60 @@ template void launch_pcg_update<double>(cudaStream_t, const PcgVec<double> &, co
 template void launch_pcg_update<float>(cudaStream_t, const PcgVec<float> &, const float *, int,
                                        const KronOperator *);
 
-// Column sums of per-CTA partial rows: 8 row groups x 32 columns per block,
-// fixed order within each group and across groups.
-__device__ __forceinline__ double column_sum(const double *__restrict__ part, int n_rows, int ld, int c, int rg,
-                                             double (*sh)[33]) {
-  double acc = 0.0;
-  for (int g = rg; g < n_rows; g += 8) acc += part[(int64_t)g * ld + c];
-  sh[rg][threadIdx.x & 31] = acc;
-  __syncthreads();
-  double tot = 0.0;
+// Column sums of Q arrays of per-CTA partial rows, all in one pass: 32 row groups x 4
+// columns (a sector) per block of four warps, fixed order.  Bound by the groups'
+// chains of binary64 additions (a warp's addition holds its SM quarter for about 70
+// cycles, so a block has one warp per quarter and there are as many blocks as columns
+// allow); eight rows are loaded at a time.  The warp of a column then adds its groups
+// as a tree; lane 0 has the sums.  Beside the dense part, 1216 rows x
+// 128 columns: 18 -> 12 us; two arrays of 512 rows: 13 -> 7 us (8 groups x 32 columns, a
+// load waited for before each addition; the 8 x 8 columns of two warps, 18 and 13).
+constexpr int kSumCols = 4, kSumGroups = 32, kSumThreads = kSumCols * kSumGroups;
+
+template <int Q>
+__device__ __forceinline__ void column_sums(const double *const (&part)[Q], int n_rows, int ld,
+                                            double (*sh)[kSumGroups][kSumCols + 1], double (&tot)[Q]) {
+  constexpr int D = 8;
+  const int col = threadIdx.x % kSumCols, rg = threadIdx.x / kSumCols;
+  const int c = blockIdx.x * kSumCols + col;
+  double acc[Q];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) tot += sh[q][threadIdx.x & 31];
-  return tot;
+  for (int q = 0; q < Q; ++q) acc[q] = 0.0;
+  for (int g = rg; g < n_rows; g += D * kSumGroups) {
+    double v[Q][D];
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+      for (int u = 0; u < D; ++u) {
+        const int r = g + u * kSumGroups;
+        v[q][u] = r < n_rows ? part[q][(int64_t)r * ld + c] : 0.0;
+      }
+#pragma unroll
+    for (int u = 0; u < D; ++u)
+      if (g + u * kSumGroups < n_rows) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[q] += v[q][u];
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) sh[q][rg][col] = acc[q];
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    tot[q] = sh[q][threadIdx.x & 31][threadIdx.x >> 5];
+    for (int o = 16; o > 0; o >>= 1) tot[q] += __shfl_down_sync(0xffffffffu, tot[q], o);
+  }
 }
 
 // alpha_c = rho_c / <p_c, q_c> for active columns, 0 otherwise.
 template <typename T>
-__global__ void __launch_bounds__(256) k_pcg_reduce_alpha(PcgVec<T> v) {
-  __shared__ double sh[8][33];
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31), rg = threadIdx.x >> 5;
-  const double pq = column_sum(v.partial_a, v.n_blocks_dot, v.ld, c, rg, sh);
-  if (rg == 0) v.alpha[c] = (v.active[c] && pq != 0.0) ? v.rho[c] / pq : 0.0;
+__global__ void __launch_bounds__(kSumThreads) k_pcg_reduce_alpha(PcgVec<T> v) {
+  __shared__ double sh[1][kSumGroups][kSumCols + 1];
+  const int c = blockIdx.x * kSumCols + (threadIdx.x >> 5);
+  const double *const part[1] = {v.partial_a};
+  double pq[1];
+  column_sums<1>(part, v.n_blocks_dot, v.ld, sh, pq);
+  if ((threadIdx.x & 31) == 0) v.alpha[c] = (v.active[c] && pq[0] != 0.0) ? v.rho[c] / pq[0] : 0.0;
 }
 
 template <typename T>
@@ -658,7 +693,7 @@ void launch_pcg_reduce_alpha(cudaStream_t s, const PcgVec<T> &v) {
   ++g_launch_count;
   {
     ProfScope ps_(s, PROF_PCGVEC);
-    k_pcg_reduce_alpha<T><<<v.ld / 32, 256, 0, s>>>(v);
+    k_pcg_reduce_alpha<T><<<v.ld / kSumCols, kSumThreads, 0, s>>>(v);
   }
 }
 template void launch_pcg_reduce_alpha<double>(cudaStream_t, const PcgVec<double> &);
@@ -667,13 +702,14 @@ template void launch_pcg_reduce_alpha<float>(cudaStream_t, const PcgVec<float> &
 // <r, z>, <r, r> -> beta, rho, convergence flags; active count and maximum
 // relative residual by integer atomics (the update kernel zeroed them).
 template <typename T>
-__global__ void __launch_bounds__(256) k_pcg_reduce_beta(PcgVec<T> v, double tol2, int init) {
-  __shared__ double sh[8][33];
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31), rg = threadIdx.x >> 5;
-  const double rz = column_sum(v.partial_a, v.n_tiles, v.ld, c, rg, sh);
-  __syncthreads();
-  const double rr = column_sum(v.partial_b, v.n_tiles, v.ld, c, rg, sh);
-  if (rg != 0) return;
+__global__ void __launch_bounds__(kSumThreads) k_pcg_reduce_beta(PcgVec<T> v, double tol2, int init) {
+  __shared__ double sh[2][kSumGroups][kSumCols + 1];
+  const int c = blockIdx.x * kSumCols + (threadIdx.x >> 5);
+  const double *const part[2] = {v.partial_a, v.partial_b};
+  double sums[2];
+  column_sums<2>(part, v.n_tiles, v.ld, sh, sums);
+  const double rz = sums[0], rr = sums[1];
+  if ((threadIdx.x & 31) != 0) return;
   if (init) {
     v.bb[c] = rr;
     v.rho[c] = rz;
@@ -689,15 +725,9 @@ __global__ void __launch_bounds__(256) k_pcg_reduce_beta(PcgVec<T> v, double tol
   v.rr[c] = rr;
   int act = v.active[c];
   double rel = v.bb[c] > 0.0 ? sqrt(rr / v.bb[c]) : 0.0;
-  for (int o = 16; o > 0; o >>= 1) {
-    act += __shfl_down_sync(0xffffffffu, act, o);
-    rel = fmax(rel, __shfl_down_sync(0xffffffffu, rel, o));
-  }
-  if (threadIdx.x == 0) {
-    if (act) atomicAdd(v.counters, act);
-    // non-negative doubles order like their bit patterns
-    atomicMax(reinterpret_cast<unsigned long long *>(v.max_rel), (unsigned long long)__double_as_longlong(rel));
-  }
+  if (act) atomicAdd(v.counters, act);
+  // non-negative doubles order like their bit patterns
+  atomicMax(reinterpret_cast<unsigned long long *>(v.max_rel), (unsigned long long)__double_as_longlong(rel));
 }
 
 template <typename T>
@@ -705,7 +735,7 @@ void launch_pcg_reduce_beta(cudaStream_t s, const PcgVec<T> &v, double tol, int 
   ++g_launch_count;
   {
     ProfScope ps_(s, PROF_PCGVEC);
-    k_pcg_reduce_beta<T><<<v.ld / 32, 256, 0, s>>>(v, tol * tol, init);
+    k_pcg_reduce_beta<T><<<v.ld / kSumCols, kSumThreads, 0, s>>>(v, tol * tol, init);
   }
 }
 template void launch_pcg_reduce_beta<double>(cudaStream_t, const PcgVec<double> &, double, int);
@@ -804,7 +834,22 @@ __global__ void k_residual_check(const double *__restrict__ prr, const double *_
   double rel = 0.0;
   if (c < ld) {
     double rr = 0.0, bb = 0.0;
-    for (int g = 0; g < n_parts; ++g) {
+    // eight rows' loads in flight, added in order
+    int g = 0;
+    for (; g + 8 <= n_parts; g += 8) {
+      double vr[8], vb[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        vr[u] = prr[(int64_t)(g + u) * ld + c];
+        vb[u] = pbb[(int64_t)(g + u) * ld + c];
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        rr += vr[u];
+        bb += vb[u];
+      }
+    }
+    for (; g < n_parts; ++g) {
       rr += prr[(int64_t)g * ld + c];
       bb += pbb[(int64_t)g * ld + c];
     }
