@@ -408,10 +408,11 @@ constexpr int PARTS = PANEL_THREADS / BM;      // threads per row of the left op
 constexpr int PART = 64 / PARTS;               // entries of a thread
 
 // Eight digits of eight neighbouring values: 16 bytes per digit plane to shared
-// (stride s_plane) and / or global memory (stride g_plane).
+// (stride s_plane; with s_twin a second time, s_twin bytes further) and / or global
+// memory (stride g_plane).
 template <bool SMEM>
 __device__ __forceinline__ void store_digits8(uint8_t *sdst, uint32_t s_plane, uint16_t *gdst, int64_t g_plane,
-                                              const double *x, int32_t E) {
+                                              const double *x, int32_t E, uint32_t s_twin = 0) {
   uint2 y[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) y[c] = digit_bytes(fixed62(x[c], E));
@@ -420,6 +421,7 @@ __device__ __forceinline__ void store_digits8(uint8_t *sdst, uint32_t s_plane, u
     const uint4 w = make_uint4(digit_pair<I>(y[0], y[1]), digit_pair<I>(y[2], y[3]),                      \
                                digit_pair<I>(y[4], y[5]), digit_pair<I>(y[6], y[7]));                     \
     if (SMEM) *reinterpret_cast<uint4 *>(sdst + (I) * s_plane) = w;                                       \
+    if (SMEM && s_twin) *reinterpret_cast<uint4 *>(sdst + s_twin + (I) * s_plane) = w;                    \
     if (gdst) *reinterpret_cast<uint4 *>(gdst + (I) * g_plane) = w;                                       \
   }
   QSEL_OZ_STORE(0)
@@ -595,6 +597,9 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
 // with 256 the operations' latencies showed (43.6 against 62 us for two tiles of
 // 128 columns an SM).  Measured, n = 32768, 128 columns: 545 us on the binary64
 // pipe (k_pcg_precond) -> 82 us; n = 9216, 64 columns, without sums: 52 -> 17 us.
+// A chunk of at most 64 columns fills both halves of the M rows with them: two threads
+// share a column, each forms the digits of half the rows (for both halves) and rounds
+// half the results: with sums and n = 2048, 20.8 -> about 14 us.
 // ---------------------------------------------------------------------------
 struct BlockParams {
   const double *B, *x;
@@ -651,28 +656,31 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __gri
     });
     const int rows = min(PART, max(0, p.n - r0 - PART * part));   // this thread's rows
     for (int c0 = 0; c0 < p.ld && go; c0 += BM) {
-      const int col = c0 + cl;
+      const bool twin = p.ld - c0 <= BM / 2;
+      const int col = c0 + (twin ? cl & (BM / 2 - 1) : cl);
       const bool valid = col < p.ld;
+      const int e_begin = twin ? cl / (BM / 2) : 0, e_end = twin ? e_begin + 1 : PART / 8;   // its eights of rows
       const int64_t at = (int64_t)(r0 + PART * part) * p.ld + col;
       const double *xc = p.x + at;
       double *zc = p.z + at;
       int f = 0;
       if (valid) {
-#pragma unroll 16
-        for (int j = 0; j < rows; ++j) f = max(f, exp_field(xc[(int64_t)j * p.ld]));
+#pragma unroll 8
+        for (int j = 8 * e_begin; j < min(rows, 8 * e_end); ++j) f = max(f, exp_field(xc[(int64_t)j * p.ld]));
       }
       red[part][cl] = f;
       __syncthreads();
-      const int32_t Ea = part_exponent(red, cl);
+      const int32_t Ea = max(part_exponent(red, cl), twin ? part_exponent(red, cl ^ (BM / 2)) : INT32_MIN);
       // eight values at a time in loops, x re-read (from L1): unrolled over the
       // tile, the kernel waited on instruction fetches for most of its time
 #pragma unroll 1
-      for (int c = 0; c < PART / 8; ++c) {
+      for (int c = e_begin; c < e_end; ++c) {
         double x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) x[u] = valid && 8 * c + u < rows ? xc[(int64_t)(8 * c + u) * p.ld] : 0.0;
-        store_digits8<true>(sa + cl * P_ROWB + (((PART / 8 * part + c) ^ (cl & 7)) << 4), PA_TILE, nullptr, 0, x,
-                            finite_exponent(Ea));
+        const int row = twin ? cl & (BM / 2 - 1) : cl;
+        store_digits8<true>(sa + row * P_ROWB + (((PART / 8 * part + c) ^ (row & 7)) << 4), PA_TILE, nullptr, 0, x,
+                            finite_exponent(Ea), twin ? BM / 2 * P_ROWB : 0);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       tc_fence_before();
@@ -693,7 +701,7 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __gri
       const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(PART * part);
       double s0 = 0.0, s1 = 0.0;
 #pragma unroll 1
-      for (int cb = 0; cb < PART / 8; ++cb) {
+      for (int cb = e_begin; cb < e_end; ++cb) {
         int64_t hi[8], lo[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
@@ -721,10 +729,13 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __gri
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
-      if (DOTS && part < 2 && valid) {
+      if (DOTS && part < 2 && valid && !(twin && cl >= BM / 2)) {
         double t = 0.0;
 #pragma unroll
         for (int h = 0; h < PARTS; ++h) t += psum[(PARTS * part + h) * BM + cl];
+        if (twin)
+#pragma unroll
+          for (int h = 0; h < PARTS; ++h) t += psum[(PARTS * part + h) * BM + cl + BM / 2];
         acc[part * p.ld + col] += t;
       }
     }
