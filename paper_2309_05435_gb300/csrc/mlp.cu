@@ -464,11 +464,12 @@ __global__ void k_feature_stats(const float *__restrict__ X, int n, float *__res
 // ---------------------------------------------------------------------------
 constexpr int kFeatSlabs = 16;
 
-// (float)log(a).  binary64 arithmetic holds a warp's issue slot for about 70 cycles an
-// instruction here, so a positive normal a = 2^e (1 + f), 1 + f in [sqrt(1/2), sqrt(2)),
-// takes pairs of floats: 2 atanh(s) = 2 s (1 + s^2/3 + s^4/5 + ...), s = f / (2 + f),
-// plus e ln 2.  The tail from s^4/5 on is in single precision, an error below 2^-34 of
-// the result: the rounding to float is what is left.
+// (float)log(a), the same float.  binary64 arithmetic holds a warp's issue slot for
+// about 70 cycles an instruction here, so a positive normal a = 2^e (1 + f), 1 + f in
+// [sqrt(1/2), sqrt(2)), takes pairs of floats: 2 atanh(s) = 2 s (1 + s^2/3 + s^4/5 + ...),
+// s = f / (2 + f), plus e ln 2.  The tail from s^4/5 on is in single precision, an
+// error below 2^-34 of the result.  Where 2^-33 to either side would round to another
+// float (one value in about 250), binary64 decides.
 __device__ __forceinline__ float log_to_float(double a) {
   const long long bits = __double_as_longlong(a);
   if (bits < 0x0010000000000000ll || bits >= 0x7ff0000000000000ll) return (float)log(a);
@@ -496,7 +497,9 @@ __device__ __forceinline__ float log_to_float(double a) {
   const float ef = (float)e, eh = ef * l1, el = fmaf(ef, l1, -eh) + ef * l2;
   const float h = eh + 2.f * zh, back = h - eh;
   const float err = (eh - (h - back)) + (2.f * zh - back);
-  return h + (err + fmaf(2.f, zl, el));
+  const float low = err + fmaf(2.f, zl, el), slack = fabsf(h) * 0x1p-33f;
+  const float r = h + (low - slack);
+  return r == h + (low + slack) ? r : (float)log(a);
 }
 
 
