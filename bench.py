@@ -540,7 +540,7 @@ def roofline_of(st, w, hbm_peak, hbm_src, tf32_peak, tf32_src, exact=False):
                     "split once in HBM, TMA, double-buffered TMEM accumulators)",
             "sweep_update": "k_tc_update (persistent rank-256 sweep panel updates, tcgen05 3xTF32)",
             "spmm": "k_bt_spmm (block-tridiagonal sliced-ELL SpMM, PCG)",
-            "pivot": "k_bsweep_pivot (64x64 double-float pivot-tile inverses, 2x2 block sweep)",
+            "pivot": "k_sweep_chain (a panel's chain of 64x64 double-float pivot inverses and steps, four SMs a matrix)",
             "precond": "k_kron_transpose_in + k_kron_tc x6 (Kronecker preconditioner on tcgen05)"}
     cand = [i for i, nm in enumerate(classes) if nm in desc and cwork[i] > 0 and cms[i] > 0]
     dom = max(cand, key=lambda i: cms[i])

@@ -114,7 +114,9 @@ enum {
 
 /* Arithmetic of the pipeline. */
 enum {
-  QSEL_FP64 = 0,      /* every kernel computes in IEEE binary64                  */
+  QSEL_FP64 = 0,      /* IEEE binary64 operands and results; the dense products
+                         and block applies form exact digit products on the tensor
+                         cores and round to binary64 once                        */
   QSEL_MIXED = 1      /* binary32 solves and factorisations, extended-precision
                          pivot tiles (double-float or binary64, see
                          pivot_precision), binary64 refinement residuals and
