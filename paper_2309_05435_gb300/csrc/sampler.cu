@@ -257,6 +257,10 @@ __global__ void __launch_bounds__(256) k_bt_spmm(BtSpmmArgs<T> a) {
         }
       }
       const int cnt = min(32, w - s0);
+      // the entries with a coupling: the couplings may live on a much smaller pattern
+      // than the diagonal blocks (K_1 against K_3 of the diffusion model, 7 of 37
+      // entries), and a binary64 FMA costs more than the warp-uniform test
+      const uint32_t coupled = COMB ? 0u : __ballot_sync(0xffffffffu, my_fm != T(0) || my_fp != T(0));
 #pragma unroll 4
       for (int s = 0; s < cnt; ++s) {
         const int j = __shfl_sync(0xffffffffu, my_col, s);
@@ -273,13 +277,17 @@ __global__ void __launch_bounds__(256) k_bt_spmm(BtSpmmArgs<T> a) {
         }
         const T *xc = a.x + ((int64_t)t * a.n_s + j) * ld + coff;
         const T f0 = __shfl_sync(0xffffffffu, my_f0, s);
-        const T fm = __shfl_sync(0xffffffffu, my_fm, s);
-        const T fp = __shfl_sync(0xffffffffu, my_fp, s);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const auto x0 = load2(xc + 64 * v);
           ax[v] = fma(f0, x0.x, ax[v]);
           ay[v] = fma(f0, x0.y, ay[v]);
+        }
+        if (!((coupled >> s) & 1u)) continue;
+        const T fm = __shfl_sync(0xffffffffu, my_fm, s);
+        const T fp = __shfl_sync(0xffffffffu, my_fp, s);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
           if (has_m) {
             const auto xm = load2(xc - slab + 64 * v);
             ax[v] = fma(fm, xm.x, ax[v]);
