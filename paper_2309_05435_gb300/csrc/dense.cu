@@ -897,12 +897,23 @@ template void launch_sp_rowgather<double, float>(cudaStream_t, const SpBatch<dou
 // ---------------------------------------------------------------------------
 // Column gathers over the symmetric pattern, (B Q_s)[r, l] =
 // sum_{j in pat(l)} B[r, j] Q_s[l, j].  A block covers 256 columns and
-// kGatherRows rows; each thread keeps its column's pattern (j, Q_s[l, j]) in
+// 16 to 64 rows; each thread keeps its column's pattern (j, Q_s[l, j]) in
 // its own shared slots [s * 256 + t] (no sharing, no block barrier) and reuses
 // it for every row.  Shared memory: max_width * 256 * (4 + sizeof(T)) bytes.
 // ---------------------------------------------------------------------------
-constexpr int kGatherRows = 64;   // rows per block (a multiple of kGatherRowBlock)
 constexpr int kGatherRowBlock = 4; // rows per thread at a time: one pattern read, four FMAs
+
+// Rows per block: 64, halved (to 16 at least) while there are fewer than eight blocks
+// an SM.  Staging a column's pattern for fewer rows costs less than an uneven last
+// wave: two 1408-node blocks in single precision 57 -> 39 us a Schur assembly and
+// 37 -> 30 a column gather (264 -> 1056 blocks), two of 1600 nodes in double 212 -> 160
+// and 179 -> 139; at 4096 nodes 64 rows fill the chip.  Eight rows at a time instead of
+// four: 38 and 33, 157 and 141.
+static int gather_rows(int n_pad, int count) {
+  int rows = 64;
+  while (rows > 16 && (int64_t)((n_pad + 255) / 256) * (n_pad / rows) * count < 8 * (int64_t)device_sms()) rows /= 2;
+  return rows;
+}
 
 template <typename T>
 __device__ __forceinline__ int stage_col_pattern(const SellPattern &pat, const double *__restrict__ val, int l,
@@ -927,7 +938,8 @@ size_t col_pattern_smem(const SellPattern &pat) {
 // columns past n_s of Out are zero.  With B = D^-1 (symmetric) this is
 // (M D^-1)^T.
 template <typename T>
-__global__ void __launch_bounds__(256) k_sp_colgather(SpBatch<T, T> bt, SellPattern pat, int n_s, int n_pad) {
+__global__ void __launch_bounds__(256) k_sp_colgather(SpBatch<T, T> bt, SellPattern pat, int n_s, int n_pad,
+                                                      int rows) {
   extern __shared__ __align__(16) unsigned char cg_smem[];
   int *s_col = reinterpret_cast<int *>(cg_smem);
   T *s_val = reinterpret_cast<T *>(s_col + pat.max_width * 256);
@@ -937,7 +949,7 @@ __global__ void __launch_bounds__(256) k_sp_colgather(SpBatch<T, T> bt, SellPatt
   const int w = stage_col_pattern(pat, e.val, l, n_s, s_col, s_val);
   const T alpha = (T)(e.alpha * (e.alpha_ptr ? *e.alpha_ptr : 1.0));
   const bool add_c = e.C != nullptr && e.beta != 0.0;
-  const int r0 = blockIdx.y * kGatherRows, r1 = min(n_pad, r0 + kGatherRows);
+  const int r0 = blockIdx.y * rows, r1 = min(n_pad, r0 + rows);
   for (int r = r0; r < r1; r += kGatherRowBlock) {
     // kGatherRowBlock rows per pattern entry read (n_pad is a multiple of 64)
     T acc[kGatherRowBlock];
@@ -969,10 +981,11 @@ template <typename T>
 void launch_sp_colgather(cudaStream_t s, const SpBatch<T, T> &b, const SellPattern &pat, int n_s, int n_pad) {
   if (b.count <= 0) return;
   ++g_launch_count;
-  dim3 grid((n_pad + 255) / 256, (n_pad + kGatherRows - 1) / kGatherRows, b.count);
+  const int rows = gather_rows(n_pad, b.count);
+  dim3 grid((n_pad + 255) / 256, n_pad / rows, b.count);
   {
     ProfScope ps_(s, PROF_GATHER);
-    k_sp_colgather<T><<<grid, 256, col_pattern_smem<T>(pat), s>>>(b, pat, n_s, n_pad);
+    k_sp_colgather<T><<<grid, 256, col_pattern_smem<T>(pat), s>>>(b, pat, n_s, n_pad, rows);
   }
 }
 template void launch_sp_colgather<double>(cudaStream_t, const SpBatch<double, double> &, const SellPattern &, int,
@@ -1038,7 +1051,7 @@ __device__ __forceinline__ T schur_sum(const T *__restrict__ Wr, int w, const in
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_schur_assemble(SchurBatch<T> bt, SellPattern pat, double obs_w, int n_s,
-                                                        int n_pad) {
+                                                        int n_pad, int rows) {
   extern __shared__ __align__(16) unsigned char sa_smem[];
   int *s_col = reinterpret_cast<int *>(sa_smem);
   T *s_val = reinterpret_cast<T *>(s_col + pat.max_width * 256);
@@ -1048,7 +1061,7 @@ __global__ void __launch_bounds__(256) k_schur_assemble(SchurBatch<T> bt, SellPa
   const int w = stage_col_pattern(pat, e.W ? e.cval : e.dval, l, n_s, s_col, s_val);
   const double *__restrict__ dval = e.dval;
   const T neg_c = e.W ? (T)(-(e.c ? *e.c : 1.0)) : T(0);
-  const int r0 = blockIdx.y * kGatherRows, r1 = min(n_pad, r0 + kGatherRows);
+  const int r0 = blockIdx.y * rows, r1 = min(n_pad, r0 + rows);
   if (e.accumulate) {
     // a second Schur term on the spatial block (the middle slab of a
     // two-ended factorisation), combined in double like the pattern entries
@@ -1122,10 +1135,11 @@ void launch_schur_assemble(cudaStream_t s, const SchurBatch<T> &b, const SellPat
                            int n_pad) {
   if (b.count <= 0) return;
   ++g_launch_count;
-  dim3 grid((n_pad + 255) / 256, (n_pad + kGatherRows - 1) / kGatherRows, b.count);
+  const int rows = gather_rows(n_pad, b.count);
+  dim3 grid((n_pad + 255) / 256, n_pad / rows, b.count);
   {
     ProfScope ps_(s, PROF_SCHUR);
-    k_schur_assemble<T><<<grid, 256, col_pattern_smem<T>(pat), s>>>(b, pat, obs_w, n_s, n_pad);
+    k_schur_assemble<T><<<grid, 256, col_pattern_smem<T>(pat), s>>>(b, pat, obs_w, n_s, n_pad, rows);
   }
 }
 // Opt the pattern-staging kernels in to the shared memory that
