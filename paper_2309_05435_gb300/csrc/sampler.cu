@@ -259,7 +259,8 @@ __global__ void __launch_bounds__(256) k_bt_spmm(BtSpmmArgs<T> a) {
       const int cnt = min(32, w - s0);
       // the entries with a coupling: the couplings may live on a much smaller pattern
       // than the diagonal blocks (K_1 against K_3 of the diffusion model, 7 of 37
-      // entries), and a binary64 FMA costs more than the warp-uniform test
+      // entries), and a binary64 FMA costs more than the warp-uniform test: 86 -> 49 us
+      // for 9216 rows x 64 columns
       const uint32_t coupled = COMB ? 0u : __ballot_sync(0xffffffffu, my_fm != T(0) || my_fp != T(0));
 #pragma unroll 4
       for (int s = 0; s < cnt; ++s) {
