@@ -513,7 +513,6 @@ __global__ void __launch_bounds__(128) k_cv_features(SellPattern pat, BtModel m,
   const int w = pat.slice_width[sl];
   const int base = pat.slice_ptr[sl] + li;
   const float bnd = bnd_dist[i];
-  const int t0 = blockIdx.y * kFeatSlabs, t1 = min(n_t, t0 + kFeatSlabs);
   double c0 = 0.0, cm = 0.0, cp = 0.0;
   const double *v0 = nullptr, *vm = nullptr, *vp = nullptr;
   float ltop[8], lplain = 0.f, lobs = 0.f;   // lplain, lobs: the diagonal's without and with the observation
@@ -522,13 +521,16 @@ __global__ void __launch_bounds__(128) k_cv_features(SellPattern pat, BtModel m,
   const bool pairs = (reinterpret_cast<uintptr_t>(F) & 7) == 0;   // a caller's buffer may start on 4 bytes
 #pragma unroll
   for (int q = 0; q < 8; ++q) ltop[q] = 0.f;
-  for (int t = t0; t < t1; ++t) {
+  // the block's ranges of kFeatSlabs slabs (one, below a million slabs)
+  const int64_t first = (int64_t)blockIdx.y * kFeatSlabs, jump = (int64_t)(gridDim.y - 1) * kFeatSlabs;
+  for (int64_t tt = first; tt < n_t; tt += (tt + 1) % kFeatSlabs ? 1 : 1 + jump) {
+    const int t = (int)tt;
     // no coupling past the ends: its scale is zero, and a zero is never among the largest
     const bool has_m = t > 0, has_p = t + 1 < n_t;
     const double b0 = m.diag.scale(t), bm = has_m ? m.off.scale(t - 1) : 0.0, bp = has_p ? m.off.scale(t) : 0.0;
     const double *u0 = m.diag.at(t), *um = has_m ? m.off.at(t - 1) : u0, *up = has_p ? m.off.at(t) : u0;
     auto same = [](double x, double y) { return __double_as_longlong(x) == __double_as_longlong(y); };
-    if (t == t0 || !same(b0, c0) || !same(bm, cm) || !same(bp, cp) || u0 != v0 || um != vm || up != vp) {
+    if (tt == first || !same(b0, c0) || !same(bm, cm) || !same(bp, cp) || u0 != v0 || um != vm || up != vp) {
       c0 = b0;
       cm = bm;
       cp = bp;
@@ -600,7 +602,7 @@ __global__ void __launch_bounds__(128) k_cv_features(SellPattern pat, BtModel m,
 void launch_cv_features(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t,
                         const float *sep_dist, const float *bnd_dist, const double th[3], float *F) {
   ++g_launch_count;
-  k_cv_features<<<dim3((n_s + 127) / 128, (n_t + kFeatSlabs - 1) / kFeatSlabs), 128, 0, s>>>(
+  k_cv_features<<<dim3((n_s + 127) / 128, std::min((n_t - 1) / kFeatSlabs + 1, 65535)), 128, 0, s>>>(
       pat, m, n_s, n_t, sep_dist, bnd_dist, th[0], th[1], th[2], F);
 }
 
