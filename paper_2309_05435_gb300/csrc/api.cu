@@ -1396,7 +1396,9 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
     TRY(c->alloc(&c->lz.zero, (size_t)c->ld));
     TRY(c->alloc(&c->lz.partial, (size_t)lz_grid(c->n) * c->ld));
     TRY(c->alloc(&c->lz.U, (size_t)m * m * c->ld));
-    QSEL_CUDA_TRY(cudaMemset(c->lz.zero, 0, (size_t)c->ld * sizeof(double)));
+    // on the sampler's stream: it is a non-blocking one beside the dense part, so
+    // a plain cudaMemset (legacy default stream) would not come before the reads
+    QSEL_CUDA_TRY(cudaMemsetAsync(c->lz.zero, 0, (size_t)c->ld * sizeof(double), s));
     c->lz.ready = true;
   }
   launch_philox_normals(s, c->opt.seed, 0u, c->n, c->k, c->ld, c->d_z1);
