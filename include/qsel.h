@@ -114,9 +114,12 @@ enum {
 
 /* Arithmetic of the pipeline. */
 enum {
-  QSEL_FP64 = 0,      /* IEEE binary64 operands and results; the dense products
-                         and block applies form exact digit products on the tensor
-                         cores and round to binary64 once                        */
+  QSEL_FP64 = 0,      /* IEEE binary64 data and results.  The dense products and
+                         block applies hold their operands' rows in 62-bit fixed
+                         point, balanced by powers of two of the matrices'
+                         diagonals, multiply them digit by digit on the tensor
+                         cores with exact sums and round to binary64 once: the
+                         accuracy does not depend on the unknowns' units        */
   QSEL_MIXED = 1      /* binary32 solves and factorisations, extended-precision
                          pivot tiles (double-float or binary64, see
                          pivot_precision), binary64 refinement residuals and

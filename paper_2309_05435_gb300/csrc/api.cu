@@ -64,6 +64,9 @@ struct DenseSlot {
   uint16_t *Od[2] = {nullptr, nullptr};
   int32_t *Oe[2] = {nullptr, nullptr};
   OzSweep oz;
+  // half exponents of the diagonals of Dinv and of SigA, SigB (the products' shifts)
+  std::vector<int32_t *> Dhx;
+  int32_t *Shx[2] = {nullptr, nullptr};
   void *wbuf = nullptr;                // T_max x n_pad x ld correction samples
   void *tra = nullptr, *trb = nullptr; // ld x n_pad transposes (tensor-core correction products)
   void *ybuf = nullptr, *tmp = nullptr, *bright = nullptr;
@@ -133,6 +136,7 @@ struct qsel_ctx {
   float *f_x = nullptr, *f_r = nullptr, *f_z = nullptr, *f_p = nullptr, *f_q = nullptr;
   double *d_pa = nullptr, *d_pb = nullptr;
   void *d_pblk = nullptr;
+  int32_t *d_pshift = nullptr;         // FP64: half exponents of its blocks' diagonals
   double *d_scal = nullptr;           // alpha, beta, rho, bb, rr (ld each) + max_rel
   int32_t *d_active = nullptr, *d_counters = nullptr;
   // estimator
@@ -175,6 +179,7 @@ struct qsel_ctx {
     double *u = nullptr, *q = nullptr, *xt = nullptr, *linv = nullptr;
     double *alpha = nullptr, *beta = nullptr, *coef = nullptr, *eta = nullptr, *zero = nullptr;
     double *partial = nullptr, *U = nullptr;
+    int32_t *shift = nullptr;           // exponents of linv's diagonal
     bool ready = false, ran = false;
   } lz;
   double *d_partials = nullptr, *d_diag_scratch = nullptr;
@@ -763,6 +768,7 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
   const int nblk = (n + c->bsize - 1) / c->bsize;
   const size_t esz = c->mixed ? sizeof(float) : sizeof(double);
   TRY(c->alloc_bytes(&c->d_pblk, (size_t)nblk * c->bsize * c->bsize * esz));
+  if (!c->mixed) TRY(c->alloc(&c->d_pshift, (size_t)round_up(n, 64)));
   TRY(c->alloc(&c->d_scal, (size_t)5 * c->ld + 8));
   TRY(c->alloc(&c->d_active, (size_t)c->ld));
   TRY(c->alloc(&c->d_counters, 8));
@@ -878,7 +884,7 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
   auto slot_bytes = [&](int T) {
     const size_t base = (size_t)(T + 5 + (split_panels ? 4 : 0)) * mat + (split_panels ? 9 : 5) * panel +
                         (size_t)kSweepPanel * (kSweepPanel + 1) * 64 * 64 * esz + (size_t)(T + 5) * svec + 4096;
-    return base + (c->oz ? 2 * oz_operand + (size_t)oz_sweep_bytes(n_pad) : 0);
+    return base + (c->oz ? 2 * oz_operand + (size_t)(T + 2) * n_pad * sizeof(int32_t) + (size_t)oz_sweep_bytes(n_pad) : 0);
   };
   size_t free_b = 0, total_b = 0;
   QSEL_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
@@ -933,13 +939,18 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
     TRY(c->alloc_bytes(&sl.Wp, panel));
     TRY(c->alloc_bytes(&sl.U2, panel));
     TRY(c->alloc_bytes(&sl.Wp2, panel));
+    sl.Dhx.assign(sl.Dinv.size(), nullptr);
     if (c->oz) {
       uint8_t *oz = nullptr;
-      TRY(c->alloc(&oz, 2 * oz_operand + (size_t)oz_sweep_bytes(n_pad)));
+      const size_t hx = (size_t)n_pad * sizeof(int32_t);
+      TRY(c->alloc(&oz, 2 * oz_operand + (own + 2) * hx + (size_t)oz_sweep_bytes(n_pad)));
       for (int q = 0; q < 2; ++q, oz += oz_operand) {
         sl.Od[q] = reinterpret_cast<uint16_t *>(oz);
         sl.Oe[q] = reinterpret_cast<int32_t *>(oz + oz_digit_bytes(oz_rows, n_pad));
       }
+      for (int t = 0; t < own; ++t, oz += hx) sl.Dhx[t] = reinterpret_cast<int32_t *>(oz);
+      for (int q = 0; q < 2; ++q, oz += hx) sl.Shx[q] = reinterpret_cast<int32_t *>(oz);
+      if (c->twist && i == 1) sl.Dhx[c->half[1].T - 1] = c->slots[0].Dhx[c->half[0].T - 1];
       sl.oz = oz_sweep_at(oz, n_pad);
     }
     if (split_panels) {
@@ -1046,6 +1057,7 @@ static PcgVec<T> make_pcg(qsel_ctx *c, T *x, T *r, T *z, T *p, T *q) {
   // the block-Jacobi apply as digit products (the scalar Jacobi one, b = 1, is not
   // a product)
   v.oz = std::is_same<T, double>::value && !c->kron && c->bsize >= 16 && oz_available();
+  v.shift = c->d_pshift;
   v.err = c->d_err;
   v.n_tiles = v.oz ? oz_block_grid(c->n) : pcg_update_grid(c->n);
   v.x = x;
@@ -1152,7 +1164,7 @@ static Err solve_R(qsel_ctx *c) {
     double *pblk = static_cast<double *>(c->d_pblk);
     if (!c->kron)
       launch_jacobi_setup<double>(s, c->pat, c->mod, c->n_s, c->n_t,
-                                  c->bsize, pblk, c->d_err);
+                                  c->bsize, pblk, c->d_pshift, c->d_err);
     QSEL_CUDA_TRY(cudaMemcpyAsync(c->d_r, c->d_R, vec * sizeof(double), cudaMemcpyDeviceToDevice, s));
     PcgVec<double> v = make_pcg<double>(c, c->d_X, c->d_r, c->d_zv, c->d_p, c->d_q);
     int it = 0;
@@ -1169,7 +1181,7 @@ static Err solve_R(qsel_ctx *c) {
   float *pblk = static_cast<float *>(c->d_pblk);
   if (!c->kron)
     launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t,
-                               c->bsize, pblk, c->d_err);
+                               c->bsize, pblk, c->d_pshift, c->d_err);
   PcgVec<float> v = make_pcg<float>(c, c->f_x, c->f_r, c->f_z, c->f_p, c->f_q);
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_X, 0, vec * sizeof(double), s));
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_q, 0, vec * sizeof(double), s));
@@ -1322,7 +1334,7 @@ static Err run_sampler_graph(qsel_ctx *c) {
   if (!c->mixed) {
     double *pblk = static_cast<double *>(c->d_pblk);
     launch_jacobi_setup<double>(s, c->pat, c->mod, c->n_s, c->n_t,
-                                c->bsize, pblk, c->d_err);
+                                c->bsize, pblk, c->d_pshift, c->d_err);
     QSEL_CUDA_TRY(cudaMemcpyAsync(c->d_r, c->d_R, vec * sizeof(double), cudaMemcpyDeviceToDevice, s));
     PcgVec<double> v = make_pcg<double>(c, c->d_X, c->d_r, c->d_zv, c->d_p, c->d_q);
     TRY(pcg_graph<double>(c, s, 0, v, pblk, c->opt.pcg_tol));
@@ -1332,7 +1344,7 @@ static Err run_sampler_graph(qsel_ctx *c) {
   }
   float *pblk = static_cast<float *>(c->d_pblk);
   launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t,
-                             c->bsize, pblk, c->d_err);
+                             c->bsize, pblk, c->d_pshift, c->d_err);
   PcgVec<float> v = make_pcg<float>(c, c->f_x, c->f_r, c->f_z, c->f_p, c->f_q);
   v.tol2_dev = c->d_tol2;
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_X, 0, vec * sizeof(double), s));
@@ -1389,6 +1401,7 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
     TRY(c->alloc(&c->lz.q, vec));
     TRY(c->alloc(&c->lz.xt, vec));
     TRY(c->alloc(&c->lz.linv, (size_t)nblk * b * b));
+    TRY(c->alloc(&c->lz.shift, (size_t)nblk * b));
     TRY(c->alloc(&c->lz.alpha, (size_t)m * c->ld));
     TRY(c->alloc(&c->lz.beta, (size_t)m * c->ld));
     TRY(c->alloc(&c->lz.coef, (size_t)m * c->ld));
@@ -1403,7 +1416,7 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
   }
   launch_philox_normals(s, c->opt.seed, 0u, c->n, c->k, c->ld, c->d_z1);
   QSEL_CUDA_TRY(cudaEventRecord(c->ev[1], s));
-  launch_bj_cholinv(s, c->pat, c->mod, c->n_s, c->n_t, b, c->lz.linv,
+  launch_bj_cholinv(s, c->pat, c->mod, c->n_s, c->n_t, b, c->lz.linv, c->lz.shift,
                     c->d_err);
   LanczosArgs la{c->n, c->ld, c->k, m};
   BtSpmmArgs<double> sp{};
@@ -1430,12 +1443,12 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
       double *alpha_j = c->lz.alpha + (size_t)j * c->ld;
       double *beta_j = c->lz.beta + (size_t)j * c->ld;
       // w = L^-1 Q L^-T v  (the SpMM's time combination uses w as scratch)
-      launch_oz_block_apply(s, c->lz.linv, b, true, c->n, c->ld, v, c->lz.u, nullptr, nullptr, c->d_err);
+      launch_oz_block_apply(s, c->lz.linv, b, true, nullptr, c->n, c->ld, v, c->lz.u, nullptr, nullptr, c->d_err);
       sp.x = c->lz.u;
       sp.y = c->lz.q;
       sp.tmp = w;
       launch_bt_spmm<double>(s, sp);
-      launch_oz_block_apply(s, c->lz.linv, b, false, c->n, c->ld, c->lz.q, w, nullptr, nullptr, c->d_err);
+      launch_oz_block_apply(s, c->lz.linv, b, false, c->lz.shift, c->n, c->ld, c->lz.q, w, nullptr, nullptr, c->d_err);
       if (pass == 0) {
         launch_lz_vec(s, 0, la, vp, v, w, nullptr, nullptr, beta_prev, c->lz.partial);
         launch_lz_reduce(s, la, c->lz.partial, false, alpha_j, nullptr);
@@ -1456,7 +1469,7 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
       launch_lz_quadrature(s, la, c->lz.alpha, c->lz.beta, c->lz.eta, c->lz.U, c->lz.coef, c->d_err);
   }
   // rewind the preconditioner: x = L^-T x~
-  launch_oz_block_apply(s, c->lz.linv, b, true, c->n, c->ld, c->lz.xt, c->d_X, nullptr, nullptr, c->d_err);
+  launch_oz_block_apply(s, c->lz.linv, b, true, nullptr, c->n, c->ld, c->lz.xt, c->d_X, nullptr, nullptr, c->d_err);
   QSEL_CUDA_TRY(cudaGetLastError());
   c->stats.pcg_iterations = m;
   c->stats.pcg_max_rel_residual = 0.0;
@@ -1528,6 +1541,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
       we.Vk = buf(sl.Vk);
       for (int q = 0; q < 4; ++q) we.Sp[q] = buf(sl.Sp[q]);
       we.oz = sl.oz;
+      we.half_exp = sl.Dhx[t];
       if (t + 1 < sd.T) {
         SpEntry<T, T> &ge = gb.e[gb.count++];
         ge.B = Dinv(p, t);
@@ -1576,8 +1590,12 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
     launch_extract<T>(s, xb, c->pat, c->dmod.n, n_s, n_pad, c->d_diag_scratch);
   }
   std::vector<T *> sig_next(p1 - p0, nullptr);
+  std::vector<const int32_t *> sig_hx(p1 - p0, nullptr);   // its diagonal's half exponents
   std::vector<int> flip(p1 - p0, 0);
-  for (int p = p0; p < p1; ++p) sig_next[p - p0] = Dinv(p, part(p).T - 1);
+  for (int p = p0; p < p1; ++p) {
+    sig_next[p - p0] = Dinv(p, part(p).T - 1);
+    sig_hx[p - p0] = slot(p).Dhx[part(p).T - 1];
+  }
   const bool use_tc = std::is_same<T, float>::value ? c->tc_passes > 0 : c->oz;
   if (use_tc) {
     {
@@ -1633,6 +1651,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
             ge.beta = 1.0;
             SweepEntry<T> &me = mb.e[mb.count++];
             me.A = sig_cur;
+            me.half_exp = sl.Shx[flip[p - p0]];
             if (tl <= sd.hi) {
               ExtractEntry<T> &xe = xs.e[xs.count++];
               xe.S = sig_cur;
@@ -1655,14 +1674,17 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
         if (active.empty()) break;
         launch_sp_colgather<T>(s, wb, c->pat, n_s, n_pad);
         if constexpr (std::is_same<T, double>::value) {
-          // digit planes of W and Sigma_{t+1}, then of Y in Sigma's place
+          // digit planes of W and Sigma_{t+1}, then of Y in Sigma's place; the
+          // contracted index of both products is slab t + 1's, with Sigma's diagonal
+          // as its scale
           OzSplitJob js[2 * kMaxBatch];
           OzGemmBatch y2{}, s2{};
           int nj = 0;
           for (int q = 0; q < yb.count; ++q) {
             DenseSlot &sl = slot(active[q]);
-            js[nj++] = OzSplitJob{yb.e[q].A, sl.Od[0], sl.Oe[0], n_pad};
-            js[nj++] = OzSplitJob{yb.e[q].B, sl.Od[1], sl.Oe[1], n_pad};
+            const int32_t *hx = sig_hx[active[q] - p0];
+            js[nj++] = OzSplitJob{yb.e[q].A, sl.Od[0], sl.Oe[0], n_pad, hx, 1};
+            js[nj++] = OzSplitJob{yb.e[q].B, sl.Od[1], sl.Oe[1], n_pad, hx, -1};
             y2.e[y2.count++] = OzGemmEntry{sl.Od[0], sl.Od[1], sl.Oe[0], sl.Oe[1], nullptr, yb.e[q].C, 0};
           }
           launch_oz_split_rows(s, js, nj, n_pad, n_pad);
@@ -1674,7 +1696,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
             DenseSlot &sl = slot(active[a]);
             const GemmEntry<T> &ge = sgb.e[s2.count];
             if (ge.A != buf(sl.Y)) continue;
-            js[nj++] = OzSplitJob{buf(sl.Y), sl.Od[1], sl.Oe[1], n_pad};
+            js[nj++] = OzSplitJob{buf(sl.Y), sl.Od[1], sl.Oe[1], n_pad, sig_hx[active[a] - p0], -1};
             s2.e[s2.count++] = OzGemmEntry{sl.Od[1], sl.Od[0], sl.Oe[1], sl.Oe[0], ge.C0, ge.C, 0};
           }
           launch_oz_split_rows(s, js, nj, n_pad, n_pad);
@@ -1734,6 +1756,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
           const int tl = sd.T - 2 - b;
           if (tl >= sd.lo) {
             sig_next[p - p0] = buf(flip[p - p0] ? sl.SigB : sl.SigA);
+            sig_hx[p - p0] = sl.Shx[flip[p - p0]];
             flip[p - p0] ^= 1;
           }
         }
@@ -1873,6 +1896,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
     // tra / trb), else the tile GEMM
     void *bt[kMaxBatch], *pt[kMaxBatch];
     DenseSlot *slot_of[kMaxBatch];
+    const int32_t *hx_of[kMaxBatch];   // half exponents of D_t^-1's diagonal
     auto block_product = [&](const GemmBatch<T> &gb) -> Err {
       if constexpr (std::is_same<T, float>::value) {
         if (c->tc_passes > 0) {
@@ -1882,13 +1906,14 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
           return ok();
         }
       } else if (c->oz) {
-        // D_t^-1's digit planes by rows, the block's by columns
+        // D_t^-1's digit planes by rows, the block's by columns; D_t^-1's diagonal is
+        // the scale of the contracted index
         OzSplitJob ja[kMaxBatch], jb[kMaxBatch];
         OzGemmBatch og{};
         for (int q = 0; q < gb.count; ++q) {
           DenseSlot &sl = *slot_of[q];
-          ja[q] = OzSplitJob{gb.e[q].A, sl.Od[0], sl.Oe[0], n_pad};
-          jb[q] = OzSplitJob{gb.e[q].B, sl.Od[1], sl.Oe[1], ld};
+          ja[q] = OzSplitJob{gb.e[q].A, sl.Od[0], sl.Oe[0], n_pad, hx_of[q], -1};
+          jb[q] = OzSplitJob{gb.e[q].B, sl.Od[1], sl.Oe[1], ld, hx_of[q], 1};
           og.e[og.count++] = OzGemmEntry{sl.Od[0], sl.Od[1], sl.Oe[0], sl.Oe[1], gb.e[q].C0, gb.e[q].C,
                                          gb.e[q].alpha < 0.0 ? 1 : 0};
         }
@@ -1916,6 +1941,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
         bt[ub.count] = sl.tra;
         pt[ub.count] = sl.trb;
         slot_of[ub.count] = &sl;
+        hx_of[ub.count] = sl.Dhx[t];
         GemmEntry<T> &g = ub.e[ub.count++];
         g.A = Dinv(p, t);
         g.B = buf(sl.ybuf);
@@ -1958,6 +1984,7 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
         bt[wb.count] = sl.tra;
         pt[wb.count] = sl.trb;
         slot_of[wb.count] = &sl;
+        hx_of[wb.count] = sl.Dhx[t];
         GemmEntry<T> &g = wb.e[wb.count++];
         g.A = Dinv(p, t);
         g.B = buf(sl.tmp);
@@ -3323,7 +3350,7 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
     for (int i = 0; i < c->n; ++i)
       for (int j = 0; j < c->k; ++j) hr[(size_t)i * c->ld + j] = (float)R[(size_t)i * ld + j];
     float *pblk = static_cast<float *>(c->d_pblk);
-    if (!c->kron) launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t, c->bsize, pblk, c->d_err);
+    if (!c->kron) launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t, c->bsize, pblk, c->d_pshift, c->d_err);
     cudaError_t ce = cudaMemcpyAsync(c->f_r, hr.data(), vec * sizeof(float), cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(c->d_scal, 0, (size_t)c->ld * sizeof(double), s);   // alpha = 0
     if (ce != cudaSuccess) return finish(c, cuda_fail(ce, "preconditioner input", __FILE__, __LINE__));
@@ -3343,7 +3370,7 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
   double *pblk = static_cast<double *>(c->d_pblk);
   if (!c->kron)
     launch_jacobi_setup<double>(s, c->pat, c->mod, c->n_s, c->n_t,
-                                c->bsize, pblk, c->d_err);
+                                c->bsize, pblk, c->d_pshift, c->d_err);
   const size_t vec = (size_t)c->n * c->ld;
   cudaError_t ce = cudaMemsetAsync(c->d_r, 0, vec * sizeof(double), s);
   if (ce == cudaSuccess)

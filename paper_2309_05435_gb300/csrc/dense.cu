@@ -21,6 +21,7 @@
 #include "qsel.h"
 #include "kernels.cuh"
 #include "sweep.cuh"
+#include "oz.cuh"
 
 #include <type_traits>
 
@@ -464,6 +465,9 @@ __global__ void __launch_bounds__(256) k_sweep_mirror(SweepBatch<T> bt, int ld, 
       const int r = idx >> 6, c = idx & 63;
       Tij[(int64_t)r * ld + c] = sg * ((r >= c) ? S[r * 65 + c] : S[c * 65 + r]);
     }
+    if constexpr (std::is_same<T, double>::value)
+      if (e.half_exp && threadIdx.x < 64)
+        e.half_exp[i * 64 + threadIdx.x] = oz::half_exponent(sg * S[threadIdx.x * 66]);
   } else {
     T *Tji = e.A + (int64_t)j * 64 * ld + i * 64;
     for (int idx = threadIdx.x; idx < 4096; idx += 256) {

@@ -132,6 +132,7 @@ struct PcgVec {
   int32_t *counters;                  // [0] active columns
   double *max_rel;                    // [0] max relative residual
   bool oz = false;                    // double: block-Jacobi apply as digit products
+  const int32_t *shift = nullptr;     // its shifts (launch_jacobi_setup)
   int32_t *err = nullptr;             // error word of its bounded waits
   const double *tol2_dev = nullptr;   // squared stopping tolerance in device memory (overrides the argument)
 };
@@ -147,9 +148,11 @@ void launch_loop_status(cudaStream_t s, const int32_t *counters, int32_t *loop);
 void launch_refine_ctl(cudaStream_t s, cudaGraphConditionalHandle h, const int32_t *counters,
                        const double *max_rel, int32_t *loop, int first, int max_outer, int max_iter, double tol,
                        double inner_floor, double *tol2_dev);
+// pblk: the inverses of the diagonal blocks of bsize rows; shift (double, or
+// null): the half exponents (oz.cuh) of their diagonals, one per row of the blocks.
 template <typename T>
 void launch_jacobi_setup(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t, int bsize,
-                         T *pblk, int32_t *err_flag);
+                         T *pblk, int32_t *shift, int32_t *err_flag);
 // Grid of the PCG update (also the number of its partial rows, PcgVec::n_tiles).
 int pcg_update_grid(int n);
 struct KronOperator;
@@ -224,6 +227,9 @@ struct SweepEntry {
   T *Sp[4];      // tensor-core path: the panel update's U and V split into TF32 hi / lo
                  // (U_hi, U_lo, V_hi, V_lo; n_pad x 64 kSweepPanel each), or null
   OzSweep oz;    // double only
+  // double, or null: the half exponents (oz.cuh) of the diagonal that the mirror
+  // leaves, n_pad of them
+  int32_t *half_exp = nullptr;
 };
 // Streams and events of the tensor-core sweep's look-ahead: the pivot chain
 // (pivots, the panel's and the next panel's rows) runs on hi (high priority);
@@ -312,6 +318,9 @@ struct OzSplitJob {
   uint16_t *dig;            // digit planes (16-byte aligned)
   int32_t *exp;             // exponent of every row (or column)
   int rows;
+  // shifts along the contracted index (16-byte aligned), times sign = +-1; null: none
+  const int32_t *shift = nullptr;
+  int sign = 0;
 };
 // Digit planes of the rows of rows x cols blocks (leading dimension ld; cols and
 // ld multiples of 4), or of the columns of K x cols blocks (cols a multiple of
@@ -340,10 +349,12 @@ bool launch_oz_gemm(cudaStream_t s, const OzGemmBatch &b, int M, int N, int K, i
 // z = B x (trans: B^T x) for a block-diagonal B of b = 16, 32 or 64 rows a block
 // (block after block, row-major) and n x ld blocks x, z (ld <= 512, z not x); with
 // partial_xz, partial_xx non-null the column sums of x z and x x per CTA
-// (oz_block_grid(n) rows of ld).  Needs oz_available().
+// (oz_block_grid(n) rows of ld).  shift (16-byte aligned, a value for every row of
+// the blocks; null: none): the digits' shifts of x's rows (oz.cuh), the binary
+// logarithms of what the columns of B scale like.  Needs oz_available().
 int oz_block_grid(int n);
-void launch_oz_block_apply(cudaStream_t s, const double *B, int b, bool trans, int n, int ld, const double *x, double *z,
-                           double *partial_xz, double *partial_xx, int32_t *err);
+void launch_oz_block_apply(cudaStream_t s, const double *B, int b, bool trans, const int32_t *shift, int n, int ld,
+                           const double *x, double *z, double *partial_xz, double *partial_xx, int32_t *err);
 // One pivot k of the binary64 sweep on digit products: the column panel and its
 // digit planes (SweepEntry::oz), see oz_gemm.cu.
 void launch_oz_sweep_panel(cudaStream_t s, const SweepBatch<double> &b, int k, int n_pad, int32_t *err);
@@ -579,7 +590,7 @@ struct LanczosArgs {
 };
 int lz_grid(int n);
 void launch_bj_cholinv(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t, int b,
-                       double *linv, int32_t *err_flag);
+                       double *linv, int32_t *shift, int32_t *err_flag);
 void launch_lz_vec(cudaStream_t s, int mode, const LanczosArgs &a, const double *vprev, const double *v, double *w,
                    double *xt, const double *coef, const double *scal, double *partial);
 void launch_lz_reduce(cudaStream_t s, const LanczosArgs &a, const double *partial, bool sqrt_out, double *out,

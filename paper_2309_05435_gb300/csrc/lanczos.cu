@@ -15,15 +15,18 @@
 #include "qsel.h"
 #include "kernels.cuh"
 #include "bjblock.cuh"
+#include "oz.cuh"
 
 namespace qsel {
 
 // ---------------------------------------------------------------------------
 // Block factor: Linv_b = chol(Q_bb)^-1 (lower triangular), b <= 64, FP64.
-// A non-positive pivot sets bit 0 of *err_flag.
+// A non-positive pivot sets bit 0 of *err_flag.  shift: the exponents of Linv's
+// diagonal, the digits' shifts of Linv q (q in the units of Q's rows).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_bj_cholinv(SellPattern pat, BtModel m, int n_s, int n_t, int b,
-                                                    double *__restrict__ linv, int32_t *err_flag) {
+                                                    double *__restrict__ linv, int32_t *__restrict__ shift,
+                                                    int32_t *err_flag) {
   extern __shared__ __align__(16) double smem_chol[];
   double *S = smem_chol;              // [64][65]
   double *X = smem_chol + 64 * 65;    // [64][65]
@@ -62,6 +65,7 @@ __global__ void __launch_bounds__(256) k_bj_cholinv(SellPattern pat, BtModel m, 
   for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
     const int i = e / b, j = e - (e / b) * b;
     L[e] = X[i * 65 + j];
+    if (i == j) shift[blockIdx.x * b + i] = oz::full_exponent(X[i * 66]);
   }
 }
 
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(32) k_lz_quadrature(const LanczosArgs a, const
 // Launchers
 // ---------------------------------------------------------------------------
 void launch_bj_cholinv(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t, int b,
-                       double *linv, int32_t *err_flag) {
+                       double *linv, int32_t *shift, int32_t *err_flag) {
   constexpr int smem = 2 * 64 * 65 * (int)sizeof(double);
   static bool attr = false;
   if (!attr) {
@@ -285,7 +289,7 @@ void launch_bj_cholinv(cudaStream_t s, const SellPattern &pat, const BtModel &m,
   }
   ++g_launch_count;
   const int nblk = (n_s * n_t + b - 1) / b;
-  k_bj_cholinv<<<nblk, 256, smem, s>>>(pat, m, n_s, n_t, b, linv, err_flag);
+  k_bj_cholinv<<<nblk, 256, smem, s>>>(pat, m, n_s, n_t, b, linv, shift, err_flag);
 }
 
 void launch_lz_vec(cudaStream_t s, int mode, const LanczosArgs &a, const double *vprev, const double *v, double *w,

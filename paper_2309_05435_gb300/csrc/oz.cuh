@@ -3,9 +3,9 @@
 // multiplication by using fast routines of matrix multiplication and its
 // applications", Numer. Algorithms 59, 2012).
 //
-// A row of an operand with exponent E (|x| < 2^E for all its entries) is held
-// as 62-bit integers X = rint(x 2^(62 - E)), and X as eight signed base-256
-// digits, X = sum_i d_i 256^(7 - i) with |d_0| <= 65 and -128 <= d_i <= 127:
+// A row of an operand with exponent E (|x_k| 2^s_k < 2^E for all its entries) is
+// held as 62-bit integers X_k = rint(x_k 2^(62 + s_k - E)), and X as eight signed
+// base-256 digits, X = sum_i d_i 256^(7 - i) with |d_0| <= 65 and -128 <= d_i <= 127:
 // exact bf16 values.  The tensor cores sum d_i e_j products in FP32; over K <=
 // kChunk the sums of the products with the same i + j = s stay below 2^24 in
 // magnitude, so they are exact integers, and
@@ -14,6 +14,17 @@
 // remains is the 62-bit rounding of the operands and one rounding to binary64
 // at the end: for entries within 2^-8 of their row's largest that is below the
 // error of a binary64 FMA chain.
+//
+// The shifts s_k are what keeps the entries of a row within that range whatever
+// the units of the unknowns: the two operands of a product carry them with
+// opposite signs, so that they cancel in it.  They are read off a symmetric
+// positive definite matrix M over the contracted index (half_exponent of M_kk): a
+// row of M satisfies |M_ik| <= sqrt(M_ii M_kk), so its entries with s_k = -log2
+// sqrt(M_kk) all lie below sqrt(M_ii), and the other operand's entries, which
+// scale like 1 / sqrt(M_kk), are as even.  A rescaling x -> D x of the unknowns by
+// powers of two therefore changes no digit, and no bit of a result but its
+// exponent.  Without the shifts D Q D lost what the spread of D exceeded 2^8 by
+// (diagonal of an inverse: 6e-12 at spreads of 10^8, 3e-8 at 10^12).
 #pragma once
 
 #include <cstdint>
@@ -25,23 +36,52 @@ constexpr int kDigits = 8;
 constexpr int kChunk = 128;                   // K of an exact FP32 sum: 7 kChunk 2^14 < 2^24
 constexpr int32_t kNonFinite = 0x7fffffff;    // exponent of a row with an infinity or a NaN
 
-// Exponent field of a binary64 value (0 for zero and subnormal numbers).
-__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-// The row exponent E of a largest exponent field (see above).
-__device__ __forceinline__ int32_t row_exponent(int field) {
-  return field == 0x7ff ? kNonFinite : max(field, 1) - 1022;
+// Largest exponent field of x_u 2^(SIGN sh_u) (fields lie in 0 .. 0x7ff, shifts
+// within +- 2048), kBadField where an infinity or a NaN is among them; a row's
+// largest decides its exponent, from kNoField on.  Zeros count as 2^-1023: with
+// shifts of M's diagonal the entries that matter lie far above it.
+constexpr int kNoField = -(1 << 16), kBadField = 1 << 16;
+template <int SIGN, int N>
+__device__ __forceinline__ int max_field(const double (&x)[N], const int (&sh)[N]) {
+  int hi = 0, s = kNoField;
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    const int f = (__double2hiint(x[u]) >> 20) & 0x7ff;
+    hi = max(hi, f);
+    s = max(s, f + SIGN * sh[u]);
+  }
+  return hi == 0x7ff ? kBadField : s;
+}
+// The row exponent E of a largest scaled field (see above).
+__device__ __forceinline__ int32_t row_exponent(int field) { return field == kBadField ? kNonFinite : field - 1022; }
+// The exponent that the digits of a row are formed with: all zero in a row with an
+// infinity or a NaN.
+__device__ __forceinline__ int32_t digit_exponent(int32_t E) { return E == kNonFinite ? 1 << 16 : E; }
+
+// log2(sqrt(v)) to the nearest integer or the next one, for a positive normal v, else 0.
+__device__ __forceinline__ int half_exponent(double v) {
+  const int f = __double2hiint(v) >> 20;   // with the sign
+  return f > 0 && f < 0x7ff ? (f >> 1) - 511 : 0;
+}
+// floor(log2 |v|) for a normal v, else 0.
+__device__ __forceinline__ int full_exponent(double v) {
+  const int f = (__double2hiint(v) >> 20) & 0x7ff;
+  return f > 0 && f < 0x7ff ? f - 1023 : 0;
 }
 
 // rint(x 2^(62 - E)) for |x| < 2^E (ties away from zero), in integer arithmetic:
-// GB300 runs binary64 at 1/64 of the integer rate.
+// GB300 runs binary64 at 1/64 of the integer rate.  E is the row's digit exponent
+// less the entry's shift.
 __device__ __forceinline__ int64_t fixed62(double x, int32_t E) {
   const uint64_t bits = (uint64_t)__double_as_longlong(x);
   const int field = (int)(bits >> 52) & 0x7ff;
-  uint64_t m = bits & 0x000fffffffffffffULL;
-  if (field) m |= 0x0010000000000000ULL;
-  // m 2^10 shifted right by one more than the distance to the largest exponent
-  const int d = E + 1023 - max(field, 1), r = min(d, 63);
-  const uint64_t v = d > 63 ? 0 : ((m << 10) + (1ULL << (r - 1))) >> r;
+  // |x| = m 2^(field - 1075), also for field 0
+  const uint64_t frac = bits & 0x000fffffffffffffULL;
+  const uint64_t m = field ? frac | 0x0010000000000000ULL : frac << 1;
+  // m 2^10 shifted right by one more than the distance to the largest exponent;
+  // out of range (below zero only for x = 0 or in an empty row) gives 0
+  const uint32_t d = (uint32_t)(E + 1022 - field), r = min(d, 62u);
+  const uint64_t v = d > 62u ? 0 : ((m << 10) + (1ULL << r)) >> (r + 1);
   return (bits >> 63) ? -(int64_t)v : (int64_t)v;
 }
 

@@ -24,7 +24,9 @@
 // 1600-node block 236 -> 44 us.  The products' error against a 113-bit reference
 // is 5e-17 relative in the 2-norm (the final rounding) at K = 64 .. 1024, the FMA
 // chain's 1e-16 .. 1e-15, on random, decaying, equal-sign and widely scaled
-// operands.  It is used at every size: a 64 x 64 x 64 product takes 66 us on one
+// operands; that an entry far below its row's largest keeps its own accuracy rests on
+// the shifts (oz.cuh): the selected inverse of D Q D, D over 10^-6 .. 10^6, has the
+// bits of Q's.  The shifts cost 1 us of a sweep panel's 30.  It is used at every size: a 64 x 64 x 64 product takes 66 us on one
 // SM's binary64 pipe and 19 us here.
 #include <algorithm>
 #include <cstring>
@@ -312,47 +314,65 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_oz_split_rows(const __grid_co
   const int row = blockIdx.x;
   if (row >= job.rows) return;
   const double *src = job.src + (int64_t)row * p.ld;
-  int f = 0;
+  auto shifts = [&](int k) {
+    if (!job.shift) return make_int4(0, 0, 0, 0);
+    const int4 v = *reinterpret_cast<const int4 *>(job.shift + k);
+    return job.sign < 0 ? make_int4(-v.x, -v.y, -v.z, -v.w) : v;
+  };
+  int f = kNoField;
   for (int k = 4 * threadIdx.x; k < p.cols; k += 4 * SPLIT_THREADS) {
     const double2 a = *reinterpret_cast<const double2 *>(src + k), b = *reinterpret_cast<const double2 *>(src + k + 2);
-    f = max(f, max(max(exp_field(a.x), exp_field(a.y)), max(exp_field(b.x), exp_field(b.y))));
+    const int4 h = shifts(k);
+    const double x[4] = {a.x, a.y, b.x, b.y};
+    const int sh[4] = {h.x, h.y, h.z, h.w};
+    f = max(f, max_field<1>(x, sh));
   }
   for (int o = 16; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f;
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < SPLIT_THREADS / 32; ++w) f = max(f, red[w]);
-  const int32_t E = row_exponent(f);
+  const int32_t E = row_exponent(f), Ef = digit_exponent(E);
   if (threadIdx.x == 0) job.exp[row] = E;
-  const int32_t Ef = E == kNonFinite ? 1025 : E;
   const int64_t plane = (int64_t)job.rows * p.cols;
   uint16_t *dst = job.dig + (int64_t)row * p.cols;
   for (int k = 4 * threadIdx.x; k < p.cols; k += 4 * SPLIT_THREADS) {
     const double2 a = *reinterpret_cast<const double2 *>(src + k), b = *reinterpret_cast<const double2 *>(src + k + 2);
-    const uint2 y[4] = {digit_bytes(fixed62(a.x, Ef)), digit_bytes(fixed62(a.y, Ef)), digit_bytes(fixed62(b.x, Ef)),
-                        digit_bytes(fixed62(b.y, Ef))};
+    const int4 h = shifts(k);
+    const uint2 y[4] = {digit_bytes(fixed62(a.x, Ef - h.x)), digit_bytes(fixed62(a.y, Ef - h.y)),
+                        digit_bytes(fixed62(b.x, Ef - h.z)), digit_bytes(fixed62(b.y, Ef - h.w))};
     store_digits4(dst + k, plane, y);
   }
 }
 
 // Digit planes of the columns of a K x N block (row-major, leading dimension
 // ld): plane i, column c, entry k at dig[i * N * K + c * K + k].  Two passes: the
-// largest exponent field of every column (atomicMax into exp, which starts at
-// zero), then 64 (k) x 32 (columns) tiles transposed through shared memory.
+// largest scaled field of every column (atomicMax into exp, less kNoField, so that
+// the zero it starts from is an empty column), then 64 (k) x 32 (columns) tiles
+// transposed through shared memory.
+__device__ __forceinline__ int shift_of(const OzSplitJob &job, int k) {
+  if (!job.shift) return 0;
+  return job.sign < 0 ? -job.shift[k] : job.shift[k];
+}
+
 __global__ void __launch_bounds__(256) k_oz_colmax(const __grid_constant__ SplitParams p, int K) {
   __shared__ int red[8][32];
   const OzSplitJob &job = p.j[blockIdx.z];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
-  int f = 0;
+  int f = kNoField;
   const int k1 = min(K, (int)(blockIdx.y + 1) * 256);
-  for (int k = blockIdx.y * 256 + w; k < k1; k += 8) f = max(f, exp_field(job.src[(int64_t)k * p.ld + c]));
+  for (int k = blockIdx.y * 256 + w; k < k1; k += 8) {
+    const double x[1] = {job.src[(int64_t)k * p.ld + c]};
+    const int sh[1] = {shift_of(job, k)};
+    f = max(f, max_field<1>(x, sh));
+  }
   red[w][lane] = f;
   __syncthreads();
   if (w == 0) {
 #pragma unroll
     for (int q = 1; q < 8; ++q) f = max(f, red[q][lane]);
-    atomicMax(&job.exp[c], f);
+    atomicMax(&job.exp[c], f - kNoField);
   }
 }
 
@@ -366,18 +386,18 @@ __global__ void __launch_bounds__(256) k_oz_split_cols(const __grid_constant__ S
   const int64_t plane = (int64_t)p.cols * K;
   for (int e = threadIdx.x; e < 16 * 32; e += 256) {
     const int k = 4 * (e & 15), c = e >> 4;
-    const int32_t E = row_exponent(job.exp[c0 + c]);
-    const int32_t Ef = E == kNonFinite ? 1025 : E;
-    const uint2 y[4] = {digit_bytes(fixed62(S[k][c], Ef)), digit_bytes(fixed62(S[k + 1][c], Ef)),
-                        digit_bytes(fixed62(S[k + 2][c], Ef)), digit_bytes(fixed62(S[k + 3][c], Ef))};
+    const int32_t Ef = digit_exponent(row_exponent(job.exp[c0 + c] + kNoField));
+    uint2 y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) y[u] = digit_bytes(fixed62(S[k + u][c], Ef - shift_of(job, k0 + k + u)));
     store_digits4(job.dig + (int64_t)(c0 + c) * K + k0 + k, plane, y);
   }
 }
-// exponent fields to row exponents, once every column has been split
+// scaled fields to row exponents, once every column has been split
 __global__ void k_oz_exponents(const __grid_constant__ SplitParams p) {
   const OzSplitJob &job = p.j[blockIdx.y];
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < p.cols) job.exp[c] = row_exponent(job.exp[c]);
+  if (c < p.cols) job.exp[c] = row_exponent(job.exp[c] + kNoField);
 }
 
 // ---------------------------------------------------------------------------
@@ -387,7 +407,8 @@ __global__ void k_oz_exponents(const __grid_constant__ SplitParams p) {
 // The product takes 64 x 64 x 64 binary64 FMAs per row tile, 63 us on one SM's
 // binary64 pipe; as digit products it is 48 MMAs.  The digits of A_ik are formed
 // in registers and stored to shared memory in the MMA's swizzled layout and to
-// global memory as V's at once.  70 us a pivot on the CUDA cores, 40 with a row per
+// global memory as V's at once.  The pivot index k carries the half exponents of
+// P_kk as shifts: + for A_ik (and V), - for P and U.  70 us a pivot on the CUDA cores, 40 with a row per
 // thread, 25 with eight threads a row (whole sectors) at 1024 and 1600 nodes.
 // ---------------------------------------------------------------------------
 struct PanelParams {
@@ -407,15 +428,16 @@ constexpr int PANEL_THREADS = 512;
 constexpr int PARTS = PANEL_THREADS / BM;      // threads per row of the left operand
 constexpr int PART = 64 / PARTS;               // entries of a thread
 
-// Eight digits of eight neighbouring values: 16 bytes per digit plane to shared
-// (stride s_plane; with s_twin a second time, s_twin bytes further) and / or global
-// memory (stride g_plane).
-template <bool SMEM>
+// Eight digits of eight neighbouring values with shifts SIGN sh: 16 bytes per digit
+// plane to shared (stride s_plane; with s_twin a second time, s_twin bytes further)
+// and / or global memory (stride g_plane).  E: the row exponent.
+template <bool SMEM, int SIGN>
 __device__ __forceinline__ void store_digits8(uint8_t *sdst, uint32_t s_plane, uint16_t *gdst, int64_t g_plane,
-                                              const double *x, int32_t E, uint32_t s_twin = 0) {
+                                              const double *x, int32_t E, const int (&sh)[8], uint32_t s_twin = 0) {
+  const int32_t Ef = digit_exponent(E);
   uint2 y[8];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) y[c] = digit_bytes(fixed62(x[c], E));
+  for (int c = 0; c < 8; ++c) y[c] = digit_bytes(fixed62(x[c], Ef - SIGN * sh[c]));
 #define QSEL_OZ_STORE(I)                                                                                  \
   {                                                                                                       \
     const uint4 w = make_uint4(digit_pair<I>(y[0], y[1]), digit_pair<I>(y[2], y[3]),                      \
@@ -434,30 +456,22 @@ __device__ __forceinline__ void store_digits8(uint8_t *sdst, uint32_t s_plane, u
   QSEL_OZ_STORE(7)
 #undef QSEL_OZ_STORE
 }
-__device__ __forceinline__ int32_t finite_exponent(int32_t E) { return E == kNonFinite ? 1025 : E; }
-
-// Digits of the 64 x 64 matrix B(row, j) as the right operand at sb, its row
-// exponents to ep: eight threads per row, eight entries each.
-template <class F>
-__device__ __forceinline__ void matrix_digits(uint8_t *sb, int32_t *ep, F B) {
+// Digits of a 64 x 64 matrix B as the right operand at sb, its row exponents to ep:
+// eight threads per row; y: B(threadIdx.x >> 3, 8 (threadIdx.x & 7) ..), shifts -sh.
+__device__ __forceinline__ void matrix_digits(uint8_t *sb, int32_t *ep, const double (&y)[8], const int (&sh)[8]) {
   const int row = threadIdx.x >> 3, part = threadIdx.x & 7;
-  double y[8];
-  int g = 0;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) y[u] = B(row, 8 * part + u);
-#pragma unroll
-  for (int u = 0; u < 8; ++u) g = max(g, exp_field(y[u]));
+  int g = max_field<-1>(y, sh);
   for (int o = 1; o < 8; o <<= 1) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
   const int32_t E = row_exponent(g);
   if (part == 0) ep[row] = E;
-  store_digits8<true>(sb + row * P_ROWB + ((part ^ (row & 7)) << 4), PB_TILE, nullptr, 0, y, finite_exponent(E));
+  store_digits8<true, -1>(sb + row * P_ROWB + ((part ^ (row & 7)) << 4), PB_TILE, nullptr, 0, y, E, sh);
 }
-// The row exponent from the parts' largest exponent fields.
-__device__ __forceinline__ int32_t part_exponent(const int (&red)[PARTS][BM], int r) {
+// The largest of the parts' scaled fields.
+__device__ __forceinline__ int part_field(const int (&red)[PARTS][BM], int r) {
   int f = red[0][r];
 #pragma unroll
   for (int h = 1; h < PARTS; ++h) f = max(f, red[h][r]);
-  return row_exponent(f);
+  return f;
 }
 
 __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __grid_constant__ PanelParams p) {
@@ -492,7 +506,15 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
   auto entries = [&](int gi) {
     return (gi >> 6) > k ? A + (int64_t)gi * ld + 64 * k + 8 * sub : A + (int64_t)(64 * k + 8 * sub) * ld + gi;
   };
-  matrix_digits(sb, ep, [&](int row, int j) { return P[row * 64 + j]; });
+  int sh[8];
+  {
+    double y[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) y[u] = P[(threadIdx.x >> 3) * 64 + 8 * sub + u];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) sh[u] = half_exponent(P[(8 * sub + u) * 65]);
+    matrix_digits(sb, ep, y, sh);
+  }
 #pragma unroll 1
   for (int r = threadIdx.x >> 3; r < BM; r += PANEL_THREADS / 8) {
     const int gi = blockIdx.x * BM + r;
@@ -500,19 +522,17 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
     const double *src = entries(gi);
     const int64_t step = (gi >> 6) > k ? 1 : ld;
     double x[8];
-    int f = 0;
 #pragma unroll
     for (int u = 0; u < 8; ++u) x[u] = live ? src[u * step] : 0.0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) f = max(f, exp_field(x[u]));
+    int f = max_field<1>(x, sh);
     for (int o = 1; o < 8; o <<= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
     const int32_t E = row_exponent(f);
     if (sub == 0) {
       ea[r] = E;
       if (valid) p.Ev[z][gi] = E;
     }
-    store_digits8<true>(sa + r * P_ROWB + ((sub ^ (r & 7)) << 4), PA_TILE,
-                        valid ? p.V[z] + (int64_t)gi * 64 + 8 * sub : nullptr, plane, x, finite_exponent(E));
+    store_digits8<true, 1>(sa + r * P_ROWB + ((sub ^ (r & 7)) << 4), PA_TILE,
+                           valid ? p.V[z] + (int64_t)gi * 64 + 8 * sub : nullptr, plane, x, E, sh);
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   tc_fence_before();
@@ -554,16 +574,14 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
       const int gi = blockIdx.x * BM + r;
       const bool valid = gi < p.n_pad, on_pivot = (gi >> 6) == k;
       double x[8];
-      int f = 0;
 #pragma unroll
       for (int u = 0; u < 8; ++u) x[u] = su[r * kUld + 8 * sub + u];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) f = max(f, exp_field(x[u]));
+      int f = max_field<-1>(x, sh);
       for (int o = 1; o < 8; o <<= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
       const int32_t E = row_exponent(f);
       if (!valid) continue;
       if (sub == 0) p.Eu[z][gi] = E;
-      store_digits8<false>(nullptr, 0, p.U[z] + (int64_t)gi * 64 + 8 * sub, plane, x, finite_exponent(E));
+      store_digits8<false, -1>(nullptr, 0, p.U[z] + (int64_t)gi * 64 + 8 * sub, plane, x, E, sh);
       if (on_pivot) {
         double *dst = A + (int64_t)gi * ld + 64 * k + 8 * sub;
         const double *src = P + (gi & 63) * 64 + 8 * sub;
@@ -596,13 +614,14 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
 // runs 48 MMAs and rounds, about 130 integer operations per entry.  512 threads:
 // with 256 the operations' latencies showed (43.6 against 62 us for two tiles of
 // 128 columns an SM).  Measured, n = 32768, 128 columns: 545 us on the binary64
-// pipe (k_pcg_precond) -> 82 us; n = 9216, 64 columns, without sums: 52 -> 17 us.
+// pipe (k_pcg_precond) -> 88 us, 3 of them for the shifts; n = 9216, 64 columns, without sums: 52 -> 17 us.
 // A chunk of at most 64 columns fills both halves of the M rows with them: two threads
 // share a column, each forms the digits of half the rows (for both halves) and rounds
 // half the results: with sums and n = 2048, 20.8 -> about 14 us.
 // ---------------------------------------------------------------------------
 struct BlockParams {
   const double *B, *x;
+  const int32_t *shift;
   double *z, *pa, *pb;
   int n, ld, b, log2b, trans;
   int32_t *err;
@@ -637,11 +656,11 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __gri
   const int q = warp & 3, part = warp >> 2, cl = 32 * q + lane;
   if (DOTS)
     for (int c = threadIdx.x; c < 2 * p.ld; c += PANEL_THREADS) acc[c] = 0.0;
+  const int n_tiles = (p.n + 63) / 64, n_blocks = (p.n + p.b - 1) / p.b;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  const int n_tiles = (p.n + 63) / 64, n_blocks = (p.n + p.b - 1) / p.b;
   uint32_t issued = 0;
   bool go = true;
   for (int tile = blockIdx.x; tile < n_tiles && go; tile += gridDim.x) {
@@ -649,11 +668,34 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __gri
     // the digits of B's rows (zero outside the blocks); the previous tile's MMAs
     // have completed
     const int blk0 = r0 >> p.log2b;
-    matrix_digits(sb, ep, [&](int row, int j) {
-      const int blk = row >> p.log2b, br = row & (p.b - 1), bj = j & (p.b - 1);
-      if (j >> p.log2b != blk || blk0 + blk >= n_blocks) return 0.0;
-      return p.B[((int64_t)(blk0 + blk) * p.b + (p.trans ? bj : br)) * p.b + (p.trans ? br : bj)];
-    });
+    // of rows j .. + 7 of the tile (j a multiple of 8): + for x, - for B
+    auto shifts = [&](int j, int (&sh)[8]) {
+      int4 v[2] = {make_int4(0, 0, 0, 0), make_int4(0, 0, 0, 0)};
+      if (p.shift && r0 + j < n_blocks * p.b) {
+        v[0] = *reinterpret_cast<const int4 *>(p.shift + r0 + j);
+        v[1] = *reinterpret_cast<const int4 *>(p.shift + r0 + j + 4);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        sh[4 * u] = v[u].x;
+        sh[4 * u + 1] = v[u].y;
+        sh[4 * u + 2] = v[u].z;
+        sh[4 * u + 3] = v[u].w;
+      }
+    };
+    {
+      const int row = threadIdx.x >> 3, blk = row >> p.log2b, br = row & (p.b - 1);
+      double y[8];
+      int sh[8];
+      shifts(8 * (threadIdx.x & 7), sh);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int j = 8 * (threadIdx.x & 7) + u, bj = j & (p.b - 1);
+        const bool live = j >> p.log2b == blk && blk0 + blk < n_blocks;
+        y[u] = live ? p.B[((int64_t)(blk0 + blk) * p.b + (p.trans ? bj : br)) * p.b + (p.trans ? br : bj)] : 0.0;
+      }
+      matrix_digits(sb, ep, y, sh);
+    }
     const int rows = min(PART, max(0, p.n - r0 - PART * part));   // this thread's rows
     for (int c0 = 0; c0 < p.ld && go; c0 += BM) {
       const bool twin = p.ld - c0 <= BM / 2;
@@ -663,14 +705,21 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __gri
       const int64_t at = (int64_t)(r0 + PART * part) * p.ld + col;
       const double *xc = p.x + at;
       double *zc = p.z + at;
-      int f = 0;
+      int f = kNoField;
       if (valid) {
-#pragma unroll 8
-        for (int j = 8 * e_begin; j < min(rows, 8 * e_end); ++j) f = max(f, exp_field(xc[(int64_t)j * p.ld]));
+#pragma unroll 1
+        for (int c = e_begin; c < e_end; ++c) {
+          double x[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) x[u] = 8 * c + u < rows ? xc[(int64_t)(8 * c + u) * p.ld] : 0.0;
+          int sh[8];
+          shifts(PART * part + 8 * c, sh);
+          f = max(f, max_field<1>(x, sh));
+        }
       }
       red[part][cl] = f;
       __syncthreads();
-      const int32_t Ea = max(part_exponent(red, cl), twin ? part_exponent(red, cl ^ (BM / 2)) : INT32_MIN);
+      const int32_t Ea = row_exponent(max(part_field(red, cl), twin ? part_field(red, cl ^ (BM / 2)) : kNoField));
       // eight values at a time in loops, x re-read (from L1): unrolled over the
       // tile, the kernel waited on instruction fetches for most of its time
 #pragma unroll 1
@@ -678,9 +727,11 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_block_apply(const __gri
         double x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) x[u] = valid && 8 * c + u < rows ? xc[(int64_t)(8 * c + u) * p.ld] : 0.0;
+        int sh[8];
+        shifts(PART * part + 8 * c, sh);
         const int row = twin ? cl & (BM / 2 - 1) : cl;
-        store_digits8<true>(sa + row * P_ROWB + (((PART / 8 * part + c) ^ (row & 7)) << 4), PA_TILE, nullptr, 0, x,
-                            finite_exponent(Ea), twin ? BM / 2 * P_ROWB : 0);
+        store_digits8<true, 1>(sa + row * P_ROWB + (((PART / 8 * part + c) ^ (row & 7)) << 4), PA_TILE, nullptr, 0, x,
+                               Ea, sh, twin ? BM / 2 * P_ROWB : 0);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       tc_fence_before();
@@ -890,9 +941,9 @@ void launch_oz_sweep_panel(cudaStream_t s, const SweepBatch<double> &b, int k, i
 
 int oz_block_grid(int n) { return std::min((n + 63) / 64, device_sms()); }
 
-void launch_oz_block_apply(cudaStream_t s, const double *B, int b, bool trans, int n, int ld, const double *x, double *z,
-                           double *partial_xz, double *partial_xx, int32_t *err) {
-  oz::BlockParams p{B, x, z, partial_xz, partial_xx, n, ld, b, b == 64 ? 6 : b == 32 ? 5 : 4, trans ? 1 : 0, err,
+void launch_oz_block_apply(cudaStream_t s, const double *B, int b, bool trans, const int32_t *shift, int n, int ld,
+                           const double *x, double *z, double *partial_xz, double *partial_xx, int32_t *err) {
+  oz::BlockParams p{B, x, shift, z, partial_xz, partial_xx, n, ld, b, b == 64 ? 6 : b == 32 ? 5 : 4, trans ? 1 : 0, err,
                     tc::wait_limit()};
   ++g_launch_count;
   if (partial_xz)

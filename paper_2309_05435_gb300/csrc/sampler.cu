@@ -9,6 +9,7 @@
 #include "kernels.cuh"
 #include "sweep.cuh"
 #include "bjblock.cuh"
+#include "oz.cuh"
 
 #include <algorithm>
 #include <type_traits>
@@ -378,7 +379,8 @@ template void launch_bt_spmm<float>(cudaStream_t, const BtSpmmArgs<float> &);
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) k_jacobi_setup(SellPattern pat, BtModel m, int n_s, int n_t, int b,
-                                                      T *__restrict__ pblk, int32_t *err_flag) {
+                                                      T *__restrict__ pblk, int32_t *__restrict__ shift,
+                                                      int32_t *err_flag) {
   __shared__ double S[64 * 65];
   assemble_diag_block(S, 65, pat, m, n_s, n_t, blockIdx.x * b, b);
   sym_sweep_inverse_smem(S, 65, b, err_flag);
@@ -386,21 +388,22 @@ __global__ void __launch_bounds__(256) k_jacobi_setup(SellPattern pat, BtModel m
   for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
     const int i = e / b, j = e - (e / b) * b;
     P[e] = (T)(-S[i * 65 + j]);
+    if (shift && i == j) shift[blockIdx.x * b + i] = oz::half_exponent(-S[i * 66]);
   }
 }
 
 template <typename T>
 void launch_jacobi_setup(cudaStream_t s, const SellPattern &pat, const BtModel &m, int n_s, int n_t, int bsize,
-                         T *pblk, int32_t *err_flag) {
+                         T *pblk, int32_t *shift, int32_t *err_flag) {
   ++g_launch_count;
   const int n = n_s * n_t;
   const int nblk = (n + bsize - 1) / bsize;
-  k_jacobi_setup<T><<<nblk, bsize >= 16 ? 256 : 32, 0, s>>>(pat, m, n_s, n_t, bsize, pblk, err_flag);
+  k_jacobi_setup<T><<<nblk, bsize >= 16 ? 256 : 32, 0, s>>>(pat, m, n_s, n_t, bsize, pblk, shift, err_flag);
 }
 template void launch_jacobi_setup<double>(cudaStream_t, const SellPattern &, const BtModel &, int, int, int, double *,
-                                          int32_t *);
+                                          int32_t *, int32_t *);
 template void launch_jacobi_setup<float>(cudaStream_t, const SellPattern &, const BtModel &, int, int, int, float *,
-                                         int32_t *);
+                                         int32_t *, int32_t *);
 
 // ---------------------------------------------------------------------------
 // PCG update for a 64-row tile: x += alpha p, r -= alpha q, z = P r (block
@@ -602,7 +605,7 @@ void launch_pcg_update(cudaStream_t s, const PcgVec<T> &v, const T *pblk, int bs
         k_pcg_axpy<T><<<(int)std::min<int64_t>((vec2 + 255) / 256, 152 * 8), 256, 0, s>>>(v);
       }
       ProfScope ps_(s, PROF_PRECOND, 2.0 * bsize * (double)v.n * v.ld);
-      launch_oz_block_apply(s, pblk, bsize, false, v.n, v.ld, v.r, v.z, v.partial_a, v.partial_b, v.err);
+      launch_oz_block_apply(s, pblk, bsize, false, v.shift, v.n, v.ld, v.r, v.z, v.partial_a, v.partial_b, v.err);
       return;
     }
   }
