@@ -10,9 +10,9 @@
 // quarters of the work, are split over the cluster's four SMs: U and B22' by rows,
 // X and N11 - U^T X by columns, so that each CTA needs the others' results only at
 // the three cluster barriers (through distributed shared memory).
-// Measured: 106 -> 43 us a tile (two 32 x 32 sweeps 26k cycles each, the products
-// 9k + 9k); the sweeps' chain -- column product, diagonal, reciprocal, barrier --
-// is what remains.
+// Measured: 106 -> 49 us a tile (two 32 x 32 sweeps 31k cycles each, the products
+// 9k + 9k); the sweeps' chain -- column product, diagonal, correctly rounded
+// reciprocal, barrier -- is what remains.
 #include <cooperative_groups.h>
 
 #include "qsel.h"
@@ -29,19 +29,9 @@ struct Smem {
 
 __device__ __forceinline__ void sweep_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-// 1 / d from the hardware's 20-bit estimate y and e = 1 - d y: y (1 + e + e^2) leaves
-// e^3 = 2^-60, about one unit in the last place, in three dependent binary64
-// operations (86 cycles each; the division's correctly rounded sequence takes
-// 490).  The range checks are on the exponent field, off the binary64 pipe.
+// 1 / d, rounded to nearest; 0 and bad for a pivot that is not positive.
 __device__ __forceinline__ double pivot_reciprocal(double d, bool &bad) {
-  const uint32_t f = (uint32_t)__double2hiint(d) >> 20;   // sign and exponent
-  if (f - 23u < 2000u) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    const double e = fma(-d, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-  }
-  if (d > 0.0) return 1.0 / d;
+  if (d > 0.0) return __drcp_rn(d);
   bad = true;
   return 0.0;
 }
