@@ -1567,7 +1567,8 @@ static Err run_wave(qsel_ctx *c, int p0, int p1, std::vector<std::pair<cudaEvent
       ae.accumulate = 1;
       launch_schur_assemble<T>(s, ab, c->pat, c->mod.obs_w, n_s, n_pad);
     }
-    spd_inverse<T>(s, wb, n_pad, c->d_err, c->tc_passes, c->mixed ? &c->sweep_ss : nullptr);
+    if (!spd_inverse<T>(s, wb, n_pad, c->d_err, c->tc_passes, c->mixed ? &c->sweep_ss : nullptr))
+      return fail(QSEL_ECUDA, "a tensor-core product of the factorisation could not be launched");
     launch_sp_rowgather<T, T>(s, gb, c->pat, n_s, n_pad, n_pad, n_pad, n_pad);
   }
   QSEL_CUDA_TRY(cudaGetLastError());
@@ -2776,7 +2777,10 @@ qsel_status qsel_loglik_grad(qsel_ctx *ctx, double grad_out[3], double terms_out
   kb.e[0].U = c->d_Ku;
   kb.e[0].V = c->d_Kv;
   if (c->d_Koz) kb.e[0].oz = oz_sweep_at(c->d_Koz, n_pad);
-  spd_inverse<double>(s, kb, n_pad, c->d_err, 0);
+  if (!spd_inverse<double>(s, kb, n_pad, c->d_err, 0)) {
+    cudaStreamSynchronize(s);   // leave no work of this call in flight
+    return finish(c, fail(QSEL_ECUDA, "a tensor-core product of the hyperparameter gradient could not be launched"));
+  }
   launch_loglik_combine(s, c->d_K, n_pad, c->d_cdiag, c->n_s, c->n_t, c->d_theta, c->d_traces,
                         c->n_beta > 0 ? c->fe_trace() : nullptr, c->d_hyp, c->d_hyp + 3, c->d_hyp + 6);
   int32_t err = 0;

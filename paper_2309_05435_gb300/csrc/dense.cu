@@ -489,9 +489,10 @@ int device_sms() {
   return sms;
 }
 template <typename T>
-void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err_flag, int tc_passes,
+bool spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err_flag, int tc_passes,
                  const SweepStreams *ss) {
-  if (b.count <= 0) return;
+  if (b.count <= 0) return true;
+  bool launched = true;   // every tensor-core product
   if (sweep_serial()) ss = nullptr;
   const int nt = n_pad / 64;
   const int n_lower = nt * (nt + 1) / 2;
@@ -529,7 +530,7 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
         }
         Profiler *saved = g_prof;
         g_prof = nullptr;  // timed under cls, not as a GEMM
-        launch_tc_gemm(st, gb, M, N, K, ldw, ldw, ldc, lower, tc_passes, err_flag, compact);
+        launched &= launch_tc_gemm(st, gb, M, N, K, ldw, ldw, ldc, lower, tc_passes, err_flag, compact);
         g_prof = saved;
         if (prof) g_prof->end(st, rec);
       };
@@ -718,7 +719,7 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
               ub.count = b.count;
               for (int e = 0; e < b.count; ++e)
                 ub.e[e] = UpdateEntry{b.e[e].Sp[0], b.e[e].Sp[1], b.e[e].Sp[2], b.e[e].Sp[3], b.e[e].A};
-              launch_tc_update(lo, ub, n_pad, 64 * bw, ldw, -1.0f, 1.0f, err_flag, upd_ctas);
+              launched &= launch_tc_update(lo, ub, n_pad, 64 * bw, ldw, -1.0f, 1.0f, err_flag, upd_ctas);
             }
             if (saved) saved->end(lo, rec);
           } else {
@@ -748,7 +749,7 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
         ProfScope ps_(s, PROF_PANEL);
         k_sweep_mirror<T><<<dim3(n_lower, b.count), 256, 0, s>>>(b, n_pad, -1.0);
       }
-      return;
+      return launched;
     }
   }
   for (int k = 0; k < nt; ++k) {
@@ -768,7 +769,7 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
         gb.count = b.count;
         for (int e = 0; e < b.count; ++e)
           gb.e[e] = OzGemmEntry{b.e[e].oz.Ud, b.e[e].oz.Vd, b.e[e].oz.Eu, b.e[e].oz.Ev, b.e[e].A, b.e[e].A, 1};
-        if (nt > 1) launch_oz_gemm(s, gb, n_pad, n_pad, 64, n_pad, true, k, err_flag);
+        if (nt > 1) launched &= launch_oz_gemm(s, gb, n_pad, n_pad, 64, n_pad, true, k, err_flag);
         continue;
       }
     }
@@ -792,10 +793,11 @@ void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
     ProfScope ps_(s, PROF_PANEL);
     k_sweep_mirror<T><<<dim3(n_lower, b.count), 256, 0, s>>>(b, n_pad, -1.0);
   }
+  return launched;
 }
-template void spd_inverse<double>(cudaStream_t, const SweepBatch<double> &, int, int32_t *, int,
+template bool spd_inverse<double>(cudaStream_t, const SweepBatch<double> &, int, int32_t *, int,
                                   const SweepStreams *);
-template void spd_inverse<float>(cudaStream_t, const SweepBatch<float> &, int, int32_t *, int, const SweepStreams *);
+template bool spd_inverse<float>(cudaStream_t, const SweepBatch<float> &, int, int32_t *, int, const SweepStreams *);
 
 template <typename T>
 void launch_mirror(cudaStream_t s, const SweepBatch<T> &b, int n_pad) {

@@ -254,8 +254,10 @@ struct SweepBatch {
 // panel on the tcgen05 tensor cores (Up, Wp and Vk are needed).  With ss the
 // next panel is pivoted on ss->hi while the update of the current one runs on
 // ss->lo (both joined back into s); without it everything runs on s.
+// False when a tensor-core product of it could not be launched (the matrices are
+// then not inverses; the streams are joined all the same).
 template <typename T>
-void spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err_flag, int tc_passes = 0,
+[[nodiscard]] bool spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err_flag, int tc_passes = 0,
                  const SweepStreams *ss = nullptr);
 // The pivots of panel [k0, k0 + bw) of the tensor-core sweep on the panel's own
 // rows of Wp[buf], in one launch of a cluster per matrix (sweep_chain.cu).
@@ -325,8 +327,8 @@ struct OzSplitJob {
 // Digit planes of the rows of rows x cols blocks (leading dimension ld; cols and
 // ld multiples of 4), or of the columns of K x cols blocks (cols a multiple of
 // 32, K of 64): the K-major operands of launch_oz_gemm.  Up to 2 kMaxBatch jobs.
-bool launch_oz_split_rows(cudaStream_t s, const OzSplitJob *jobs, int count, int cols, int ld);
-bool launch_oz_split_cols(cudaStream_t s, const OzSplitJob *jobs, int count, int K, int cols, int ld);
+void launch_oz_split_rows(cudaStream_t s, const OzSplitJob *jobs, int count, int cols, int ld);
+[[nodiscard]] bool launch_oz_split_cols(cudaStream_t s, const OzSplitJob *jobs, int count, int K, int cols, int ld);
 struct OzGemmEntry {
   const uint16_t *A, *B;    // digit planes: A of M rows, B of N rows, K entries each
   const int32_t *Ea, *Eb;
@@ -343,7 +345,7 @@ struct OzGemmBatch {
 // rows and columns of that 64-wide tile index are left as they are.  err gets bit 1 when a
 // bounded wait gives up.  False when nothing could be launched.
 bool oz_available();
-bool launch_oz_gemm(cudaStream_t s, const OzGemmBatch &b, int M, int N, int K, int ldc, bool lower, int skip,
+[[nodiscard]] bool launch_oz_gemm(cudaStream_t s, const OzGemmBatch &b, int M, int N, int K, int ldc, bool lower, int skip,
                     int32_t *err);
 
 // z = B x (trans: B^T x) for a block-diagonal B of b = 16, 32 or 64 rows a block
@@ -366,7 +368,7 @@ void launch_oz_sweep_panel(cudaStream_t s, const SweepBatch<double> &b, int k, i
 // two stages (81 KB of shared memory), so that a CTA fits on an SM beside one
 // of the persistent sweep update's.
 bool tc_gemm_available();
-bool launch_tc_gemm(cudaStream_t s, const GemmBatch<float> &b, int M, int N, int K, int lda, int ldb, int ldc,
+[[nodiscard]] bool launch_tc_gemm(cudaStream_t s, const GemmBatch<float> &b, int M, int N, int K, int lda, int ldb, int ldc,
                     bool lower, int passes, int32_t *err, bool compact = false);
 // Persistent tcgen05 update of the lower 128 x 128 tiles of n x n matrices:
 // C = alpha U V^T + beta C with U, V (n x K, leading dimension ldp) given as
@@ -380,7 +382,7 @@ struct UpdateBatch {
   UpdateEntry e[kMaxBatch];
   int count;
 };
-bool launch_tc_update(cudaStream_t s, const UpdateBatch &b, int n, int K, int ldp, float alpha, float beta,
+[[nodiscard]] bool launch_tc_update(cudaStream_t s, const UpdateBatch &b, int n, int K, int ldp, float alpha, float beta,
                       int32_t *err, int max_ctas = 0);
 // C = alpha A B^T + beta C0 on operands given as TF32 hi / lo parts (A: M x K,
 // B: N x K, row-major; K a multiple of 32, leading dimensions multiples of 4):
@@ -398,7 +400,7 @@ struct SplitGemmBatch {
   SplitGemmEntry e[kMaxBatch];
   int count;
 };
-bool launch_tc_gemm_split(cudaStream_t s, const SplitGemmBatch &b, int M, int N, int K, int lda, int ldb, int ldc,
+[[nodiscard]] bool launch_tc_gemm_split(cudaStream_t s, const SplitGemmBatch &b, int M, int N, int K, int lda, int ldb, int ldc,
                           bool lower, int32_t *err, int max_ctas = 0);
 // hi = rn_tf32(x), lo = rn_tf32(x - hi) elementwise (16-byte aligned arrays).
 void launch_split_tf32(cudaStream_t s, const float *src, float *hi, float *lo, int64_t count);
@@ -430,7 +432,7 @@ void launch_transpose_axpby(cudaStream_t s, const TransBatch &b, int rows, int c
 // K-major product Pt = Bt A^T (= (A B)^T, A row-major serves as the N x K
 // operand), C = alpha Pt^T + beta C0; bt[q], pt[q] are ld x n_pad scratch.
 // False when a tensor map cannot be encoded.
-bool launch_symm_block_tc(cudaStream_t s, const GemmBatch<float> &b, float *const *bt, float *const *pt, int n_pad,
+[[nodiscard]] bool launch_symm_block_tc(cudaStream_t s, const GemmBatch<float> &b, float *const *bt, float *const *pt, int n_pad,
                           int ld, int passes, int32_t *err);
 
 template <typename T>
@@ -552,7 +554,7 @@ struct KronOperator {
 // scratch; false when the shape is not supported or a tensor map cannot be
 // encoded (nothing is launched then).
 bool kron_tc_supported(int dim, int ld);
-bool launch_kron_apply_tc(cudaStream_t s, const KronOperator &op, const float *r, float *q, float *z);
+[[nodiscard]] bool launch_kron_apply_tc(cudaStream_t s, const KronOperator &op, const float *r, float *q, float *z);
 template <typename T>
 void launch_kron_tables(cudaStream_t s, const KronOperator &op);
 template <typename T>

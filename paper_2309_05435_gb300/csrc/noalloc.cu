@@ -113,10 +113,11 @@ extern "C" qsel_status qsel_spd_inverse_noalloc(double *a_dev, int32_t n, int32_
   if (e == cudaSuccess) {
     ++g_launch_count;
     k_noalloc_pad_in<<<dim3((n_pad + 255) / 256, n_pad), 256, 0, s>>>(a_dev, n, lda, n_pad, A);
-    spd_inverse(s, b, n_pad, flag);
+    const bool launched = spd_inverse(s, b, n_pad, flag);
     ++g_launch_count;
     k_noalloc_copy_out<<<dim3((n + 255) / 256, n), 256, 0, s>>>(A, n_pad, n, a_dev, lda);
     e = cudaGetLastError();
+    if (e == cudaSuccess && !launched) e = cudaErrorLaunchFailure;
   }
   int32_t hflag = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s);

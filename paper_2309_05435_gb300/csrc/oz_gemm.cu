@@ -826,8 +826,8 @@ OzSweep oz_sweep_at(void *base, int n_pad) {
 
 int64_t oz_digit_bytes(int rows, int cols) { return (int64_t)oz::kDigits * rows * cols * 2; }
 
-bool launch_oz_split_rows(cudaStream_t s, const OzSplitJob *jobs, int count, int cols, int ld) {
-  if (count <= 0) return true;
+void launch_oz_split_rows(cudaStream_t s, const OzSplitJob *jobs, int count, int cols, int ld) {
+  if (count <= 0) return;
   oz::SplitParams p;
   memset(&p, 0, sizeof(p));
   int rows = 0;
@@ -839,7 +839,6 @@ bool launch_oz_split_rows(cudaStream_t s, const OzSplitJob *jobs, int count, int
   p.ld = ld;
   ++g_launch_count;
   oz::k_oz_split_rows<<<dim3(rows, count), oz::SPLIT_THREADS, 0, s>>>(p);
-  return true;
 }
 
 bool launch_oz_split_cols(cudaStream_t s, const OzSplitJob *jobs, int count, int K, int cols, int ld) {
