@@ -185,7 +185,8 @@ struct qsel_ctx {
   double *d_partials = nullptr, *d_diag_scratch = nullptr;
   TraceSlab *d_slabs = nullptr;
   int n_trace_slabs = 0;
-  int32_t *d_err = nullptr;
+  int32_t *d_err = nullptr;            // error words: [0] the dense part's, [1] the sampler's (it runs beside it)
+  int32_t *sampler_err() const { return d_err + 1; }
   // host staging
   int32_t *h_counters = nullptr;
   double *h_small = nullptr;
@@ -519,7 +520,7 @@ static Err kron_prepare(qsel_ctx *c) {
               kron_tc_supported(n_t, c->ld))
                  ? 1
                  : 0;
-  k.err = c->d_err;
+  k.err = c->sampler_err();
   if (c->mixed)
     launch_kron_tables<float>(c->stream, k);
   else
@@ -1058,7 +1059,7 @@ static PcgVec<T> make_pcg(qsel_ctx *c, T *x, T *r, T *z, T *p, T *q) {
   // a product)
   v.oz = std::is_same<T, double>::value && !c->kron && c->bsize >= 16 && oz_available();
   v.shift = c->d_pshift;
-  v.err = c->d_err;
+  v.err = c->sampler_err();
   v.n_tiles = v.oz ? oz_block_grid(c->n) : pcg_update_grid(c->n);
   v.x = x;
   v.r = r;
@@ -1124,7 +1125,7 @@ static Err pcg_solve(qsel_ctx *c, const PcgVec<T> &v, const T *pblk, double tol,
     if (c->h_counters[0] == 0) done = true;
   }
   QSEL_CUDA_TRY(cudaMemcpyAsync(c->h_small, v.max_rel, sizeof(double), cudaMemcpyDeviceToHost, s));
-  if (v.oz) QSEL_CUDA_TRY(cudaMemcpyAsync(c->h_counters, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  if (v.oz) QSEL_CUDA_TRY(cudaMemcpyAsync(c->h_counters, v.err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   QSEL_CUDA_TRY(cudaStreamSynchronize(s));
   if (v.oz && (c->h_counters[0] & 2))
     return fail(QSEL_ETIMEOUT, "a bounded device-side wait of the preconditioner gave up");
@@ -1164,7 +1165,7 @@ static Err solve_R(qsel_ctx *c) {
     double *pblk = static_cast<double *>(c->d_pblk);
     if (!c->kron)
       launch_jacobi_setup<double>(s, c->pat, c->mod, c->n_s, c->n_t,
-                                  c->bsize, pblk, c->d_pshift, c->d_err);
+                                  c->bsize, pblk, c->d_pshift, c->sampler_err());
     QSEL_CUDA_TRY(cudaMemcpyAsync(c->d_r, c->d_R, vec * sizeof(double), cudaMemcpyDeviceToDevice, s));
     PcgVec<double> v = make_pcg<double>(c, c->d_X, c->d_r, c->d_zv, c->d_p, c->d_q);
     int it = 0;
@@ -1181,7 +1182,7 @@ static Err solve_R(qsel_ctx *c) {
   float *pblk = static_cast<float *>(c->d_pblk);
   if (!c->kron)
     launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t,
-                               c->bsize, pblk, c->d_pshift, c->d_err);
+                               c->bsize, pblk, c->d_pshift, c->sampler_err());
   PcgVec<float> v = make_pcg<float>(c, c->f_x, c->f_r, c->f_z, c->f_p, c->f_q);
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_X, 0, vec * sizeof(double), s));
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_q, 0, vec * sizeof(double), s));
@@ -1334,7 +1335,7 @@ static Err run_sampler_graph(qsel_ctx *c) {
   if (!c->mixed) {
     double *pblk = static_cast<double *>(c->d_pblk);
     launch_jacobi_setup<double>(s, c->pat, c->mod, c->n_s, c->n_t,
-                                c->bsize, pblk, c->d_pshift, c->d_err);
+                                c->bsize, pblk, c->d_pshift, c->sampler_err());
     QSEL_CUDA_TRY(cudaMemcpyAsync(c->d_r, c->d_R, vec * sizeof(double), cudaMemcpyDeviceToDevice, s));
     PcgVec<double> v = make_pcg<double>(c, c->d_X, c->d_r, c->d_zv, c->d_p, c->d_q);
     TRY(pcg_graph<double>(c, s, 0, v, pblk, c->opt.pcg_tol));
@@ -1344,7 +1345,7 @@ static Err run_sampler_graph(qsel_ctx *c) {
   }
   float *pblk = static_cast<float *>(c->d_pblk);
   launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t,
-                             c->bsize, pblk, c->d_pshift, c->d_err);
+                             c->bsize, pblk, c->d_pshift, c->sampler_err());
   PcgVec<float> v = make_pcg<float>(c, c->f_x, c->f_r, c->f_z, c->f_p, c->f_q);
   v.tol2_dev = c->d_tol2;
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_X, 0, vec * sizeof(double), s));
@@ -1417,7 +1418,7 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
   launch_philox_normals(s, c->opt.seed, 0u, c->n, c->k, c->ld, c->d_z1);
   QSEL_CUDA_TRY(cudaEventRecord(c->ev[1], s));
   launch_bj_cholinv(s, c->pat, c->mod, c->n_s, c->n_t, b, c->lz.linv, c->lz.shift,
-                    c->d_err);
+                    c->sampler_err());
   LanczosArgs la{c->n, c->ld, c->k, m};
   BtSpmmArgs<double> sp{};
   sp.pat = c->pat;
@@ -1443,12 +1444,12 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
       double *alpha_j = c->lz.alpha + (size_t)j * c->ld;
       double *beta_j = c->lz.beta + (size_t)j * c->ld;
       // w = L^-1 Q L^-T v  (the SpMM's time combination uses w as scratch)
-      launch_oz_block_apply(s, c->lz.linv, b, true, nullptr, c->n, c->ld, v, c->lz.u, nullptr, nullptr, c->d_err);
+      launch_oz_block_apply(s, c->lz.linv, b, true, nullptr, c->n, c->ld, v, c->lz.u, nullptr, nullptr, c->sampler_err());
       sp.x = c->lz.u;
       sp.y = c->lz.q;
       sp.tmp = w;
       launch_bt_spmm<double>(s, sp);
-      launch_oz_block_apply(s, c->lz.linv, b, false, c->lz.shift, c->n, c->ld, c->lz.q, w, nullptr, nullptr, c->d_err);
+      launch_oz_block_apply(s, c->lz.linv, b, false, c->lz.shift, c->n, c->ld, c->lz.q, w, nullptr, nullptr, c->sampler_err());
       if (pass == 0) {
         launch_lz_vec(s, 0, la, vp, v, w, nullptr, nullptr, beta_prev, c->lz.partial);
         launch_lz_reduce(s, la, c->lz.partial, false, alpha_j, nullptr);
@@ -1466,10 +1467,10 @@ static Err run_sampler_lanczos(qsel_ctx *c) {
       w = t;
     }
     if (pass == 0)
-      launch_lz_quadrature(s, la, c->lz.alpha, c->lz.beta, c->lz.eta, c->lz.U, c->lz.coef, c->d_err);
+      launch_lz_quadrature(s, la, c->lz.alpha, c->lz.beta, c->lz.eta, c->lz.U, c->lz.coef, c->sampler_err());
   }
   // rewind the preconditioner: x = L^-T x~
-  launch_oz_block_apply(s, c->lz.linv, b, true, nullptr, c->n, c->ld, c->lz.xt, c->d_X, nullptr, nullptr, c->d_err);
+  launch_oz_block_apply(s, c->lz.linv, b, true, nullptr, c->n, c->ld, c->lz.xt, c->d_X, nullptr, nullptr, c->sampler_err());
   QSEL_CUDA_TRY(cudaGetLastError());
   c->stats.pcg_iterations = m;
   c->stats.pcg_max_rel_residual = 0.0;
@@ -2060,7 +2061,7 @@ static Err run_pipeline_body(qsel_ctx *c) {
   cudaStream_t s = c->stream;
   const int64_t launches0 = g_launch_count;
   c->phase_used = 0;
-  QSEL_CUDA_TRY(cudaMemsetAsync(c->d_err, 0, sizeof(int32_t), s));
+  QSEL_CUDA_TRY(cudaMemsetAsync(c->d_err, 0, 2 * sizeof(int32_t), s));
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_corr, 0, (size_t)c->n * sizeof(double), s));
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_corr4, 0, (size_t)c->n * sizeof(double), s));
   QSEL_CUDA_TRY(cudaEventRecord(c->ev[0], s));
@@ -2123,8 +2124,9 @@ static Err run_pipeline_body(qsel_ctx *c) {
   QSEL_CUDA_TRY(cudaEventRecord(c->ev[3], s));
   QSEL_CUDA_TRY(cudaStreamSynchronize(s));
   QSEL_CUDA_TRY(cudaGetLastError());
-  int32_t err = 0;
-  QSEL_CUDA_TRY(cudaMemcpy(&err, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost));
+  int32_t words[2] = {0, 0};
+  QSEL_CUDA_TRY(cudaMemcpy(words, c->d_err, sizeof(words), cudaMemcpyDeviceToHost));
+  const int32_t err = words[0] | words[1];
   // a timed-out GEMM leaves its output unwritten, so later pivots are
   // meaningless: the timeout is reported first
   if (err & 2) return fail(QSEL_ETIMEOUT, "a bounded device-side wait of the tensor-core GEMM gave up");
@@ -2155,7 +2157,7 @@ static Err run_pipeline_body(qsel_ctx *c) {
 // conditional while nodes).
 static Err enqueue_pipeline_graph(qsel_ctx *c) {
   cudaStream_t s = c->stream;
-  QSEL_CUDA_TRY(cudaMemsetAsync(c->d_err, 0, sizeof(int32_t), s));
+  QSEL_CUDA_TRY(cudaMemsetAsync(c->d_err, 0, 2 * sizeof(int32_t), s));
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_corr, 0, (size_t)c->n * sizeof(double), s));
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_corr4, 0, (size_t)c->n * sizeof(double), s));
   TRY(run_model(c));
@@ -2182,9 +2184,10 @@ static Err enqueue_pipeline_graph(qsel_ctx *c) {
 
 // After a replay of the graph: error flags, sampler status and statistics.
 static Err collect_graph(qsel_ctx *c) {
-  int32_t err = 0, loop[4] = {0, 0, 0, 0};
+  int32_t words[2] = {0, 0}, loop[4] = {0, 0, 0, 0};
   double rel = 0.0;
-  QSEL_CUDA_TRY(cudaMemcpy(&err, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost));
+  QSEL_CUDA_TRY(cudaMemcpy(words, c->d_err, sizeof(words), cudaMemcpyDeviceToHost));
+  const int32_t err = words[0] | words[1];
   QSEL_CUDA_TRY(cudaMemcpy(loop, c->d_loop, sizeof(loop), cudaMemcpyDeviceToHost));
   if (c->parts.size() > 1)
     QSEL_CUDA_TRY(cudaMemcpy(&rel, c->d_scal + 5 * c->ld, sizeof(double), cudaMemcpyDeviceToHost));
@@ -2655,6 +2658,8 @@ static Err compute_mean(qsel_ctx *c) {
   cudaStream_t s = c->stream;
   if (!c->d_mu) TRY(c->alloc(&c->d_mu, (size_t)c->n));
   TRY(run_model(c));
+  // the solve reads its error word: nothing of an earlier call may be left in it
+  QSEL_CUDA_TRY(cudaMemsetAsync(c->sampler_err(), 0, sizeof(int32_t), s));
   QSEL_CUDA_TRY(cudaMemsetAsync(c->d_R, 0, (size_t)c->n * c->ld * sizeof(double), s));
   const double inv_s2 = 1.0 / (c->sigma * c->sigma);
   launch_data_rhs(s, c->d_R, c->ld, c->d_obs, c->d_obs_index, c->d_y, c->n, inv_s2);
@@ -3345,7 +3350,7 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
   Err e = run_model(c);
   if (e.code == 0 && c->kron) e = kron_prepare(c);
   if (e.code) return finish(c, e);
-  cudaError_t ce0 = cudaMemsetAsync(c->d_err, 0, sizeof(int32_t), s);
+  cudaError_t ce0 = cudaMemsetAsync(c->sampler_err(), 0, sizeof(int32_t), s);
   if (ce0 != cudaSuccess) return finish(c, cuda_fail(ce0, "error flag", __FILE__, __LINE__));
   if (c->mixed) {
     // the mixed form's binary32 preconditioner: R rounded to float, Z widened
@@ -3354,7 +3359,7 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
     for (int i = 0; i < c->n; ++i)
       for (int j = 0; j < c->k; ++j) hr[(size_t)i * c->ld + j] = (float)R[(size_t)i * ld + j];
     float *pblk = static_cast<float *>(c->d_pblk);
-    if (!c->kron) launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t, c->bsize, pblk, c->d_pshift, c->d_err);
+    if (!c->kron) launch_jacobi_setup<float>(s, c->pat, c->mod, c->n_s, c->n_t, c->bsize, pblk, c->d_pshift, c->sampler_err());
     cudaError_t ce = cudaMemcpyAsync(c->f_r, hr.data(), vec * sizeof(float), cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(c->d_scal, 0, (size_t)c->ld * sizeof(double), s);   // alpha = 0
     if (ce != cudaSuccess) return finish(c, cuda_fail(ce, "preconditioner input", __FILE__, __LINE__));
@@ -3364,7 +3369,7 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (ce != cudaSuccess) return finish(c, cuda_fail(ce, "preconditioner output", __FILE__, __LINE__));
     int32_t err = 0;
-    ce = cudaMemcpy(&err, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost);
+    ce = cudaMemcpy(&err, c->sampler_err(), sizeof(int32_t), cudaMemcpyDeviceToHost);
     if (ce != cudaSuccess) return finish(c, cuda_fail(ce, "error flag", __FILE__, __LINE__));
     if (err & 2) return finish(c, fail(QSEL_ETIMEOUT, "a bounded device-side wait of the tensor-core pass gave up"));
     for (int i = 0; i < c->n; ++i)
@@ -3374,7 +3379,7 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
   double *pblk = static_cast<double *>(c->d_pblk);
   if (!c->kron)
     launch_jacobi_setup<double>(s, c->pat, c->mod, c->n_s, c->n_t,
-                                c->bsize, pblk, c->d_pshift, c->d_err);
+                                c->bsize, pblk, c->d_pshift, c->sampler_err());
   const size_t vec = (size_t)c->n * c->ld;
   cudaError_t ce = cudaMemsetAsync(c->d_r, 0, vec * sizeof(double), s);
   if (ce == cudaSuccess)
@@ -3386,7 +3391,7 @@ qsel_status qsel_debug_apply_precond(qsel_ctx *ctx, const double *R, double *Z, 
   launch_pcg_update<double>(s, v, pblk, c->bsize, c->kron ? &c->kop : nullptr);
   ce = cudaMemcpy2DAsync(Z, (size_t)ld * sizeof(double), c->d_zv, (size_t)c->ld * sizeof(double),
                          (size_t)c->k * sizeof(double), c->n, cudaMemcpyDeviceToHost, s);
-  if (ce == cudaSuccess) ce = cudaMemcpyAsync(c->h_counters, c->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(c->h_counters, c->sampler_err(), sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
   if (ce != cudaSuccess) return finish(c, cuda_fail(ce, "preconditioner output", __FILE__, __LINE__));
   if (c->h_counters[0] & 2)
