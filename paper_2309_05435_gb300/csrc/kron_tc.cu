@@ -199,8 +199,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_kron_tc(const __grid_constant__ 
           ++g;
         }
       }
-      if (*abort) {
-        // let the loads already issued land before the CTA's shared memory goes away
+      {
+        // let the loads already issued land before the CTA's shared memory goes away:
+        // a consumer may give up after this thread has issued its last one
         for (long long q = (g > S ? g - S : 0); q < g; ++q)
           drain(full_bar((int)(q % S)), (uint32_t)((q / S) & 1));
       }

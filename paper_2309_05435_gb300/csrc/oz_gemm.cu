@@ -172,8 +172,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
           tma_load_3d(smem_u32(st + A_BYTES), &p.tm[z][1], kb * KS, bn * BN_OZ, 0, full_bar(s));
         }
       }
-      if (*abort) {
-        // let the loads already issued land before the CTA's shared memory goes away
+      {
+        // let the loads already issued land before the CTA's shared memory goes away:
+        // a consumer may give up after this thread has issued its last one
         for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
           drain(full_bar((int)(q % STAGES)), (uint32_t)((q / STAGES) & 1));
       }

@@ -125,8 +125,9 @@ __global__ void __launch_bounds__(192) k_tc_gemm(const __grid_constant__ Params 
         tma_load_2d(smem_u32(st + TILE_A), tmb, kb * BK, bn * BN, full_bar(s));
         issued = kb + 1;
       }
-      if (*abort) {
-        // let the loads already issued land before the CTA's shared memory goes away
+      {
+        // let the loads already issued land before the CTA's shared memory goes away:
+        // a consumer may give up after this thread has issued its last one
         for (int kb = max(0, issued - STAGES); kb < issued; ++kb) {
           const long long t0 = clock64();
           uint32_t done = 0;

@@ -181,8 +181,9 @@ __global__ void __launch_bounds__(192, 1) k_tc_gemm256(const __grid_constant__ P
           ++g;
         }
       }
-      if (*abort) {
-        // let the loads already issued land before the CTA's shared memory goes away
+      {
+        // let the loads already issued land before the CTA's shared memory goes away:
+        // a consumer may give up after this thread has issued its last one
         for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
           drain(full_bar((int)(q % STAGES)), (uint32_t)((q / STAGES) & 1));
       }

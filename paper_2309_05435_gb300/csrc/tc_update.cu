@@ -133,8 +133,9 @@ __global__ void __launch_bounds__(192, 1) k_tc_update(const __grid_constant__ Pa
           ++g;
         }
       }
-      if (*abort) {
-        // let the loads already issued land before the CTA's shared memory goes away
+      {
+        // let the loads already issued land before the CTA's shared memory goes away:
+        // a consumer may give up after this thread has issued its last one
         for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q) {
           const long long t0 = clock64();
           uint32_t done = 0;
