@@ -542,6 +542,7 @@ struct RestInputs {
   std::vector<std::vector<int>> adj;       // spatial neighbours (boundary distance feature)
 };
 static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *part, int32_t overlap);
+static size_t later_bytes(const qsel_ctx *c);
 static Err build_pattern(qsel_ctx *c, const PatRows &rows, int n_arrays, std::vector<std::vector<double>> &sell);
 
 static Err build(qsel_ctx *c, const qsel_model *m, const qsel_partition *part, int32_t overlap) {
@@ -903,13 +904,17 @@ static Err build_rest(qsel_ctx *c, const RestInputs &in, const qsel_partition *p
     c->T_max = sd.T;
   }
   // Digit products for the binary64 form where the tensor cores can be used and
-  // their scratch (about four matrices a slot) neither makes a wave smaller nor
-  // takes a slot of the two-ended form; the sums are exact up to K = 16384.
+  // their scratch (about four matrices a slot) neither makes a wave smaller, nor
+  // takes a slot of the two-ended form, nor leaves too little for what later calls
+  // allocate (with 2 MiB of rounding an allocation); the sums are exact up to K = 16384.
   if (!c->mixed && n_pad <= 16384 && oz_available()) {
     const size_t want = c->twist ? 2 : (size_t)std::min({kMaxBatch, c->slot_cap, np});
     const size_t plain = std::min(want, budget / slot_bytes(c->T_max));
     c->oz = true;
-    if (plain == 0 || budget / slot_bytes(c->T_max) < plain) c->oz = false;
+    const size_t rounding = (plain * (size_t)(c->T_max + 20) + 32) << 21;
+    if (plain == 0 || budget / slot_bytes(c->T_max) < plain ||
+        plain * slot_bytes(c->T_max) + later_bytes(c) + rounding > free_b)
+      c->oz = false;
   }
   const size_t per_slot = slot_bytes(c->T_max);
   const size_t fit = budget / per_slot;
@@ -1385,6 +1390,20 @@ static Err run_sampler_graph(qsel_ctx *c) {
         QSEL_CUDA_TRY(cudaGetLastError());
         return ok();
       });
+}
+
+// Device memory that calls on the context allocate after its creation: the
+// Lanczos sampler's buffers, the data, the fixed effects, the gradient's K and the
+// planner's features.
+static size_t later_bytes(const qsel_ctx *c) {
+  size_t doubles = 0;
+  if (c->opt.sampler == QSEL_SAMPLER_LANCZOS && c->parts.size() > 1) {
+    const size_t m = c->opt.lanczos_steps, b = c->bsize, nblk = ((size_t)c->n + b - 1) / b;
+    doubles += 6 * (size_t)c->n * c->ld + nblk * b * (b + 1) + (3 * m + 2 + lz_grid(c->n) + m * m) * c->ld;
+  }
+  if (c->model_kind == QSEL_MODEL_SEPARABLE)
+    doubles += 2 * (size_t)c->n + 66 * (size_t)c->n_obs + (size_t)c->n_pad * (c->n_pad + 512) + 4 * 64 * 64;
+  return doubles * sizeof(double) + (size_t)c->n * (QSEL_CV_FEATURES + 1) * sizeof(float);
 }
 
 // Preconditioned Krylov sampler (Algorithm 5.1), FP64: two passes of m
