@@ -200,9 +200,10 @@ __global__ void __launch_bounds__(32) k_lz_quadrature(const LanczosArgs a, const
   for (int r = lane; r < mc; r += 32)
     for (int j = 0; j < mc; ++j) Z[(int64_t)r * m + j] = (r == j) ? 1.0 : 0.0;
   __syncwarp();
-  // every lane runs the same scalar recurrence on d and e (and writes the
-  // same values), so no lane reads another lane's write there; the rows of Z
-  // are split across the lanes
+  // every lane runs the same scalar recurrence on d and e and writes the same
+  // values; a step reads what it overwrites before the warp's barrier and writes
+  // after it, so that no lane takes another's new value for the old one.  The rows of
+  // Z are split across the lanes
   bool failed = false;
   for (int l = 0; l < mc && !failed; ++l) {
     int iter = 0;
@@ -224,24 +225,28 @@ __global__ void __launch_bounds__(32) k_lz_quadrature(const LanczosArgs a, const
       double s = 1.0, cs = 1.0, p = 0.0;
       bool early = false;
       for (int i = mm - 1; i >= l; --i) {
-        const double f = s * e[i], bb = cs * e[i];
-        // one reciprocal square root for both quotients, within a few ulp like
-        // hypot and two divisions, which were most of the step's instructions
+        const double ei = e[i], di = d[i], di1 = d[i + 1];
+        __syncwarp();
+        const double f = s * ei, bb = cs * ei;
+        // r, s and cs by one reciprocal square root: each within 4 2^-53 of its value (r2's
+        // error of 2 2^-53 halved, rsqrt's one unit in the last place, the product's
+        // rounding); hypot's two units and a division each, which were most of the
+        // step's instructions, bound r by 4 and s, cs by 5
         const double r2 = fma(f, f, g * g);
         const bool plain = r2 > 1e-290 && r2 < 1e290;
         const double ri = plain ? rsqrt(r2) : 0.0;
         r = plain ? r2 * ri : hypot(f, g);
         e[i + 1] = r;
         if (r == 0.0) {
-          d[i + 1] -= p;
+          d[i + 1] = di1 - p;
           e[mm] = 0.0;
           early = true;
           break;
         }
         s = plain ? f * ri : f / r;
         cs = plain ? g * ri : g / r;
-        g = d[i + 1] - p;
-        r = (d[i] - g) * s + 2.0 * cs * bb;
+        g = di1 - p;
+        r = (di - g) * s + 2.0 * cs * bb;
         p = s * r;
         d[i + 1] = g + p;
         g = cs * r - bb;
@@ -254,7 +259,9 @@ __global__ void __launch_bounds__(32) k_lz_quadrature(const LanczosArgs a, const
         }
       }
       if (early) continue;
-      d[l] -= p;
+      const double dl = d[l];
+      __syncwarp();
+      d[l] = dl - p;
       e[l] = g;
       e[mm] = 0.0;
     }
