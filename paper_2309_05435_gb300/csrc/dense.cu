@@ -229,9 +229,9 @@ template void launch_gemm<float>(cudaStream_t, const GemmBatch<float> &, int, in
 // After every step the swept matrix holds -A^-1 (Goodnight's sweep operator);
 // the final mirror negates it and fills the upper triangle.
 // ---------------------------------------------------------------------------
-// P = Tk^-1 for the 64 x 64 tile at Tk (row stride ld), from its lower half:
-// in binary64 for double tiles; for float tiles in double-float (about 48
-// bits, on the FP32 pipe) or, with fp64, in binary64.  NT threads.
+// P = Tk^-1 for the 64 x 64 float tile at Tk (row stride ld), from its lower half:
+// in double-float (about 48 bits, on the FP32 pipe) or, with fp64, in binary64.
+// NT threads.  (Double tiles: sweep_f64.cu.)
 template <int NT>
 __device__ __forceinline__ void invert_pivot_tile(const float *Tk, int ld, float *P, int32_t *err_flag, bool fp64) {
   // one buffer for either arithmetic (dfloat and double are both 8 bytes)
@@ -504,10 +504,11 @@ bool spd_inverse(cudaStream_t s, const SweepBatch<T> &b, int n_pad, int32_t *err
       // U_i = W_iK (-W_KK) = A_iK A_KK^-1 (the block form of the same sweep), and
       // the rest of the matrix the rank-64 bw update A -= U W^T.  On hi (the
       // critical path): the pivots, then the next panel's rows K' (their U),
-      // its gather, its look-ahead product on rows K' and its rows K; the next
-      // panel's pivots follow at once.  On lo: U on every other row, the
-      // look-ahead on those rows, the update and the scatter.  Buffers (W, U,
-      // V, P, Vk) alternate with the panel's parity; the events order the two
+      // their gather and the look-ahead product on them; the next panel's pivots
+      // follow at once.  On lo: the next panel's other rows (their gather, and rows
+      // K from U), U on every other row, the look-ahead on those rows, the update
+      // and the scatter.  W and U alternate with the panel's parity; P and Vk, one
+      // of each per pivot of a panel, live on hi only.  The events order the two
       // streams' shared rows.
       constexpr int ldw = 64 * kSweepPanel;
       cudaStream_t hi = s, lo = s;

@@ -312,7 +312,7 @@ template <typename T>
 void launch_diag64_rows(cudaStream_t s, const DiagRowBatch<T> &b, int n_s, int n_pad);
 
 // ---------------------------------------------------------------- oz_gemm.cu
-// Binary64 products as exact bf16 digit products on the tensor cores (oz.cuh).
+// Binary64 products as bf16 digit products on the tensor cores (oz.cuh).
 // Bytes of the eight digit planes of a rows x cols operand.
 int64_t oz_digit_bytes(int rows, int cols);
 struct OzSplitJob {

@@ -70,10 +70,6 @@ __global__ void __launch_bounds__(256) k_bj_cholinv(SellPattern pat, BtModel m, 
 }
 
 // ---------------------------------------------------------------------------
-// y = B x per 64-row tile with B = blockdiag(Linv) (TRANS = false) or its
-// transpose (TRANS = true); b in {16, 32, 64}.  The block is staged so that
-// Bs[j][row] = B[row][j]; each thread accumulates an 8-row x 2-column tile.
-// ---------------------------------------------------------------------------
 // Lanczos vector kernels.  Rows are split across CTAs; within a CTA, 64
 // consecutive columns x 4 row groups; per-CTA partial column sums in double
 // are reduced in a fixed order by k_lz_reduce.  Columns >= k are held at 0.

@@ -1,4 +1,4 @@
-// Binary64 products on the bf16 tensor cores by exact digit products (the
+// Binary64 products on the bf16 tensor cores by digit products (the
 // splitting of Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix
 // multiplication by using fast routines of matrix multiplication and its
 // applications", Numer. Algorithms 59, 2012).

@@ -1,4 +1,4 @@
-// Binary64 matrix products as exact bf16 digit products on the tensor cores
+// Binary64 matrix products as bf16 digit products on the tensor cores, exactly summed
 // (oz.cuh): C = alpha A B^T + beta C0 with A: M x K, B: N x K given as digit
 // planes, alpha = +-1, beta = 0 or 1.
 //
@@ -21,12 +21,12 @@
 // Measured: two 1600 x 1600 x 1600 products 13.3 ms on the CUDA cores (k_gemm64)
 // -> 0.53 ms (31 TFLOP/s of binary64 products; 38 at 4096, where a K = 128 block
 // takes 9.2k cycles of MMAs and 8k of reading the sums); one 64-wide update of a
-// 1600-node block 236 -> 44 us.  The products' error against a 113-bit reference
+// 1600-node block 236 -> 35 us (of two in a launch: 49).  The products' error against a 113-bit reference
 // is 5e-17 relative in the 2-norm (the final rounding) at K = 64 .. 1024, the FMA
 // chain's 1e-16 .. 1e-15, on random, decaying, equal-sign and widely scaled
 // operands; that an entry far below its row's largest keeps its own accuracy rests on
 // the shifts (oz.cuh): the selected inverse of D Q D, D over 10^-6 .. 10^6, has the
-// bits of Q's.  The shifts cost 1 us of a sweep panel's 30.  It is used at every size: a 64 x 64 x 64 product takes 66 us on one
+// bits of Q's.  The shifts cost 1 us of a sweep panel's 27.  It is used at every size: a 64 x 64 x 64 product takes 66 us on one
 // SM's binary64 pipe and 19 us here.
 #include <algorithm>
 #include <cstring>
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
       const double *c0 = p.C0[z] ? p.C0[z] + (int64_t)row * p.ldc + col : nullptr;
       double *c = p.C[z] + (int64_t)row * p.ldc + col;
       // rows straight from the registers: staging them for whole-sector stores made
-      // no difference (39.6 against 37.4 us an update)
+      // no difference (39.6 against 37.4 us an update, between events)
 #pragma unroll
       for (int cc = 0; cc < EP_COLS; cc += 2) {
         double2 o = make_double2(value(hi[cc], lo[cc], Ea, Eb[cc], neg), value(hi[cc + 1], lo[cc + 1], Ea, Eb[cc + 1], neg));
@@ -410,7 +410,8 @@ __global__ void k_oz_exponents(const __grid_constant__ SplitParams p) {
 // in registers and stored to shared memory in the MMA's swizzled layout and to
 // global memory as V's at once.  The pivot index k carries the half exponents of
 // P_kk as shifts: + for A_ik (and V), - for P and U.  70 us a pivot on the CUDA cores, 40 with a row per
-// thread, 25 with eight threads a row (whole sectors) at 1024 and 1600 nodes.
+// thread, 25 with eight threads a row (whole sectors) at 1024 and 1600 nodes, 27 with
+// the shifts.
 // ---------------------------------------------------------------------------
 struct PanelParams {
   double *A[kMaxBatch];
@@ -615,7 +616,7 @@ __global__ void __launch_bounds__(PANEL_THREADS, 1) k_oz_sweep_panel(const __gri
 // runs 48 MMAs and rounds, about 130 integer operations per entry.  512 threads:
 // with 256 the operations' latencies showed (43.6 against 62 us for two tiles of
 // 128 columns an SM).  Measured, n = 32768, 128 columns: 545 us on the binary64
-// pipe (k_pcg_precond) -> 88 us, 3 of them for the shifts; n = 9216, 64 columns, without sums: 52 -> 17 us.
+// pipe (k_pcg_precond) -> 85 us, 3 of them for the shifts; n = 9216, 64 columns, without sums: 52 -> 17 us.
 // A chunk of at most 64 columns fills both halves of the M rows with them: two threads
 // share a column, each forms the digits of half the rows (for both halves) and rounds
 // half the results: with sums and n = 2048, 20.8 -> about 14 us.

@@ -10,7 +10,7 @@
 // quarters of the work, are split over the cluster's four SMs: U and B22' by rows,
 // X and N11 - U^T X by columns, so that each CTA needs the others' results only at
 // the three cluster barriers (through distributed shared memory).
-// Measured: 106 -> 49 us a tile (two 32 x 32 sweeps 31k cycles each, the products
+// Measured: 106 -> 46 us a tile (two 32 x 32 sweeps 31k cycles each, the products
 // 9k + 9k); the sweeps' chain -- column product, diagonal, correctly rounded
 // reciprocal, barrier -- is what remains.
 #include <cooperative_groups.h>

@@ -11,9 +11,10 @@
 // One CTA per SM walks a static list of (matrix, tile row, tile column)
 // lower tiles:
 //   warp 0      one thread issues the TMA loads of the four 128 x 32 operand
-//               tiles of every K-block into a 2-stage ring (129 KB of shared
-//               memory: the sweep's pivot and panel kernels, and its compact
-//               look-ahead GEMM, fit on the same SM and run beside it);
+//               tiles of every K-block into a 3-stage ring (193 KB of shared
+//               memory; the pivot chain then runs on SMs that a smaller grid leaves
+//               free), or a 2-stage one (129 KB: the chain and the compact look-ahead
+//               GEMM fit beside it);
 //   warp 1      owns 256 TMEM columns = two 128-column accumulators; one
 //               thread issues tcgen05.mma.kind::tf32 (M = N = 128, K = 8) for
 //               tile i into accumulator i % 2 while the epilogue drains the
@@ -35,9 +36,9 @@ using namespace tc;
 constexpr int BN = 128;
 constexpr int TILE = BM * BK * 4;            // 16 KiB: 128 rows x 32 floats
 constexpr int STAGE_BYTES = 4 * TILE;        // U_hi, U_lo, V_hi, V_lo
-// Two stages (129 KB) leave room on the SM for the sweep's pivot and panel
-// CTAs beside the update; three (193 KB) do not, so those run on the SMs
-// that a capped update grid leaves free.
+// Two stages (129 KB) leave room on the SM for the sweep's pivot chain beside the
+// update; three (193 KB, the default) do not, so it runs on the SMs that a capped
+// update grid leaves free.
 template <int STAGES>
 constexpr int smem_bytes() { return STAGES * STAGE_BYTES + 256 + 1024; }
 constexpr uint32_t kTmemCols = 2 * BN;
